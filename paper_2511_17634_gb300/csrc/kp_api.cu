@@ -36,12 +36,13 @@ kp_status cuda_error(kp_ctx* c, cudaError_t e, const char* what) {
 }
 
 cudaError_t launch_solver(const GmresParams& p, const Shape& sh, bool mixed, cudaStream_t st) {
-  if (sh.cs > 0) return launch_gmres_cluster(p, sh.ept, sh.nt, sh.cs, sh.minb, sh.smem, st);
-  return mixed ? launch_gmres_mixed(p, sh.ept, sh.nt, sh.smem, st)
+  if (sh.cs > 0) return launch_gmres_cluster(p, sh.ept, sh.nt, sh.cs, sh.reg, sh.smem, st);
+  return mixed ? launch_gmres_mixed(p, sh.ept, sh.nt, sh.reg, sh.smem, st)
                : launch_gmres_fp64(p, sh.ept, sh.nt, sh.minb, sh.smem, st);
 }
 
-kp_status gmres_shape(kp_ctx* c, int nmax, int m, Shape* out, bool mixed, int wmin) {
+kp_status gmres_shape(kp_ctx* c, int nmax, int m, Shape* out, bool mixed, int wmin, int hmax,
+                      bool one_size) {
   Shape sh;
   sh.minb = 1;
   if (nmax <= 1024) {
@@ -53,15 +54,19 @@ kp_status gmres_shape(kp_ctx* c, int nmax, int m, Shape* out, bool mixed, int wm
     sh.ept = 1024 / sh.nt;
     sh.minb = c->opt.blocks_per_sm ? c->opt.blocks_per_sm : (sh.nt == 128 && !c->opt.block_threads ? 4
                                                              : sh.nt == 64 ? 4 : 2);
-    if (mixed) {                                 // the FP32 solver has the 2-block 256/128 shapes
-      sh.minb = 2;
+    if (mixed) {                                 // the FP32 solver has the 256- and 128-thread shapes
       if (sh.nt == 64) { sh.nt = 128; sh.ept = 8; }
+      sh.minb = sh.nt == 128 ? 6 : 4;
     }
-  }
-  else if (nmax <= 4096 && !(mixed && c->opt.cluster_size)) { sh.ept = 8; sh.nt = 512; }
-  else if (mixed) {
-    // a cluster of cs CTAs, each holding W/cs whole columns (<= 2048 points;
-    // 16-CTA clusters: 128 threads and <= 1024 points per CTA)
+  } else if (nmax <= 4096 && !(mixed && c->opt.cluster_size)) {
+    sh.ept = 8;
+    sh.nt = 512;
+    if (mixed) sh.minb = 2;
+  } else if (mixed) {
+    // a cluster of CTAs, each holding whole columns: on request 2, 4 or 8 of
+    // 256 threads and <= 2048 points, or 16 of 128 threads and <= 1024 points;
+    // by default half as many CTAs of <= 4096 points (the grid's width has to
+    // be divisible by the cluster of 2048-point CTAs either way)
     sh.ept = 8; sh.nt = c->opt.cluster_size == 16 ? 128 : 256;
     if (c->opt.cluster_size) {
       if ((nmax + c->opt.cluster_size - 1) / c->opt.cluster_size <= sh.ept * sh.nt) sh.cs = c->opt.cluster_size;
@@ -74,29 +79,43 @@ kp_status gmres_shape(kp_ctx* c, int nmax, int m, Shape* out, bool mixed, int wm
     sh.minb = c->opt.cluster_blocks_per_sm ? c->opt.cluster_blocks_per_sm : (sh.cs == 16 ? 4 : 2);
     if (sh.cs == 16 ? (sh.minb != 2 && sh.minb != 4) : sh.minb > 2)
       return set_error(c, KP_ERR_UNSUPPORTED, "cluster of %d CTAs: %d CTAs per SM not built", sh.cs, sh.minb);
+    if (!c->opt.cluster_size) { sh.cs /= 2; sh.nt = 512; }
+  } else {
+    return set_error(c, KP_ERR_UNSUPPORTED, "N=%d: FP64 grids above 4096 unknowns are not supported (use the mixed-precision mode)", nmax);
   }
-  else return set_error(c, KP_ERR_UNSUPPORTED, "N=%d: FP64 grids above 4096 unknowns are not supported (use the mixed-precision mode)", nmax);
   const int npad = sh.ept * sh.nt;
-  const size_t fixed = sh.cs ? gmres_cluster_smem_bytes(sh.ept, sh.nt, 0, m)
-                     : mixed ? gmres_mixed_smem_bytes(sh.ept, sh.nt, 0, m)
-                             : gmres_fp64_smem_bytes(sh.ept, sh.nt, 0, m);
-  const size_t per = (size_t)npad * (mixed ? sizeof(float) : sizeof(double));
+  sh.vld = npad;
+  if (mixed) {
+    // full CTAs, columns that divide the threads of a sub-block (half a CTA
+    // of the default clusters); the shapes on request have no such kernel
+    const int ns = sh.cs ? 256 : sh.nt;
+    sh.reg = one_size && nmax == sh.ctas() * npad && hmax > 0 && ns % hmax == 0 && !c->opt.cluster_size && sh.nt != 128;
+    sh.hmax = sh.cs || sh.reg ? hmax : 0;
+    sh.vld += 2 * sh.hmax;
+  }
+  auto bytes = [&](int S) {
+    return mixed ? gmres_mixed_smem_bytes(sh.nt, sh.ctas(), sh.hmax, sh.vld, S, m)
+                 : gmres_fp64_smem_bytes(sh.ept, sh.nt, S, m);
+  };
+  // shared memory of one CTA when minb of them share an SM (1 KB per CTA is
+  // reserved by the hardware)
+  const size_t budget = mixed ? c->smem_optin / sh.minb - (sh.minb >= 2 ? 1024 : 0)
+                      : npad <= 1024 ? c->smem_optin / sh.minb - (sh.minb > 2 ? 1024 : 0)
+                                     : c->smem_optin;
+  // the mixed-precision solver keeps x (hi, lo) in two slots between cycles
+  const int smin = mixed ? 2 : 1;
   int S = c->opt.smem_vectors;
   if (S <= 0) {
-    // small systems: leave room for minb resident blocks per SM (1 KB of
-    // shared memory per block is reserved by the hardware)
-    // (clusters: every CTA of a system's cluster sits on its own SM, and MINB
-    // systems' CTAs share one)
-    const size_t budget = sh.cs ? c->smem_optin / sh.minb - (sh.minb >= 2 ? 1024 : 0)
-                        : npad <= 1024 ? c->smem_optin / sh.minb - (sh.minb > 2 ? 1024 : 0)
-                                       : c->smem_optin;
-    S = budget > fixed ? (int)((budget - fixed) / per) : 0;
+    S = smin;
+    while (S < m + 1 && bytes(S + 1) <= budget) ++S;
   }
-  S = std::min(S, m + 1);
-  while (S > 1 && fixed + S * per > c->smem_optin) --S;
-  if (S < 1) return set_error(c, KP_ERR_UNSUPPORTED, "shared memory too small");
+  S = std::max(std::min(S, m + 1), smin);
+  while (S > smin && bytes(S) > c->smem_optin) --S;
+  if (bytes(S) > c->smem_optin) return set_error(c, KP_ERR_UNSUPPORTED, "shared memory too small");
   sh.S = S;
-  sh.smem = fixed + S * per;
+  sh.smem = bytes(S);
+  sh.ws = (size_t)std::max(m + 1 - S, 0) * sh.vld + (mixed ? 2 * (size_t)sh.vld + 2 * (size_t)npad : 0);
+  sh.ws = (sh.ws + 1) / 2 * 2;                   // (x and the coefficients are float pairs)
   *out = sh;
   return KP_OK;
 }
@@ -183,6 +202,7 @@ SysDesc make_desc(const kp_op& o, const double* b, double* x, int slot) {
   d.h = o.h;
   d.slot = slot;
   d.pad_ = 0;
+  kp::set_quotients(&d, 1.0);
   return d;
 }
 
@@ -201,20 +221,22 @@ kp_status run_gmres(kp_ctx* c, int nsys, const kp_op* ops, const double* const* 
   for (int k = 0; k < nsys; ++k) {
     if (!ops[k].mtilde || !b[k] || !x[k]) return kp::set_error(c, KP_ERR_ARG, "system %d: NULL vector", k);
   }
-  int wmin = 1 << 30;
-  for (int k = 0; k < nsys; ++k) wmin = std::min(wmin, ops[k].W);
+  int wmin = 1 << 30, hmax = 0;
+  bool one_size = true;
+  for (int k = 0; k < nsys; ++k) {
+    wmin = std::min(wmin, ops[k].W);
+    hmax = std::max(hmax, ops[k].H);
+    one_size = one_size && ops[k].H == ops[0].H && ops[k].W == ops[0].W;
+  }
   for (int k = 0; k < nsys && nmax > 4096; ++k)
     if ((long long)ops[k].H * ops[k].W != nmax)
       return kp::set_error(c, KP_ERR_UNSUPPORTED, "grids above 4096 unknowns must share one size per call");
   kp::Shape sh;
-  st = kp::gmres_shape(c, nmax, m, &sh, mixed, wmin);
+  st = kp::gmres_shape(c, nmax, m, &sh, mixed, wmin, hmax, one_size);
   if (st != KP_OK) return st;
-  const int ept = sh.ept, nt = sh.nt, S = sh.S, npad = ept * nt;
-  const size_t smem = sh.smem;
   cudaError_t e;
-  if (S < m + 1) {
-    const size_t need = (size_t)nsys * (sh.cs ? sh.cs : 1) * (m + 1 - S) * npad *
-                        (mixed ? sizeof(float) : sizeof(double));
+  if (sh.ws) {
+    const size_t need = (size_t)nsys * sh.ctas() * sh.ws * (mixed ? sizeof(float) : sizeof(double));
     e = mixed ? grow(&c->spill32, &c->spill32_bytes, need) : grow(&c->spill, &c->spill_bytes, need);
     if (e != cudaSuccess) return kp::cuda_error(c, e, "cudaMalloc(Krylov workspace)");
   }
@@ -247,14 +269,13 @@ kp_status run_gmres(kp_ctx* c, int nsys, const kp_op* ops, const double* const* 
   p.tol = tol;
   p.m = m;
   p.maxit = maxit;
-  p.S = S;
+  kp::set_shape(&p, sh);
   p.reorth = c->opt.reorth;
   p.inner_eta = kp::inner_eta(c->opt);
-  p.npad = npad;
   p.b_scale = 1.0;
   p.x0_mode = kp::X0_READ;
-  p.spill = (!mixed && S < m + 1) ? c->spill : nullptr;
-  p.spill32 = (mixed && S < m + 1) ? c->spill32 : nullptr;
+  p.spill = (!mixed && sh.ws) ? c->spill : nullptr;
+  p.spill32 = mixed ? c->spill32 : nullptr;
   p.info = info;
   if (capture) {
     p.capV = c->capV;
@@ -265,7 +286,6 @@ kp_status run_gmres(kp_ctx* c, int nsys, const kp_op* ops, const double* const* 
     p.cap_ld = c->opt.max_n;
     p.fixed_a = c->opt.fixed_a;
   }
-  (void)ept; (void)nt; (void)smem;
   e = kp::launch_solver(p, sh, mixed, c->stream);
   if (e != cudaSuccess) return kp::cuda_error(c, e, "GMRES launch");
   return KP_OK;

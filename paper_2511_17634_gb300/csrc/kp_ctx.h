@@ -74,14 +74,32 @@ struct Shape {
   int minb = 1;   // resident blocks per SM the kernel is compiled for (launch bounds)
   size_t smem = 0;
   int cs = 0;   // > 0: thread-block cluster of cs CTAs per system (slices of W/cs columns)
+  // device workspace of a CTA, in values of the vectors' type: the Krylov
+  // vectors past the shared-memory window; mixed precision also x and the low
+  // parts of the operator coefficients
+  size_t ws = 0;
+  int vld = 0;    // values of a vector slot (mixed precision on a cluster: with its halo columns)
+  int hmax = 0;   // longest column of the systems (mixed precision with halo columns)
+  bool reg = false;   // mixed precision: see launch_gmres_mixed
+  int ctas() const { return cs ? cs : 1; }
 };
 
 kp_status set_error(kp_ctx* c, kp_status s, const char* fmt, ...);
 kp_status cuda_error(kp_ctx* c, cudaError_t e, const char* what);
 // Chooses threads, elements per thread and the shared-memory Krylov window
-// (FP64 vectors, or FP32 ones for the mixed-precision solver).
+// (FP64 vectors, or FP32 ones for the mixed-precision solver).  wmin, hmax:
+// narrowest and longest grid of the systems, one_size: they are all hmax x
+// (nmax / hmax) (mixed precision).
 kp_status gmres_shape(kp_ctx* c, int nmax, int m, Shape* out, bool mixed = false,
-                      int wmin = 0);
+                      int wmin = 0, int hmax = 0, bool one_size = false);
+// The shape's part of the solver parameters and the CTAs' workspace.
+inline void set_shape(GmresParams* p, const Shape& sh) {
+  p->S = sh.S;
+  p->npad = sh.ept * sh.nt;
+  p->vld = sh.vld;
+  p->hmax = sh.hmax;
+  p->ws_ld = sh.ws;
+}
 // Inner FP32 residual reduction of the mixed-precision solvers.
 inline double inner_eta(const kp_options& o) {
   static const double k[8] = {1e-5, 1e-1, 1e-2, 1e-3, 1e-4, 1e-5, 1e-6, 1e-7};

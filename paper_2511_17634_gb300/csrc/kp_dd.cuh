@@ -19,7 +19,7 @@
 // integer operations (no FP64 instruction): hi = x truncated to 24
 // significant bits, lo = the remaining 29 bits rounded to 24; |x| < 2^-74 maps
 // to (hi, 0) and below 2^-100 to zero, far under any quantity the solvers
-// compare.  dd_to_double is exact (hi + lo has at most 48 significant bits).
+// compare.  dd_to_double rounds hi + lo to FP64 (exact up to 53 significant bits).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -57,7 +57,7 @@ __device__ __forceinline__ dd dd_add_f(dd x, float y) {
 }
 
 __device__ __forceinline__ dd dd_mul(dd x, dd y) {
-  const float p = x.hi * y.hi;
+  const float p = __fmul_rn(x.hi, y.hi);   // (never contracted with the sum below)
   float e = fmaf(x.hi, y.hi, -p);
   e = fmaf(x.hi, y.lo, e);
   e = fmaf(x.lo, y.hi, e);
@@ -78,7 +78,43 @@ __device__ __forceinline__ dd dd_from_double(double x) {
   return {hi, __uint2float_rn(ul & 0x1FFFFFFFu) * scale};
 }
 
-__device__ __forceinline__ double dd_to_double(dd x) { return (double)x.hi + (double)x.lo; }
+// 1 / sqrt(x) for x > 0: the FP32 estimate y and one correction from the
+// residual e = 1 - x y^2 taken in double-float, y (1 + e/2 + 3 e^2/8)
+// (Taylor's series of (1 - e)^(-1/2); e is about 1e-7, so the next term is
+// below 2^-60).
+__device__ __forceinline__ dd dd_rsqrt(dd x) {
+  const float y = rsqrtf(x.hi);
+  const float q = __fmul_rn(y, y), ql = fmaf(y, y, -q);              // y^2 = q + ql exactly
+  const float p = __fmul_rn(x.hi, q);
+  const float pl = fmaf(x.hi, ql, fmaf(x.lo, q, fmaf(x.hi, q, -p)));
+  const float e = (1.f - p) - pl;
+  return dd_fast_two_sum(y, y * (e * fmaf(0.375f, e, 0.5f)));
+}
+
+// sqrt(x) for x >= 0: the FP32 root and one Newton correction.
+__device__ __forceinline__ dd dd_sqrt(dd x) {
+  const float y = sqrtf(x.hi);
+  if (!(y > 0.f) || isinf(y)) return {y, 0.f};             // zero, NaN, Inf
+  const float r = fmaf(-y, y, x.hi) + x.lo;
+  return dd_fast_two_sum(y, r * (0.5f / y));
+}
+
+// hi + lo rounded to FP64.  A conversion and an add on the FP64 pipe cost
+// three warp instructions of 64 cycles each; this composes the bit pattern
+// with integer operations: hi's pattern plus lo as a signed count of units in
+// the last place of hi's binade (of the binade below where hi is a power of
+// two and lo points towards zero).  Values outside the range where that count
+// is an ordinary float go through the conversions.
+__device__ __forceinline__ double dd_to_double(dd x) {
+  const unsigned int u = __float_as_uint(x.hi);
+  const unsigned int e = (u >> 23) & 0xFFu;
+  if (e < 56 || e > 254) return (double)x.hi + (double)x.lo;   // small, zero, Inf, NaN
+  const float lo = (u >> 31) ? -x.lo : x.lo;                   // relative to |hi|
+  const unsigned int below = (u & 0x7FFFFFu) == 0u && lo < 0.f;
+  const int t = __float2int_rn(lo * __uint_as_float((306u + below - e) << 23));
+  const unsigned long long m = ((unsigned long long)(e + 896u) << 52) + ((unsigned long long)(u & 0x7FFFFFu) << 29);
+  return __longlong_as_double((long long)((m + (long long)t) | ((unsigned long long)(u & 0x80000000u) << 32)));
+}
 
 // The FP32 value nearest to x (ties to even) by integer operations on its bit
 // pattern -- the top 24 significant bits, rounded on the 29 below -- for x in

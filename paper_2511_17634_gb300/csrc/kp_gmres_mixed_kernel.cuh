@@ -1,0 +1,881 @@
+// kp_gmres_mixed_kernel.cuh -- mixed-precision solver for the five-point
+// systems of Sec. 2.3: iterative refinement around an FP32 restarted GMRES,
+// one CTA per system (grids of up to 4096 points, kp_gmres_mixed.cu) or one
+// thread-block cluster of CS CTAs per system (kp_gmres_cluster.cu), CTA r
+// holding columns [r W/CS, (r+1) W/CS) of every vector (whole columns, so
+// north/south neighbours stay local).
+//
+// Precision.  The Krylov work (stencil, Gram-Schmidt updates, normalisation)
+// is FP32 on FP32 vectors.  The refinement's high-precision arithmetic -- the
+// solution x, the operator coefficients and the true residual r = b - A x --
+// and the small least-squares problem (Hessenberg matrix, Givens rotations,
+// back substitution, the projection's triangular solve) are double-float
+// (kp_dd.cuh: a pair of floats, about 48 bits).  Inner products of FP32
+// vectors are summed in FP32 within a CTA and in double-float across CTAs.
+// Outer loop: r = b - A x; inner GMRES(m) on A d = r in FP32 until the
+// residual estimate drops by eta = 1e-5 (FP32 cannot resolve much more) or to
+// half the outer target (kInnerFloor); x += d.  The outer loop stops on the
+// true residual, so every returned solve meets ||b - A x|| <= tol ||b||.  The
+// residual's error is a few units of 2^-44 times ||b||, far below every
+// tolerance the solver is asked for (>= 1e-12).
+//
+// No FP64 instruction runs per step.  GB300 issues an FP64 warp instruction
+// over 64 cycles of one scheduler, whether one lane or 32 take part, so a
+// Givens step of some 60 FP64 instructions on one lane held up its CTA for
+// about 2 us per Arnoldi step, and the FP64 pipe of that one scheduler was
+// 75 % (64x64) to 86 % (128x128) busy: it bounded the kernel.  In
+// double-float the same chain is about 0.2 us.
+//
+// Barriers.  A reduction's per-warp partials go to every CTA of the cluster
+// (distributed shared memory); after one barrier every warp adds all of them
+// itself, in the same order, so the coefficients need no second barrier and
+// are bit-identical everywhere.  Warp 0 takes the Givens step beside its
+// vector work; its stop flag is read at the barrier that v_{j+1} needs in any
+// case.  Halos: every CTA keeps its neighbours' edge columns of each Krylov
+// vector and of x.  Only w = A v_j crosses the cluster (its edge columns are
+// pushed with the partials); v_{j+1} and x on the halo follow from the same
+// coefficients by the same operations as in the neighbour, bit for bit.  That
+// leaves one cluster barrier per Arnoldi step (without a second Gram-Schmidt
+// pass) and one per residual.
+//
+// Memory.  Shared memory holds the first S Krylov vectors; the others, x and
+// the low parts of the coefficients live in a per-CTA device workspace (L2).
+// During a residual the first two vector slots hold x (hi, lo): the Krylov
+// vectors are dead by then.  Two 256-thread CTAs of 4096 points share an SM,
+// so that one system's barriers and serial work overlap the other's vector
+// work.
+//
+// The operator is applied from q_x = f_x/(2h) - e (m~_E - m~_W) and q_y per
+// point:
+//   A x = cd x_p - c (x_E + x_W + x_N + x_S) + q_x (x_E - x_W) + q_y (x_N - x_S)
+// with out-of-grid neighbours zero -- algebraically the coefficients of the
+// listing after Eq. 11.  The Arnoldi process runs on A - cd I (same Krylov
+// space, H_A = H + cd I), which avoids the cancellation of the large
+// diagonal in Gram-Schmidt -- in FP32 it would cost a digit per step.
+#pragma once
+
+#include <cooperative_groups.h>
+
+#include "kp_dd.cuh"
+#include "kp_internal.cuh"
+
+namespace kp {
+namespace {
+
+// Values per reduction round: longer Gram-Schmidt sums take several rounds
+// (and barriers), which keeps the partials of 32 warps within 4 KB.
+constexpr int kRedV = 16;
+
+__device__ __forceinline__ float2 as_f2(dd x) { return make_float2(x.hi, x.lo); }
+__device__ __forceinline__ dd as_dd(float2 x) { return {x.x, x.y}; }
+
+// Warp reduce-scatter of 4 FP32 values per lane: every lane ends with the
+// warp sum of value lane >> 3.
+__device__ __forceinline__ float warp_reduce4f(float (&a)[4], int lane) {
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const bool up = lane & 16;
+    const float send = up ? a[k] : a[k + 2];
+    const float keep = up ? a[k + 2] : a[k];
+    a[k] = keep + __shfl_xor_sync(kFull, send, 16);
+  }
+  {
+    const bool up = lane & 8;
+    const float send = up ? a[0] : a[1];
+    const float keep = up ? a[1] : a[0];
+    a[0] = keep + __shfl_xor_sync(kFull, send, 8);
+  }
+  a[0] += __shfl_xor_sync(kFull, a[0], 4);
+  a[0] += __shfl_xor_sync(kFull, a[0], 2);
+  a[0] += __shfl_xor_sync(kFull, a[0], 1);
+  return a[0];
+}
+
+// alpha = R^{-1} (G c) in double-float by one warp (the double-float form of
+// solve_projected_warp): c in shared memory, a <= 64, the FP64 factors split
+// as they are loaded, eight columns of R ahead of their use.  alpha -> out
+// (FP32).  Every lane of the warp calls it; ends with __syncwarp.
+__device__ __forceinline__ void solve_projected_dd(float2* c, int a, int nrot, const double* R, int ld,
+                                                   const double* rot, const double* rinv, float* out, int lane) {
+  // rotations: lane l holds pairs l and l + 32, every lane follows the chain
+  dd rc[2], rs[2], ri[2];
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const int l = lane + 32 * u;
+    rc[u] = l < nrot ? dd_from_double(rot[2 * l]) : dd{1.f, 0.f};
+    rs[u] = l < nrot ? dd_from_double(rot[2 * l + 1]) : dd{0.f, 0.f};
+    ri[u] = l < a ? dd_from_double(rinv[l]) : dd{0.f, 0.f};
+  }
+  auto bcast = [&](const dd (&v)[2], int j) -> dd {
+    const dd s = j < 32 ? v[0] : v[1];
+    return {__shfl_sync(kFull, s.hi, j & 31), __shfl_sync(kFull, s.lo, j & 31)};
+  };
+  dd cur = as_dd(c[0]);
+  dd g[2] = {{0.f, 0.f}, {0.f, 0.f}};
+  auto put = [&](int j, dd v) {
+    if (lane == (j & 31)) g[j >> 5] = v;
+  };
+  int j = 0;
+  for (; j < nrot; ++j) {
+    const dd cc = bcast(rc, j), s = bcast(rs, j), nx = as_dd(c[j + 1]);
+    put(j, dd_add(dd_mul(cc, cur), dd_mul(s, nx)));
+    cur = dd_sub(dd_mul(cc, nx), dd_mul(s, cur));
+  }
+  if (j < a) put(j, cur);
+  for (++j; j < a; ++j) put(j, as_dd(c[j]));
+  for (int i0 = a - 1; i0 >= 0; i0 -= 8) {
+    double r0[8], r1[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int i = i0 - u;
+      r0[u] = (i >= 0 && lane < i) ? R[lane + (size_t)i * ld] : 0.0;
+      r1[u] = (i >= 0 && lane + 32 < i) ? R[lane + 32 + (size_t)i * ld] : 0.0;
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int i = i0 - u;
+      if (i < 0) break;
+      const dd ai = dd_mul(bcast(g, i), bcast(ri, i));
+      if (lane == 0) out[i] = ai.hi;
+      if (lane < i) g[0] = dd_sub(g[0], dd_mul(dd_from_double(r0[u]), ai));
+      if (lane + 32 < i) g[1] = dd_sub(g[1], dd_mul(dd_from_double(r1[u]), ai));
+    }
+  }
+  __syncwarp();
+}
+
+// SUB: sub-blocks of a CTA, each with its own half of the slice (SUB = 2: the
+// sums then have the bits of twice as many CTAs of half the threads, whose
+// FP32 sums stop at the CTA).  REG: every system of the launch fills its CTAs
+// (N = CS EPT NT) and its columns divide a sub-block's threads, so that all of
+// a thread's points share one row j: two neighbour flags per thread instead of
+// four bits per point, no guards, and zero halo columns beside the grid (66
+// against 89 instructions per point and step; the launcher decides).
+template <int EPT, int NT, int CS, int MINB, int SUB, bool REG>
+__global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams p) {
+  namespace cg = cooperative_groups;
+  constexpr int NS = NT / SUB;                   // threads of a sub-block
+  constexpr int VC = CS * SUB;                   // sub-blocks of a system
+  constexpr int P = (NS / 32) * VC;              // per-warp partials of one value
+  constexpr int PL = P < 32 ? P : 32;            // lanes that add them
+  constexpr bool HALO = CS > 1 || REG;
+  static_assert(EPT <= 8, "the neighbour bits of a thread fill one word");
+  extern __shared__ __align__(16) unsigned char smem_mx[];
+  cg::cluster_group cluster = cg::this_cluster();
+  const int rank = CS > 1 ? (int)cluster.block_rank() : 0;
+  const int m = p.m;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int sub = SUB > 1 ? tid / NS : 0, st = SUB > 1 ? tid % NS : tid;
+  // shared-memory carve (identical offsets in every CTA of the cluster);
+  // gmres_mixed_smem_bytes counts the same pieces
+  float2* cs = reinterpret_cast<float2*>(smem_mx);            // [m]
+  float2* sn = cs + m;                                        // [m]
+  float2* rinv = sn + m;                                      // [m]
+  float2* gv = rinv + m;                                      // [m + 1]
+  float2* hball = gv + m + 1;                                 // [NT / 32][kMaxV] sums, a copy per warp
+  float2* hb = hball + warp * kMaxV;
+  float* red = reinterpret_cast<float*>(hball + (NT / 32) * kMaxV);   // [2][kRedV][P]
+  float* yf = red + 2 * kRedV * P;                            // [kMaxV] combination coefficients
+  int* fl = reinterpret_cast<int*>(yf + kMaxV);               // [8]
+  float* whalo = reinterpret_cast<float*>(fl + 8);            // [2][2 hmax] pushed edge columns
+  float2* Hr = reinterpret_cast<float2*>(whalo + 4 * p.hmax); // packed columns of R: j at j (j + 1) / 2
+  float* V = reinterpret_cast<float*>(Hr + m * (m + 1) / 2);  // [S][vld]
+  const int vld = p.vld;
+  // workspace of this CTA: x (hi, lo) over the extended slice, the low parts
+  // of q_x, q_y, then the Krylov vectors past the shared-memory window
+  float2* xs = reinterpret_cast<float2*>(p.spill32 + (size_t)blockIdx.x * p.ws_ld);
+  float2* ql = xs + vld;
+  float* Vg = reinterpret_cast<float*>(ql + EPT * NT);
+  auto slot = [&](int i) -> float* {
+    return i < p.S ? V + (size_t)i * vld : Vg + (size_t)(i - p.S) * vld;
+  };
+  int tstep = 0;
+  if (p.step) {
+    tstep = *p.step + p.step_offset;
+    if (tstep >= *p.step_end) return;            // uniform over the whole grid
+  }
+  const int parity_base = slot_set_base(p, tstep);
+  const float kEta = p.inner_eta > 0.0 ? (float)p.inner_eta : 1e-5f;
+  int buf = 0, hbuf = 0;                         // parities of the reductions and of the halo pushes
+
+  for (int sysi = blockIdx.x / CS; sysi < p.nsys; sysi += gridDim.x / CS) {
+    const SysDesc d = p.sys[sysi];
+    const int H = d.H, W = d.W, N = H * W;
+    const int SL = N / CS;                       // slice length (whole columns)
+    const int SH = SL / SUB;                     // a sub-block's part
+    const int base = rank * SL;
+    const int hal = HALO ? H : 0;                // halo columns before and after the slice
+    const int l0 = sub * SH + st;                // this thread's points l0 + k NS of the slice
+    auto inside = [&](int k) { return REG || st + k * NS < SH; };
+    // points past the slice (w = 0 there): on one CTA their slots hold zeros;
+    // on a cluster that space is the halo's, so short slices are guarded
+    const bool full = REG || CS == 1 || SH == EPT * NS;
+    // the operator constants c = g^2/(2h^2), e = c/4, c_d = 1/dt + 4c from the
+    // descriptor's quotients: a division is a dozen FP64 instructions on
+    // every warp.  Solved as (A / s) x = b / s with s = b_scale: the scale is
+    // in those quotients instead of on every point of b.
+    const double g2 = p.step ? p.g2_sched[tstep] : d.g2;
+    const double cc = g2 * d.kc;
+    const dd ccd = dd_from_double(cc), cdd = dd_from_double(fma(4.0, cc, d.kd));
+    const float ccf = ccd.lo + ccd.hi;
+    const bool capture = p.capV32 != nullptr;
+    const int cidx = p.factor ? parity_base + sysi : sysi;
+    float* capV = capture ? p.capV32 + (size_t)cidx * (p.cap_a + 1) * p.cap_ld : nullptr;
+    double* capH = capture ? p.capH + (size_t)cidx * (p.cap_a + 1) * p.cap_a : nullptr;
+
+    // fn(index in a vector slot, point of the grid or -1 outside) over this
+    // thread's points of the slice and of its halo columns
+    auto each_ext = [&](auto&& fn) {
+#pragma unroll
+      for (int k = 0; k < EPT; ++k)
+        if (inside(k)) fn(hal + l0 + k * NS, base + l0 + k * NS);
+      if (CS > 1)
+        for (int q = tid; q < 2 * H; q += NT) {
+          const int pp = q < H ? base - H + q : base + SL + q - H;
+          fn(q < H ? q : SL + q, (unsigned)pp < (unsigned)N ? pp : -1);
+        }
+    };
+    // x (hi, lo) lives in the workspace and, outside the Krylov phases, in the
+    // first two vector slots
+    float* xh = V;
+    float* xl = V + vld;
+    auto put_x = [&](int at, dd v) {
+      xh[at] = v.hi;
+      xl[at] = v.lo;
+      xs[at] = as_f2(v);
+    };
+    // x = u + yf-combination of the nc rows U (indexed by grid point)
+    auto add_basis = [&](const float* U, int nc, bool from_zero) {
+      each_ext([&](int at, int pp) {
+        float xv = 0.f;
+        if (pp >= 0)
+          for (int i = 0; i < nc; ++i) xv = fmaf(yf[i], U[(size_t)i * p.slot_ld + pp], xv);
+        put_x(at, from_zero ? dd{xv, 0.f} : dd_add_f(dd{xh[at], xl[at]}, xv));
+      });
+    };
+    auto load_x = [&](const double* src) {
+      each_ext([&](int at, int pp) { put_x(at, src && pp >= 0 ? dd_from_double(src[pp]) : dd{0.f, 0.f}); });
+    };
+    // zero columns beside the grid, in the shared-memory slots (REG on one CTA)
+    auto zero_halo = [&]() {
+      if (REG && CS == 1)
+        for (int q = tid; q < p.S * 2 * H; q += NT) {
+          const int r = q / (2 * H), o = q - r * 2 * H;
+          V[(size_t)r * vld + (o < H ? o : SL + o)] = 0.f;
+        }
+    };
+
+    // neighbours of this thread's points: 1 E, 2 W, 4 N, 8 S per point (REG:
+    // N and S of all its points).  With halo columns E and W are always there.
+    unsigned msk = 0;
+    if (REG) {
+      const int j = l0 % H;
+      msk = (j + 1 < H ? 4u : 0u) | (j > 0 ? 8u : 0u);
+    } else {
+#pragma unroll
+      for (int k = 0; k < EPT; ++k)
+        if (inside(k)) {
+          const int pp = base + l0 + k * NS;
+          const int i = pp / H, j = pp - i * H;
+          msk |= ((CS > 1 || i + 1 < W ? 1u : 0u) | (CS > 1 || i > 0 ? 2u : 0u) | (j + 1 < H ? 4u : 0u) |
+                  (j > 0 ? 8u : 0u)) << (4 * k);
+        }
+    }
+    const bool rN = msk & 4u, rS = msk & 8u;
+    auto nbE = [&](const float* v, int at, int k) { return REG || (msk & (1u << (4 * k))) ? v[at + H] : 0.f; };
+    auto nbW = [&](const float* v, int at, int k) { return REG || (msk & (2u << (4 * k))) ? v[at - H] : 0.f; };
+    auto nbN = [&](const float* v, int at, int k) {
+      if (REG) { const float t = v[at + 1]; return rN ? t : 0.f; }
+      return (msk & (4u << (4 * k))) ? v[at + 1] : 0.f;
+    };
+    auto nbS = [&](const float* v, int at, int k) {
+      if (REG) { const float t = v[at - 1]; return rS ? t : 0.f; }
+      return (msk & (8u << (4 * k))) ? v[at - 1] : 0.f;
+    };
+
+    // the lagged field, then q_x, q_y (hi parts in registers for the Krylov
+    // operator, low parts in the workspace for the residual)
+    if (CS > 1)
+      for (int q = tid; q < 4 * H; q += NT) whalo[q] = 0.f;
+    zero_halo();
+    load_x(d.mt);
+    if (CS == 1) __syncthreads();
+    else cluster.sync();                         // (every CTA runs and its halo buffer is zero)
+    float qx[EPT], qy[EPT];
+    {
+      const dd eed = {0.25f * ccd.hi, 0.25f * ccd.lo};
+      const dd i2hd = dd_from_double(d.ki);
+#pragma unroll
+      for (int k = 0; k < EPT; ++k) {
+        const int at = hal + l0 + k * NS;
+        qx[k] = qy[k] = 0.f;
+        if (inside(k)) {
+          const dd mE = {nbE(xh, at, k), nbE(xl, at, k)}, mW = {nbW(xh, at, k), nbW(xl, at, k)};
+          const dd mN = {nbN(xh, at, k), nbN(xl, at, k)}, mS = {nbS(xh, at, k), nbS(xl, at, k)};
+          dd x = dd_mul(eed, dd_sub(mW, mE)), y = dd_mul(eed, dd_sub(mS, mN));
+          const int pp = base + l0 + k * NS;
+          if (d.fx) x = dd_add(x, dd_mul(dd_from_double(d.fx[pp]), i2hd));
+          if (d.fy) y = dd_add(y, dd_mul(dd_from_double(d.fy[pp]), i2hd));
+          qx[k] = x.hi;
+          qy[k] = y.hi;
+          ql[l0 + k * NS] = make_float2(x.lo, y.lo);
+        }
+      }
+    }
+
+    float w[EPT];                                // r, then w = A v_j
+    float bb = 0.f, sw = 0.f;                    // this thread's part of ||b||^2, of the warm start's ||r||^2
+    auto sumsq = [&]() {
+      float s = 0.f;
+#pragma unroll
+      for (int k = 0; k < EPT; ++k) s = fmaf(w[k], w[k], s);
+      return s;
+    };
+    // push this CTA's edge columns of w to the neighbours' halo buffers
+    // (visible after the next cluster barrier)
+    auto push_edges = [&]() {
+      if (CS == 1) return;
+      float* wl = rank > 0 ? cluster.map_shared_rank(whalo, rank - 1) + hbuf * 2 * p.hmax + H : nullptr;
+      float* wr = rank + 1 < CS ? cluster.map_shared_rank(whalo, rank + 1) + hbuf * 2 * p.hmax : nullptr;
+#pragma unroll
+      for (int k = 0; k < EPT; ++k) {
+        const int l = l0 + k * NS;
+        if (wl && inside(k) && l < H) wl[l] = w[k];
+        if (wr && inside(k) && l >= SL - H) wr[l - (SL - H)] = w[k];
+      }
+    };
+    // sums over the system of nv values part(0..nv-1) -> hb[0..nv) of every
+    // warp of every CTA, identical bits; ends with __syncwarp
+    auto reduce = [&](int nv, auto&& part) {
+      for (int c0 = 0; c0 < nv; c0 += kRedV) {
+        const int nc = min(kRedV, nv - c0);
+        float* rb = red + buf * kRedV * P;
+#pragma unroll 1
+        for (int i0 = 0; i0 < nc; i0 += 4) {
+          float a[4];
+          part(c0 + i0, nv, a);
+          const float s = warp_reduce4f(a, lane);
+          const int v = i0 + (lane >> 3);
+          const int q = (warp % (NS / 32)) * VC + rank * SUB + sub;
+          if (v < nc) {
+            if (CS == 1) {
+              if ((lane & 7) == 0) rb[v * P + q] = s;
+            } else {
+              for (int r = lane & 7; r < CS; r += 8) cluster.map_shared_rank(rb, r)[v * P + q] = s;
+            }
+          }
+        }
+        if (CS == 1) __syncthreads();
+        else cluster.sync();
+#pragma unroll 1
+        for (int i0 = 0; i0 < nc; i0 += 32 / PL) {
+          const int i = i0 + lane / PL, q = lane % PL;
+          float s = 0.f, e = 0.f;
+          if (i < nc) {
+            s = rb[i * P + q];
+            if (P > 32) s += rb[i * P + (q + 32) % P];
+          }
+#pragma unroll
+          for (int o = PL / 2; o >= VC; o /= 2) s += __shfl_xor_sync(kFull, s, o);   // warps of a sub-block
+#pragma unroll
+          for (int o = VC / 2; o > 0; o /= 2) {                                      // sub-blocks
+            const float so = __shfl_xor_sync(kFull, s, o), eo = __shfl_xor_sync(kFull, e, o);
+            const dd t = dd_two_sum(s, so);
+            s = t.hi;
+            e = (e + eo) + t.lo;
+          }
+          if (q == 0 && i < nc) hb[c0 + i] = as_f2(dd_fast_two_sum(s, e));
+        }
+        buf ^= 1;
+      }
+      __syncwarp();
+    };
+
+    // ---- initial guess
+    const bool judge = p.x0_mode == X0_GUESS_PROJECT;
+    unsigned long long proj_flops = 0;
+    const int sl = d.slot + parity_base;         // the target's seed basis
+    const float* U = p.slotV32 + (size_t)sl * (p.max_a + 1) * p.slot_ld;
+    SlotMeta mt;
+    mt.a = 0;
+    if (judge || p.x0_mode == X0_PROJECT || p.x0_mode == X0_GALERKIN) {
+      mt = p.slotMeta[sl];
+      if (mt.timestep != tstep || mt.N != N) mt.a = 0;   // no basis: no projection
+    }
+    // x_init of a given guess: the learned guess m~ + dt rho net, from the
+    // network's FP32 output, in double-float, or x as it is
+    auto load_guess = [&]() {
+      if (p.gdelta) {
+        const float sg = (float)(p.grho[sysi] * p.gmul);
+        const float* dl = p.gdelta + (size_t)sysi * p.gdelta_ld;
+        each_ext([&](int at, int pp) {
+          put_x(at, pp >= 0 ? dd_add_f(dd_from_double(d.mt[pp]), sg * dl[pp]) : dd{0.f, 0.f});
+        });
+      } else {
+        load_x(d.x);
+      }
+    };
+    if (p.x0_mode != X0_WARM && !judge) {
+      __syncthreads();                           // every read of the lagged field in the slots is done
+      if (p.x0_mode == X0_READ) load_guess();
+      else load_x(nullptr);
+    }
+    if (CS == 1 && p.x0_mode == X0_GALERKIN && p.gram) {
+      // Sec. 3, Phase 2 without the seed-matrix shortcut: G alpha = V_a^T b
+      // with G = V_a^T A_i V_a of this target's own operator, assembled from
+      // the seed basis part G0 and this target's tensor-core part (kp_gram.cu),
+      // x0 = V_a alpha; c = V^T b from the projection GEMM.  G (FP64) takes
+      // the space of the Hessenberg matrix and the vector slots.
+      const int a = mt.a, A = p.gram_a;
+      if (a > 0 && a <= A && a * a <= (m + 1) * m && p.cproj) {
+        const float* g0 = p.gram0 + (size_t)sl * A * A;
+        const float* gi = p.gram + (size_t)sysi * A * A;
+        double* G = reinterpret_cast<double*>(Hr);               // a x a, column-major: G[l + k a] = v_l^T A v_k
+        double* cv = reinterpret_cast<double*>(hball);
+        __syncthreads();                         // the zeroed slots are written
+        for (int e = tid; e < a * a; e += NT) {
+          const int l = e % a, k = e / a;
+          G[e] = (double)g0[l * A + k] + (double)gi[l * A + k];
+        }
+        if (tid < a) cv[tid] = (double)p.cproj[(size_t)sysi * p.cproj_ld + tid];
+        __syncthreads();
+        if (warp == 0) {
+          const bool ok = lu_solve_warp(G, a, cv, lane);
+          for (int i = lane; i < a; i += 32) yf[i] = ok ? (float)cv[i] : 0.f;
+        }
+        __syncthreads();
+        zero_halo();
+        add_basis(U, a, true);
+        proj_flops = (unsigned long long)(2 * a) * (unsigned long long)N;
+      }
+    }
+
+    // ---- refinement.  One loop body serves the judge's two residuals, the
+    // projection's right-hand side and the residual of every outer step, so
+    // that the unrolled stencil exists once (the kernel is sensitive to the
+    // size of its code: instruction fetch was its first stall).
+    enum { kWarm, kGuess, kProject, kSolve };
+    int phase = judge ? kWarm : p.x0_mode == X0_PROJECT && mt.a > 0 ? kProject : kSolve;
+    bool first_norm = true;
+    dd bnorm = {0.f, 0.f}, rnorm = {0.f, 0.f};   // ||b||, ||r||
+    float tolb = 0.f;
+    int steps = 0, status = KP_NOT_CONVERGED, outer = 0;
+    // power of two that brings the diagonal of H_A to [1, 2): the squares of
+    // the least-squares problem then stay inside the FP32 range for any dt
+    const unsigned cde = (__float_as_uint(cdd.hi) >> 23) & 255u;
+    const float hsc = (cde > 0 && cde < 254) ? __uint_as_float((254u - cde) << 23) : 1.f;
+#pragma unroll 1
+    for (;;) {
+      __syncthreads();                           // x complete for the stencil
+      const bool no_x = phase == kProject || (p.x0_mode == X0_ZERO && outer == 0);
+      // w = b - A x in double-float: the hi parts of the terms are added by
+      // TwoSum and all low parts and errors in FP32; w is its FP32 value,
+      // which is all the Krylov process and the norms need (no_x: w = b)
+      {
+        float sb = 0.f;
+        auto mul = [](float ah, float al, float bh, float bl) -> dd {   // a b, unnormalised
+          const float t = __fmul_rn(ah, bh);
+          return {t, fmaf(al, bh, fmaf(ah, bl, fmaf(ah, bh, -t)))};
+        };
+#pragma unroll
+        for (int k = 0; k < EPT; ++k) {
+          const int at = hal + l0 + k * NS;
+          w[k] = 0.f;
+          if (inside(k)) {
+            const dd b = dd_from_double(d.b[base + l0 + k * NS]);
+            sb = fmaf(b.hi, b.hi, sb);
+            w[k] = b.hi;
+            if (!no_x) {
+              const float2 q = ql[l0 + k * NS];
+              const dd x = {xh[at], xl[at]};
+              const dd xE = {nbE(xh, at, k), nbE(xl, at, k)}, xW = {nbW(xh, at, k), nbW(xl, at, k)};
+              const dd xN = {nbN(xh, at, k), nbN(xl, at, k)}, xS = {nbS(xh, at, k), nbS(xl, at, k)};
+              const dd s1 = dd_two_sum(xE.hi, xW.hi), s2 = dd_two_sum(xN.hi, xS.hi), s = dd_two_sum(s1.hi, s2.hi);
+              const float sl_ = ((xE.lo + xW.lo) + (xN.lo + xS.lo)) + ((s1.lo + s2.lo) + s.lo);
+              const dd dx = dd_two_sum(xE.hi, -xW.hi), dy = dd_two_sum(xN.hi, -xS.hi);
+              const float dxl = dx.lo + (xE.lo - xW.lo), dyl = dy.lo + (xN.lo - xS.lo);
+              const dd t1 = mul(cdd.hi, cdd.lo, x.hi, x.lo), t2 = mul(ccd.hi, ccd.lo, s.hi, sl_);
+              const dd t3 = mul(qx[k], q.x, dx.hi, dxl), t4 = mul(qy[k], q.y, dy.hi, dyl);
+              const dd a1 = dd_two_sum(b.hi, -t1.hi), a2 = dd_two_sum(a1.hi, t2.hi);
+              const dd a3 = dd_two_sum(a2.hi, -t3.hi), a4 = dd_two_sum(a3.hi, -t4.hi);
+              w[k] = a4.hi + (((b.lo - t1.lo) + (t2.lo - t3.lo)) + ((a1.lo + a2.lo) + (a3.lo + a4.lo)) - t4.lo);
+            }
+          }
+        }
+        bb = sb;
+      }
+      if (phase == kWarm) {
+        sw = sumsq();
+        __syncthreads();                         // every read of the warm start in the slots is done
+        load_guess();
+        phase = kGuess;
+        continue;
+      }
+      bool project = phase == kProject;
+      if (!project) {
+        push_edges();
+        reduce(first_norm ? 3 : 1, [&](int, int, float (&a)[4]) {
+          a[0] = sumsq();
+          a[1] = bb;
+          a[2] = sw;
+          a[3] = 0.f;
+        });
+        if (phase == kGuess) {
+          // the judge of a given guess (the learned one): its true residual
+          // against the warm start's; a kept guess is projected, the warm
+          // start (the fallback) starts unprojected, as in the warm mode
+          proj_flops = 26ull * (unsigned long long)N;
+          phase = kSolve;
+          if (hb[2].x < hb[0].x || (hb[2].x == hb[0].x && hb[2].y < hb[0].y)) {
+            load_x(d.mt);
+            continue;
+          }
+          project = mt.a > 0;
+        }
+      }
+      if (project) {
+        // Sec. 3, Phase 2 with the seed's FP32 basis: c = V^T w for w = b (the
+        // paper) or the residual of the guess (tensor-core GEMM, or FP32
+        // products and sums here), alpha = H_a^{-1} c, x0 = x_init + V alpha
+        const int a = mt.a;
+        const int nv = mt.lsq ? a + 1 : a;
+        if (phase == kProject && p.cproj) {
+          if (warp == 0) {
+            for (int i = lane; i < nv; i += 32) hb[i] = make_float2(p.cproj[(size_t)sysi * p.cproj_ld + i], 0.f);
+            __syncwarp();
+          }
+        } else {
+          reduce(nv, [&](int i0, int n, float (&s)[4]) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+              s[u] = 0.f;
+              if (i0 + u < n) {
+                const float* ui = U + (size_t)(i0 + u) * p.slot_ld + base + l0;
+#pragma unroll
+                for (int k = 0; k < EPT; ++k)
+                  if (inside(k)) s[u] = fmaf(ui[k * NS], w[k], s[u]);
+              }
+            }
+          });
+        }
+        if (warp == 0) {
+          const double* rot = p.slotRot + (size_t)sl * 3 * p.max_a;
+          solve_projected_dd(hb, a, mt.nrot, p.slotR + (size_t)sl * (p.max_a + 1) * p.max_a, p.max_a + 1, rot,
+                             rot + 2 * p.max_a, yf, lane);
+        }
+        __syncthreads();
+        add_basis(U, a, phase == kProject);
+        proj_flops += (unsigned long long)(2 * nv + 2 * a) * (unsigned long long)N;
+        phase = kSolve;
+        continue;
+      }
+      rnorm = dd_sqrt(as_dd(hb[0]));
+      if (first_norm) {
+        first_norm = false;
+        bnorm = dd_sqrt(as_dd(hb[1]));
+        tolb = __fmul_rd(__double2float_rd(p.tol), bnorm.hi);   // rounded down
+        if (bnorm.hi == 0.f) {
+          load_x(nullptr);
+          rnorm = bnorm;
+          status = KP_OK;
+          break;
+        }
+      }
+      const float beta = rnorm.hi;
+      if (beta <= tolb) { status = KP_OK; break; }
+      if (!isfinite(beta)) { status = KP_BREAKDOWN; break; }
+      if (steps >= p.maxit || outer >= 64) break;
+      const bool first = (outer == 0);
+      // the seed's captured cycle runs to the seed tolerance, so its basis has
+      // the dimension the FP64 method would keep (Sec. 3, Phase 1)
+      const float target = (capture && first) ? tolb : fmaxf(kEta * beta, (float)kInnerFloor * tolb);
+
+      // ---- inner FP32 GMRES(m) on A d = r, from d = 0.  v_n = w scale, kept
+      // as the next Krylov vector (and captured for the seed basis)
+      auto next_vector = [&](int n, float scale) {
+        float* vn = slot(n);
+        const bool keep = capture && first && n <= p.cap_a;
+#pragma unroll
+        for (int k = 0; k < EPT; ++k) {
+          const int l = l0 + k * NS;
+          const float v = w[k] * scale;
+          if (full || inside(k)) vn[hal + l] = v;
+          if (keep && inside(k)) {
+            capV[(size_t)n * p.cap_ld + base + l] = v;
+            if (p.capVb && n < kVbRows)
+              p.capVb[((size_t)cidx * kVbRows + n) * p.capVb_ld + base + l] = __float2bfloat16_rn(v);
+          }
+        }
+        if (CS > 1) {
+          const float* wh = whalo + hbuf * 2 * p.hmax;
+          for (int q = tid; q < 2 * H; q += NT) vn[q < H ? q : SL + q] = wh[q] * scale;
+        } else if (REG && n >= p.S) {
+          for (int q = tid; q < 2 * H; q += NT) vn[q < H ? q : SL + q] = 0.f;
+        }
+      };
+      next_vector(0, 1.f / beta);
+      hbuf ^= 1;
+      int kdone = 0, brk = 0;
+      dd gcur = rnorm;                           // running right-hand side (warp 0)
+#pragma unroll 1
+      for (int j = 0; j < m; ++j) {
+        __syncthreads();                         // v_j complete (own slice and halo)
+        {
+          auto apply = [&](const float* v) {
+#pragma unroll
+            for (int k = 0; k < EPT; ++k) {
+              const int at = hal + l0 + k * NS;
+              float xE = 0.f, xW = 0.f, xN = 0.f, xS = 0.f;
+              if (full || inside(k)) {
+                xE = nbE(v, at, k);
+                xW = nbW(v, at, k);
+                xN = nbN(v, at, k);
+                xS = nbS(v, at, k);
+              }
+              w[k] = -ccf * (xE + xW + xN + xS) + qx[k] * (xE - xW) + qy[k] * (xN - xS);
+            }
+          };
+          if (j < p.S) apply(V + (size_t)j * vld);
+          else apply(Vg + (size_t)(j - p.S) * vld);
+        }
+        push_edges();
+        ++steps;
+        const int nh = j + 1;
+        float2* col = Hr + j * (j + 1) / 2;      // column j of the Hessenberg matrix (warp 0)
+        float ww0 = 0.f;
+        dd hn2 = {0.f, 0.f};                     // ||w||^2 after Gram-Schmidt
+        // Gram-Schmidt: pass 0; pass 1 (re-orthogonalisation) always or, with
+        // reorth, when the first removed more than half of ||w||^2; pass 2
+        // only measures the norm, after a large correction in pass 1
+#pragma unroll 1
+        for (int pass = 0;; ++pass) {
+          reduce(nh + 1, [&](int i0, int n, float (&s)[4]) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+              s[u] = 0.f;
+              const int i = i0 + u;
+              if (i < n - 1) {
+                auto dot = [&](const float* vi) {
+#pragma unroll
+                  for (int k = 0; k < EPT; ++k)
+                    if (full || inside(k)) s[u] = fmaf(vi[k * NS], w[k], s[u]);
+                };
+                if (i < p.S) dot(V + (size_t)i * vld + hal + l0);
+                else dot(Vg + (size_t)(i - p.S) * vld + hal + l0);
+              } else if (i == n - 1) {
+                s[u] = sumsq();
+              }
+            }
+          });
+          const dd ww = as_dd(hb[nh]);
+          if (pass == 2) { hn2 = ww; break; }
+          dd sq = {0.f, 0.f};                    // sum of the squared coefficients
+          for (int i = 0; i < nh; ++i) sq = dd_add(sq, dd_mul(as_dd(hb[i]), as_dd(hb[i])));
+          hn2 = dd_sub(ww, sq);
+          if (warp == 0)
+            for (int i = lane; i < nh; i += 32) col[i] = pass ? as_f2(dd_add(as_dd(col[i]), as_dd(hb[i]))) : hb[i];
+          // w -= sum h_i v_i on the slice and, in the halo buffer, on the halo
+#pragma unroll 1
+          for (int i = 0; i < nh; ++i) {
+            const float hi = hb[i].x;
+            auto sub_ = [&](const float* vi) {
+#pragma unroll
+              for (int k = 0; k < EPT; ++k)
+                if (full || inside(k)) w[k] = fmaf(-hi, vi[k * NS], w[k]);
+            };
+            if (i < p.S) sub_(V + (size_t)i * vld + hal + l0);
+            else sub_(Vg + (size_t)(i - p.S) * vld + hal + l0);
+          }
+          if (CS > 1)
+            for (int q = tid; q < 2 * H; q += NT) {
+              float* wh = whalo + hbuf * 2 * p.hmax + q;
+              float v = *wh;
+              for (int i = 0; i < nh; ++i) v = fmaf(-hb[i].x, slot(i)[q < H ? q : SL + q], v);
+              *wh = v;
+            }
+          if (pass == 0) {
+            ww0 = ww.hi;
+            if (p.reorth != 0 && hn2.hi >= 0.5f * ww0) break;
+          } else if (sq.hi <= 0.25f * ww.hi) {
+            break;
+          }
+        }
+        const dd ihn = hn2.hi > 0.f ? dd_rsqrt(hn2) : dd{0.f, 0.f};
+        brk = !(hn2.hi > 1e-14f * ww0);          // h_{j+1,j} <= 1e-7 ||w_0||: breakdown at FP32 level
+        if (!brk) next_vector(j + 1, ihn.hi);
+        hbuf ^= 1;
+        if (warp == 0) {
+          // Givens step of column j (every lane; lane 0 stores): rotations,
+          // residual estimate, stop flag
+          __syncwarp();
+          const dd hn = dd_mul(hn2, ihn);
+          auto entry = [&](int i) -> dd { return i == j ? dd_add(as_dd(col[i]), cdd) : as_dd(col[i]); };   // H_A = H + cd I
+          if (capture && first && j < p.cap_a && rank == 0)
+            for (int i = lane; i <= j + 1; i += 32) capH[i + j * (p.cap_a + 1)] = dd_to_double(i <= j ? entry(i) : hn);
+          auto scaled = [&](dd v) -> dd { return {v.hi * hsc, v.lo * hsc}; };
+          dd cur = scaled(entry(0));
+          for (int i = 0; i < j; ++i) {
+            const dd c = as_dd(cs[i]), s = as_dd(sn[i]), nx = scaled(entry(i + 1));
+            const dd top = dd_add(dd_mul(c, cur), dd_mul(s, nx));
+            cur = dd_sub(dd_mul(c, nx), dd_mul(s, cur));
+            __syncwarp();
+            if (lane == 0) col[i] = as_f2(top);
+          }
+          const dd hs = scaled(hn);
+          const dd rr = dd_add(dd_mul(cur, cur), dd_mul(hs, hs));
+          const dd ir = dd_rsqrt(rr);
+          const dd c = dd_mul(cur, ir), s = dd_mul(hs, ir);
+          const dd gj = dd_mul(c, gcur);
+          gcur = dd_mul(dd{-s.hi, -s.lo}, gcur);
+          __syncwarp();
+          if (lane == 0) {
+            cs[j] = as_f2(c);
+            sn[j] = as_f2(s);
+            col[j] = as_f2(dd_mul(rr, ir));
+            rinv[j] = as_f2(ir);
+            gv[j] = as_f2(gj);
+            // fixed basis dimension: the seed's captured cycle reaches cap_a
+            // steps before the residual test may end it
+            const bool short_of_a = p.fixed_a && capture && first && j + 1 < p.cap_a;
+            fl[0] = (fabsf(gcur.hi) <= target && !short_of_a) || brk || (steps >= p.maxit) || (j + 1 == m);
+          }
+          __syncwarp();
+        }
+        kdone = j + 1;
+        __syncthreads();
+        if (fl[0]) break;
+      }
+      // y = R^{-1} g: column-oriented back substitution on warp 0 (lane l
+      // owns rows l and l + 32), reciprocal pivots from the Givens steps
+      if (warp == 0) {
+        dd g0 = lane < kdone ? as_dd(gv[lane]) : dd{0.f, 0.f};
+        dd g1 = lane + 32 < kdone ? as_dd(gv[lane + 32]) : dd{0.f, 0.f};
+        for (int i = kdone - 1; i >= 0; --i) {
+          const dd s = i < 32 ? g0 : g1;
+          const dd gi = {__shfl_sync(kFull, s.hi, i & 31), __shfl_sync(kFull, s.lo, i & 31)};
+          const dd yi = dd_mul(gi, as_dd(rinv[i]));
+          if (lane == 0) yf[i] = yi.hi * hsc;    // (R was scaled by hsc)
+          const float2* col = Hr + i * (i + 1) / 2;
+          if (lane < i) g0 = dd_sub(g0, dd_mul(as_dd(col[lane]), yi));
+          if (lane + 32 < i) g1 = dd_sub(g1, dd_mul(as_dd(col[lane + 32]), yi));
+        }
+      }
+      if (tid == 0 && rank == 0 && capture && first) {
+        const int a = kdone < p.cap_a ? kdone : p.cap_a;
+        const int hn = (a < kdone) || !brk;
+        if (p.factor) {
+          SlotMeta sm;
+          double* rot = p.slotRot + (size_t)cidx * 3 * p.max_a;
+          factor_hessenberg(capH, p.cap_a + 1, a, hn, p.slotR + (size_t)cidx * (p.max_a + 1) * p.max_a, rot,
+                            rot + 2 * p.max_a, &sm.lsq, &sm.nrot);
+          sm.a = a;
+          sm.has_next = hn;
+          sm.timestep = tstep;
+          sm.N = N;
+          sm.dense = sm.pad_ = 0;
+          p.slotMeta[cidx] = sm;
+        } else {
+          p.capMeta[sysi].a = a;
+          p.capMeta[sysi].has_next = hn;
+          p.capMeta[sysi].N = N;
+          p.capMeta[sysi].valid = 1;
+        }
+      }
+      __syncthreads();
+      // d = V y in FP32, x += d in double-float; x goes to the first two slots
+      // (each thread has read its own points of every vector by then)
+      each_ext([&](int at, int) {
+        const dd x = as_dd(xs[at]);
+        float dv = 0.f;
+        for (int i = 0; i < kdone; ++i) dv = fmaf(yf[i], slot(i)[at], dv);
+        put_x(at, dd_add_f(x, dv));
+      });
+      ++outer;
+    }
+    if (capture && outer == 0 && tid == 0 && rank == 0) {
+      if (p.factor) {
+        SlotMeta sm;
+        sm.a = 0; sm.has_next = 0; sm.timestep = tstep; sm.N = N; sm.lsq = 0; sm.nrot = 0;
+        sm.dense = sm.pad_ = 0;
+        p.slotMeta[cidx] = sm;
+      } else {
+        p.capMeta[sysi].a = 0;
+        p.capMeta[sysi].has_next = 0;
+        p.capMeta[sysi].N = N;
+        p.capMeta[sysi].valid = 1;
+      }
+    }
+    // (the loop ends with x in the first two slots: every exit follows a
+    // residual of x, or x0 = 0 put there)
+#pragma unroll
+    for (int k = 0; k < EPT; ++k)
+      if (inside(k)) {
+        const int at = hal + l0 + k * NS, pp = base + l0 + k * NS;
+        const dd x = {xh[at], xl[at]};
+        d.x[pp] = dd_to_double(x);
+        if (p.bnext) p.bnext[(size_t)sysi * p.bnext_ld + pp] = __float2bfloat16_rn(x.hi);
+      }
+    if (tid == 0 && rank == 0) {
+      const double rel = bnorm.hi > 0.f ? dd_to_double(rnorm) / dd_to_double(bnorm) : 0.0;
+      if (p.info) {
+        kp_info inf;
+        inf.iters = steps;
+        inf.status = status;
+        inf.rel_res = rel;
+        p.info[sysi] = inf;
+      }
+      if (p.acc) {
+        StepAcc* a = p.acc + tstep;
+        // high-precision flops of the refinement (residuals, x update: in
+        // double-float); FP32 Krylov work is counted separately
+        const unsigned long long fl64 = (unsigned long long)(14 + outer * 13) * (unsigned long long)N;
+        const unsigned long long fl32 = (gmres_flops(steps, m) - 14ull) * (unsigned long long)N;
+        if (p.acc_kind == 0) {
+          atomicAdd(&a->seed_iters, (unsigned long long)steps);
+          atomicAdd(&a->seed_flops, fl64 + fl32);
+        } else {
+          atomicAdd(&a->tgt_iters, (unsigned long long)steps);
+          atomicAdd(&a->tgt_flops, fl64);
+          atomicAdd(&a->tgt_flops32, fl32);
+          atomicMax(&a->tgt_max_iters, (unsigned int)steps);
+          atomicMax(&a->max_res_bits, (unsigned long long)__double_as_longlong(rel));
+          if (proj_flops) atomicAdd(&a->proj_flops, proj_flops);
+        }
+        if (status != KP_OK) atomicAdd(&a->not_converged, 1u);
+      }
+    }
+    __syncthreads();                             // shared memory is reused by the next system
+  }
+  if (CS > 1) cluster.sync();                    // no CTA leaves while others write its memory
+}
+
+template <int EPT, int NT, int CS, int MINB, int SUB, bool REG>
+cudaError_t launch_mx(const GmresParams& p, size_t smem, cudaStream_t st) {
+  auto k = gmres_mixed_kernel<EPT, NT, CS, MINB, SUB, REG>;
+  int dev = 0, optin = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e != cudaSuccess) return e;
+  if (smem > (size_t)optin) return cudaErrorInvalidValue;
+  e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
+  if (e == cudaSuccess && CS > 8) e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(p.nsys * CS));
+  cfg.blockDim = dim3(NT);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = CS;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = CS > 1 ? 1 : 0;
+  e = cudaLaunchKernelEx(&cfg, k, p);
+  if (e != cudaSuccess) return e;
+  return cudaGetLastError();
+}
+
+}  // namespace
+}  // namespace kp

@@ -21,11 +21,22 @@ struct SysDesc {
   double* x;
   int H, W;
   double dt, g2, h;
+  // quotients of the operator constants, taken once on the host and divided
+  // by the system's scale s (set_quotients): 1/(2 h^2), 1/dt and 1/(2h)
+  double kc, kd, ki;
   int slot;   // basis slot (projection) / unused
   int pad_;
   double* score;   // march targets, optional: this system's [2][N] score plane set of timestep 0
   double* emb;     // march targets, optional: this system's [2][N] probability-flow embedding
 };
+
+// The system is solved as (A / s) x = b / s (s: the march's 1/dt, else 1).
+inline void set_quotients(SysDesc* d, double s) {
+  const double h2 = d->h * d->h;
+  d->kc = 1.0 / (2.0 * h2) / s;
+  d->kd = 1.0 / d->dt / s;
+  d->ki = 1.0 / (2.0 * d->h) / s;
+}
 
 // Metadata of one stored seed basis.
 struct SlotMeta {
@@ -111,7 +122,10 @@ struct GmresParams {
   StepAcc* acc;             // per-timestep totals (indexed like g2_sched) or null
   int acc_kind;             // 0 seeds, 1 targets
   // mixed precision (FP32 Krylov vectors)
-  float* spill32;           // [gridDim.x][m + 1 - S][npad] workspace
+  float* spill32;           // [gridDim.x][ws_ld] workspace (mixed_shape)
+  int vld;                  // floats of a vector slot: npad and two halo columns
+  int hmax;                 // longest column of the launch's systems (cluster halos)
+  size_t ws_ld;             // floats of a CTA's workspace
   float* capV32;            // capture target for FP32 bases (slot layout when factor)
   const float* slotV32;     // [max_seeds][max_a + 1][slot_ld] FP32 seed bases
   const float* cproj;       // if set: c = V^T b per target, [nsys][cproj_ld] (tensor-core GEMM)
@@ -150,12 +164,12 @@ struct GmresParams {
   const float* gram;
   int gram_a;
   // learned guess (X0_READ / X0_GUESS_PROJECT in a march): if gdelta is set,
-  // x_init of system s is m~ + (grho[s] / gdiv) gdelta[s * gdelta_ld + p]
-  // (the network's output in units of dt rho, gdiv = T), formed in the solver
+  // x_init of system s is m~ + (grho[s] gmul) gdelta[s * gdelta_ld + p]
+  // (the network's output in units of dt rho, gmul = dt), formed in the solver
   const float* gdelta;
   int gdelta_ld;
   const double* grho;
-  double gdiv;
+  double gmul;
 };
 
 constexpr int kWaitLimit = 1 << 22;   // polls (>= 256 ns apart) before a wait gives up
@@ -382,21 +396,7 @@ __device__ __forceinline__ float warp_reduce8f(float (&a)[8], int lane) {
   return a[0];
 }
 
-template <int NT, typename F>
-__device__ __forceinline__ void block_partials_f32(int nv, F&& partial, double* red) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int i0 = 0; i0 < nv; i0 += 8) {
-    float a[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) a[k] = (i0 + k < nv) ? partial(i0 + k) : 0.f;
-    const float s = warp_reduce8f(a, lane);
-    const int v = ((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1);
-    if ((lane & 3) == 0 && i0 + v < nv) red[warp * kMaxV + i0 + v] = (double)s;
-  }
-  __syncthreads();
-}
-
-// As block_partials_f32, with the per-warp partials kept in FP32 (red32[warp][i]).
+// As block_partials, FP32 values and partials (red32[warp][i]).
 template <int NT, typename F>
 __device__ __forceinline__ void block_partials_f32x(int nv, F&& partial, float* red32) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -554,12 +554,13 @@ cudaError_t launch_gmres_fp64_score(const GmresParams& p, int ept, int nt, int m
 cudaError_t launch_gmres_fp64_picard(const GmresParams& p, int ept, int nt, int minb, size_t smem,
                                      cudaStream_t st);
 size_t gmres_fp64_smem_bytes(int ept, int nt, int S, int m);
-size_t gmres_mixed_smem_bytes(int ept, int nt, int S, int m);
-cudaError_t launch_gmres_mixed(const GmresParams& p, int ept, int nt, size_t smem,
-                               cudaStream_t st);
-size_t gmres_cluster_smem_bytes(int ept, int nt, int S, int m);
-// Cluster of cs CTAs per system (grids above 4096 unknowns, mixed precision).
-cudaError_t launch_gmres_cluster(const GmresParams& p, int ept, int nt, int cs, int minb, size_t smem,
+// Mixed precision: shared memory of a CTA with S vector slots of vld floats
+// (cs CTAs per system, 1 for the one-block solver; hmax: longest column).
+size_t gmres_mixed_smem_bytes(int nt, int cs, int hmax, int vld, int S, int m);
+// reg: every system fills its CTAs and its columns divide a sub-block (the REG kernels).
+cudaError_t launch_gmres_mixed(const GmresParams& p, int ept, int nt, bool reg, size_t smem, cudaStream_t st);
+// Cluster of cs CTAs per system (grids above 4096 unknowns, or on request).
+cudaError_t launch_gmres_cluster(const GmresParams& p, int ept, int nt, int cs, bool reg, size_t smem,
                                  cudaStream_t st);
 // The N <= 1024 instantiation (4 points x 256 threads) on an explicit grid;
 // the kernel strides over systems, block b using Krylov workspace slice b.

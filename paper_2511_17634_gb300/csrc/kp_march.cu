@@ -133,18 +133,12 @@ kp::GmresParams solver_params(kp_march_plan* P, bool seeds, int par, int offset,
   g.tol = seeds ? P->opt.tol_seed : P->opt.tol;
   g.m = seeds ? P->opt.m_seed : P->opt.m;
   g.maxit = seeds && P->opt.maxit_seed > 0 ? P->opt.maxit_seed : P->opt.maxit;
-  g.S = sh.S;
+  kp::set_shape(&g, sh);
   g.reorth = c->opt.reorth;
   g.inner_eta = kp::inner_eta(c->opt);
-  g.npad = sh.ept * sh.nt;
-  size_t spS = 0;
-  if (P->ns && P->shS.S < P->opt.m_seed + 1)
-    spS = (size_t)P->ns * (P->shS.cs ? P->shS.cs : 1) * (P->opt.m_seed + 1 - P->shS.S) * P->shS.ept *
-          P->shS.nt;
-  if (P->mixed)
-    g.spill32 = (sh.S < g.m + 1) ? P->spill32 + (seeds ? 0 : spS + tc.spill_off) : nullptr;
-  else
-    g.spill = (sh.S < g.m + 1) ? P->spill + (seeds ? 0 : spS + tc.spill_off) : nullptr;
+  const size_t spS = P->ns ? (size_t)P->ns * P->shS.ctas() * P->shS.ws : 0;
+  if (P->mixed) g.spill32 = sh.ws ? P->spill32 + (seeds ? 0 : spS + tc.spill_off) : nullptr;
+  else g.spill = sh.ws ? P->spill + (seeds ? 0 : spS + tc.spill_off) : nullptr;
   g.slotV32 = c->slotV32;
   g.info = nullptr;
   g.step = P->step;
@@ -223,11 +217,11 @@ kp::GmresParams solver_params(kp_march_plan* P, bool seeds, int par, int offset,
       g.gram = P->Cg;
       g.gram_a = P->gram_A;
     }
-    if (P->gdelta) {                         // learned guess: x_init = m + (rho / T) net
+    if (P->gdelta) {                         // learned guess: x_init = m + dt rho net
       g.gdelta = P->gdelta;
       g.gdelta_ld = P->groups[0].H * P->groups[0].W;
       g.grho = P->grho;
-      g.gdiv = (double)P->opt.T;
+      g.gmul = 1.0 / P->opt.T;
     }
   }
   return g;
@@ -482,7 +476,7 @@ kp_status kp_march_create(kp_ctx* c, int ngroups, const kp_group* groups, const 
   P->ctx = c;
   P->opt = o;
   P->groups.assign(groups, groups + ngroups);
-  int nmaxS = 0, nmaxT = 0, wminS = 1 << 30, wminT = 1 << 30;
+  int nmaxS = 0, nmaxT = 0, wminS = 1 << 30, wminT = 1 << 30, hmaxS = 0, hmaxT = 0;
   for (int gi = 0; gi < ngroups; ++gi) {
     const kp_group& g = groups[gi];
     const int N = g.H * g.W;
@@ -504,8 +498,8 @@ kp_status kp_march_create(kp_ctx* c, int ngroups, const kp_group* groups, const 
     P->tgt_elems += (size_t)g.ntgt * N;
     P->ns += g.nseed;
     P->nt += g.ntgt;
-    if (g.nseed) { nmaxS = std::max(nmaxS, N); wminS = std::min(wminS, g.W); }
-    if (g.ntgt) { nmaxT = std::max(nmaxT, N); wminT = std::min(wminT, g.W); }
+    if (g.nseed) { nmaxS = std::max(nmaxS, N); wminS = std::min(wminS, g.W); hmaxS = std::max(hmaxS, g.H); }
+    if (g.ntgt) { nmaxT = std::max(nmaxT, N); wminT = std::min(wminT, g.W); hmaxT = std::max(hmaxT, g.H); }
   }
   if (2 * P->ns > c->opt.max_seeds) {
     kp_march_destroy(P);
@@ -514,8 +508,8 @@ kp_status kp_march_create(kp_ctx* c, int ngroups, const kp_group* groups, const 
   }
   P->mixed = c->opt.precision == KP_PREC_MIXED;
   kp_status s = KP_OK;
-  if (P->ns) s = kp::gmres_shape(c, nmaxS, o.m_seed, &P->shS, P->mixed, wminS);
-  if (s == KP_OK && P->nt) s = kp::gmres_shape(c, nmaxT, o.m, &P->shT, P->mixed, wminT);
+  if (P->ns) s = kp::gmres_shape(c, nmaxS, o.m_seed, &P->shS, P->mixed, wminS, hmaxS, ngroups == 1);
+  if (s == KP_OK && P->nt) s = kp::gmres_shape(c, nmaxT, o.m, &P->shT, P->mixed, wminT, hmaxT, ngroups == 1);
   if (s == KP_OK && ((P->shS.cs && ngroups > 1) || (P->shT.cs && ngroups > 1))) {
     kp_march_destroy(P);
     return kp::set_error(c, KP_ERR_UNSUPPORTED, "grids above 4096 unknowns: one grid size per plan");
@@ -669,13 +663,11 @@ kp_status kp_march_create(kp_ctx* c, int ngroups, const kp_group* groups, const 
 
   // one Krylov workspace per branch: seed blocks first, then target blocks
   size_t spS = 0, spT = 0;
-  const int csS = P->shS.cs ? P->shS.cs : 1, csT = P->shT.cs ? P->shT.cs : 1;
-  if (ns && P->shS.S < o.m_seed + 1) spS = (size_t)ns * csS * (o.m_seed + 1 - P->shS.S) * P->shS.ept * P->shS.nt;
+  if (ns) spS = (size_t)ns * P->shS.ctas() * P->shS.ws;
   for (int ci = 0; ci < P->ncls; ++ci) {
     kp_march_plan::TClass& tc = P->cls[ci];
     tc.spill_off = spT;
-    if (tc.count && tc.sh.S < o.m + 1)
-      spT += (size_t)tc.count * csT * (o.m + 1 - tc.sh.S) * tc.sh.ept * tc.sh.nt;
+    spT += (size_t)tc.count * tc.sh.ctas() * tc.sh.ws;
   }
   if (e == cudaSuccess && spS + spT) {
     if (P->mixed) e = dmalloc(&P->spill32, spS + spT);
@@ -733,6 +725,7 @@ kp_status kp_march_create(kp_ctx* c, int ngroups, const kp_group* groups, const 
         const size_t off = P->seed_off[gi] + (size_t)k * N;
         SysDesc d{};
         d.H = g.H; d.W = g.W; d.dt = dt; d.g2 = 0.0; d.h = 1.0 / g.H;
+        kp::set_quotients(&d, (double)o.T);   // scaled as b (b_scale)
         d.mt = P->S[1 - par] + off;
         d.b = d.mt;
         d.x = P->S[par] + off;
@@ -743,6 +736,7 @@ kp_status kp_march_create(kp_ctx* c, int ngroups, const kp_group* groups, const 
         const size_t off = P->tgt_off[gi] + (size_t)k * N;
         SysDesc d{};
         d.H = g.H; d.W = g.W; d.dt = dt; d.g2 = 0.0; d.h = 1.0 / g.H;
+        kp::set_quotients(&d, (double)o.T);   // scaled as b (b_scale)
         d.mt = P->Tt[par] + off;
         d.b = d.mt;
         d.x = P->Tt[1 - par] + off;

@@ -131,6 +131,7 @@ extern "C" kp_status kp_refine_static(int nsys, const kp_op* ops, const double* 
       d.dt = o.dt;
       d.g2 = o.g2;
       d.h = o.h;
+      kp::set_quotients(&d, 1.0);
       chunk.d[k] = d;
     }
     upload_desc_kernel<<<1, 128, 0, stream>>>(chunk, ddesc);
