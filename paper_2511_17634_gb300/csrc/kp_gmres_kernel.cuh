@@ -84,6 +84,7 @@ __global__ void __launch_bounds__(NT, MINB) gmres_fp64_kernel(const GmresParams 
   const int ld = m + 1;
   Smem sm = carve(smem_raw, p.S, npad, NWARPS, m);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int swarp = scalar_warp(NWARPS);
   double* spill = p.spill ? p.spill + (size_t)blockIdx.x * (m + 1 - p.S) * npad : nullptr;
   auto slot = [&](int i) -> double* {
     return i < p.S ? sm.V + (size_t)i * npad : spill + (size_t)(i - p.S) * npad;
@@ -99,7 +100,6 @@ __global__ void __launch_bounds__(NT, MINB) gmres_fp64_kernel(const GmresParams 
       return;
     }
   }
-  const double bsc = p.b_scale;
   const int nitems = p.nsys * nstep;
   int sysi = blockIdx.x, kstep = 0;          // static schedule: a block marches its systems
   for (;;) {
@@ -135,16 +135,15 @@ __global__ void __launch_bounds__(NT, MINB) gmres_fp64_kernel(const GmresParams 
     const int parity_base = slot_set_base(p, tstep);
     const SysDesc d = p.sys_par[0] ? p.sys_par[(tstep + p.sys_shift) & 1][sysi] : p.sys[sysi];
     const int H = d.H, W = d.W, N = H * W;
-    const double hh = d.h;
-    const double g2 = p.step ? p.g2_sched[tstep] : d.g2;
     // the system is solved as (A / s) x = b / s with s = b_scale (the march's
-    // 1/dt): the right-hand side is read as stored and the scale goes on the
-    // four operator constants, once per solve
-    const double osc = bsc != 0.0 ? 1.0 / bsc : 1.0;
-    const double cc = g2 / (2.0 * hh * hh) * osc;
-    const double ee = g2 / (8.0 * hh * hh) * osc;
-    const double cd = (1.0 / d.dt + 2.0 * g2 / (hh * hh)) * osc;
-    const double i2h = osc / (2.0 * hh);
+    // 1/dt): the right-hand side is read as stored and the scale is in the
+    // descriptor's quotients, from which the four operator constants take two
+    // instructions (five FP64 divisions on every warp were 7 % of a solve)
+    const double g2 = p.step ? p.g2_sched[tstep] : d.g2;
+    const double cc = g2 * d.kc;
+    const double ee = 0.25 * cc;
+    const double cd = fma(4.0, cc, d.kd);
+    const double i2h = d.ki;
     bool capture = p.capV != nullptr;          // first solve of the timestep only
     const int cidx = p.factor ? parity_base + sysi : sysi;   // capture record (or seed slot)
     double* capV = capture ? p.capV + (size_t)cidx * (p.cap_a + 1) * p.cap_ld : nullptr;
@@ -166,7 +165,7 @@ __global__ void __launch_bounds__(NT, MINB) gmres_fp64_kernel(const GmresParams 
     // from here; the last timestep of a run writes the score of its own
     // solution in the epilogue
     const bool score_on = SCORE && p.score_stride && d.score;
-    const double s_i2h = SCORE ? 0.5 / hh : 0.0;
+    const double s_i2h = SCORE ? 0.5 / d.h : 0.0;
     double cei = 0.0;                            // the Euler factor times 1/(2h)
     double* sc_in = nullptr;                     // score of the input, timestep tstep - 1
     if (SCORE && score_on) {
@@ -300,8 +299,8 @@ __global__ void __launch_bounds__(NT, MINB) gmres_fp64_kernel(const GmresParams 
           }
           return s;
         }, sm.red);
-        if (warp == 0) {
-          for (int i = lane; i < nv; i += 32) sm.hb[i] = cross_warp<NT>(sm.red, i);
+        if (warp == swarp) {
+          cross_warp_all<NT>(sm.red, nv, lane, [&](int i, double s) { sm.hb[i] = s; });
           __syncwarp();
           const double* R = p.slotR + (size_t)sl * (p.max_a + 1) * p.max_a;
           if (DENSE && mt.dense) {
@@ -372,8 +371,8 @@ __global__ void __launch_bounds__(NT, MINB) gmres_fp64_kernel(const GmresParams 
             }
             return s;
           }, sm.red);
-          if (warp == 0)
-            for (int l = lane; l < a; l += 32) G[l + k * a] = cross_warp<NT>(sm.red, l);
+          if (warp == swarp)
+            cross_warp_all<NT>(sm.red, a, lane, [&](int l, double s) { G[l + k * a] = s; });
           __syncthreads();                       // partials of the next column reuse red
         }
         double bv[EPT];
@@ -389,8 +388,8 @@ __global__ void __launch_bounds__(NT, MINB) gmres_fp64_kernel(const GmresParams 
           }
           return s;
         }, sm.red);
-        if (warp == 0) {
-          for (int l = lane; l < a; l += 32) sm.hb[l] = cross_warp<NT>(sm.red, l);
+        if (warp == swarp) {
+          cross_warp_all<NT>(sm.red, a, lane, [&](int l, double s) { sm.hb[l] = s; });
           __syncwarp();
           const bool ok = lu_solve_warp(G, a, sm.hb, lane);
           if (lane == 0) sm.fl[5] = ok;
@@ -432,8 +431,8 @@ __global__ void __launch_bounds__(NT, MINB) gmres_fp64_kernel(const GmresParams 
       // block sums of nv values fn(i) into sm.hb[0..nv)
       auto reduce = [&](int nv, auto&& fn) {
         block_partials<NT>(nv, fn, sm.red);
-        if (warp == 0)
-          for (int i = lane; i < nv; i += 32) sm.hb[i] = cross_warp<NT>(sm.red, i);
+        if (warp == swarp)
+          cross_warp_all<NT>(sm.red, nv, lane, [&](int i, double s) { sm.hb[i] = s; });
         __syncthreads();
       };
       auto apply_full = [&](const double* v) {   // w = A v
@@ -673,10 +672,7 @@ __global__ void __launch_bounds__(NT, MINB) gmres_fp64_kernel(const GmresParams 
         }
         return s;
       }, sm.red);
-      if (tid == 0) {
-        sm.sc[0] = sqrt(cross_warp<NT>(sm.red, 0));
-        sm.sc[1] = sqrt(cross_warp<NT>(sm.red, 1));
-      }
+      if (warp == swarp) cross_warp_all<NT>(sm.red, 2, lane, [&](int i, double s) { sm.sc[i] = sqrt(s); });
       __syncthreads();
       bnorm = sm.sc[0];
       beta = sm.sc[1];
@@ -707,7 +703,7 @@ __global__ void __launch_bounds__(NT, MINB) gmres_fp64_kernel(const GmresParams 
         // Givens update of Hessenberg column j once h_{j+1,j}^2 = hn2 is known
         // (one lane): rotations, residual estimate, convergence flags.
         auto givens_step = [&](int j, double hn2) {
-          const double ihn = hn2 > 0.0 ? rsqrt(hn2) : 0.0;
+          const double ihn = hn2 > 0.0 ? rsqrt_fast(hn2) : 0.0;
           const double hn = hn2 * ihn;
           const int b = !(hn2 > 1e-28 * sm.sc[2]);  // h_{j+1,j} <= 1e-14 ||A v_j||
           sm.Hr[j + j * ld] += cd;                 // H_A = H_{A - cd I} + cd I
@@ -722,7 +718,7 @@ __global__ void __launch_bounds__(NT, MINB) gmres_fp64_kernel(const GmresParams 
           }
           const double a0 = sm.Hr[j + j * ld];
           const double rr = a0 * a0 + hn2;
-          const double ir = rsqrt(rr);
+          const double ir = rsqrt_fast(rr);
           const double c = a0 * ir, s = hn * ir;
           sm.cs[j] = c;
           sm.sn[j] = s;
@@ -758,14 +754,13 @@ __global__ void __launch_bounds__(NT, MINB) gmres_fp64_kernel(const GmresParams 
           };
           // CGS pass 1: h_i = <v_i, w> and ||w||^2 in one batched reduction
           block_partials<NT>(nh + 1, dots, sm.red);
-          if (warp == 0) {
+          if (warp == swarp) {
             double sq = 0.0;
-            for (int i = lane; i <= nh; i += 32) {
-              const double s = cross_warp<NT>(sm.red, i);
+            cross_warp_all<NT>(sm.red, nh + 1, lane, [&](int i, double s) {
               sm.hb[i] = s;
               if (i < nh) { sm.Hr[i + j * ld] = s; sq += s * s; }
-            }
-            sq = warp_sum(sq);
+            });
+            sq = value_lanes_sum<NT>(sq, nh);
             if (lane == 0) {
               const double ww0 = sm.hb[nh];
               sm.sc[2] = ww0;
@@ -795,14 +790,13 @@ __global__ void __launch_bounds__(NT, MINB) gmres_fp64_kernel(const GmresParams 
             // ||w_2||^2 = ||w_1||^2 - ||h_2||^2 (h_2 = O(eps) after pass 1), checked
             const int big = sm.fl[4];
             block_partials<NT>(big ? nh + 1 : nh, dots, sm.red);
-            if (warp == 0) {
+            if (warp == swarp) {
               double sq = 0.0;
-              for (int i = lane; i < (big ? nh + 1 : nh); i += 32) {
-                const double s = cross_warp<NT>(sm.red, i);
+              cross_warp_all<NT>(sm.red, big ? nh + 1 : nh, lane, [&](int i, double s) {
                 sm.hb[i] = s;
                 if (i < nh) { sm.Hr[i + j * ld] += s; sq += s * s; }
-              }
-              sq = warp_sum(sq);
+              });
+              sq = value_lanes_sum<NT>(sq, nh);
               if (lane == 0) {
                 const double ww1 = big ? sm.hb[nh] : sm.sc[4];
                 const int exact = sq > 0.25 * ww1;     // large correction: recompute the norm
@@ -824,7 +818,7 @@ __global__ void __launch_bounds__(NT, MINB) gmres_fp64_kernel(const GmresParams 
                 for (int k = 0; k < EPT; ++k) s += w[k] * w[k];
                 return s;
               }, sm.red);
-              if (tid == 0) givens_step(j, cross_warp<NT>(sm.red, 0));
+              if (tid == swarp * 32) givens_step(j, cross_warp<NT>(sm.red, 0));
               __syncthreads();
             }
           }
@@ -845,7 +839,7 @@ __global__ void __launch_bounds__(NT, MINB) gmres_fp64_kernel(const GmresParams 
         }
         // y = R^{-1} g: column-oriented back substitution on warp 0 (lane l owns
         // rows l and l+32), reciprocal pivots stored by the Givens step
-        if (warp == 0) {
+        if (warp == swarp) {
           double g0 = (lane < kdone) ? sm.g[lane] : 0.0;
           double g1 = (lane + 32 < kdone) ? sm.g[lane + 32] : 0.0;
           for (int i = kdone - 1; i >= 0; --i) {
@@ -856,29 +850,33 @@ __global__ void __launch_bounds__(NT, MINB) gmres_fp64_kernel(const GmresParams 
             if (lane + 32 < i) g1 = fma(-sm.Hr[(lane + 32) + i * ld], yi, g1);
           }
         }
-        if (tid == 0) {
-          if (capture && cycle == 0) {
-            const int a = kdone < p.cap_a ? kdone : p.cap_a;
-            const int hn = (a < kdone) || !brk;
+        if (warp == swarp && capture && cycle == 0) {
+          const int a = kdone < p.cap_a ? kdone : p.cap_a;
+          const int hn = (a < kdone) || !brk;
+          double* rot = p.capRot + (size_t)cidx * 3 * p.cap_a;
+          int lsq, nrot;
+          store_factors(a, hn, capH, p.cap_a + 1, [&](int i, int j) { return sm.Hr[i + j * ld]; },
+                        [&](int j) { return sm.cs[j]; }, [&](int j) { return sm.sn[j]; },
+                        [&](int j) { return sm.rinv[j]; }, p.capR + (size_t)cidx * (p.cap_a + 1) * p.cap_a,
+                        p.cap_a + 1, rot, rot + 2 * p.cap_a, &lsq, &nrot, lane);
+          if (lane == 0) {
             if (p.factor) {
-              // fused basis store: factor H_a of the slot just written
               SlotMeta mt;
-              const int sl = cidx;
-              double* rot = p.slotRot + (size_t)sl * 3 * p.max_a;
-              factor_hessenberg(capH, p.cap_a + 1, a, hn,
-                                p.slotR + (size_t)sl * (p.max_a + 1) * p.max_a, rot,
-                                rot + 2 * p.max_a, &mt.lsq, &mt.nrot);
               mt.a = a;
               mt.has_next = hn;
               mt.timestep = tstep;
               mt.N = N;
+              mt.lsq = lsq;
+              mt.nrot = nrot;
               mt.dense = mt.pad_ = 0;
-              p.slotMeta[sl] = mt;
+              p.slotMeta[cidx] = mt;
             } else {
               p.capMeta[sysi].a = a;
               p.capMeta[sysi].has_next = hn;
               p.capMeta[sysi].N = N;
               p.capMeta[sysi].valid = 1;
+              p.capMeta[sysi].lsq = lsq;
+              p.capMeta[sysi].nrot = nrot;
             }
           }
         }
@@ -897,7 +895,7 @@ __global__ void __launch_bounds__(NT, MINB) gmres_fp64_kernel(const GmresParams 
           for (int k = 0; k < EPT; ++k) s += w[k] * w[k];
           return s;
         }, sm.red);
-        if (tid == 0) sm.sc[1] = sqrt(cross_warp<NT>(sm.red, 0));
+        if (warp == swarp) cross_warp_all<NT>(sm.red, 1, lane, [&](int, double s) { sm.sc[1] = sqrt(s); });
         __syncthreads();
         beta = sm.sc[1];
         ++cycle;
@@ -918,6 +916,7 @@ __global__ void __launch_bounds__(NT, MINB) gmres_fp64_kernel(const GmresParams 
           p.capMeta[sysi].has_next = 0;
           p.capMeta[sysi].N = N;
           p.capMeta[sysi].valid = 1;
+          p.capMeta[sysi].lsq = p.capMeta[sysi].nrot = 0;
         }
       }
     }                                          // Picard iterations
@@ -942,7 +941,7 @@ __global__ void __launch_bounds__(NT, MINB) gmres_fp64_kernel(const GmresParams 
         }
       }
     }
-    if (tid == 0) {
+    if (tid == swarp * 32) {
       const double rel = bnorm > 0.0 ? beta / bnorm : 0.0;
       if (p.info) {
         kp_info inf;

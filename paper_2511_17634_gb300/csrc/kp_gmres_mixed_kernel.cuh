@@ -760,25 +760,36 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
           if (lane + 32 < i) g1 = dd_sub(g1, dd_mul(as_dd(col[lane + 32]), yi));
         }
       }
-      if (tid == 0 && rank == 0 && capture && first) {
+      if (warp == 0 && rank == 0 && capture && first) {
         const int a = kdone < p.cap_a ? kdone : p.cap_a;
         const int hn = (a < kdone) || !brk;
-        if (p.factor) {
-          SlotMeta sm;
-          double* rot = p.slotRot + (size_t)cidx * 3 * p.max_a;
-          factor_hessenberg(capH, p.cap_a + 1, a, hn, p.slotR + (size_t)cidx * (p.max_a + 1) * p.max_a, rot,
-                            rot + 2 * p.max_a, &sm.lsq, &sm.nrot);
-          sm.a = a;
-          sm.has_next = hn;
-          sm.timestep = tstep;
-          sm.N = N;
-          sm.dense = sm.pad_ = 0;
-          p.slotMeta[cidx] = sm;
-        } else {
-          p.capMeta[sysi].a = a;
-          p.capMeta[sysi].has_next = hn;
-          p.capMeta[sysi].N = N;
-          p.capMeta[sysi].valid = 1;
+        double* rot = p.capRot + (size_t)cidx * 3 * p.cap_a;
+        const double us = 1.0 / (double)hsc;     // (a power of two: exact)
+        int lsq, nrot;
+        store_factors(a, hn, capH, p.cap_a + 1, [&](int i, int j) { return dd_to_double(as_dd(Hr[j * (j + 1) / 2 + i])) * us; },
+                      [&](int j) { return dd_to_double(as_dd(cs[j])); }, [&](int j) { return dd_to_double(as_dd(sn[j])); },
+                      [&](int j) { return dd_to_double(as_dd(rinv[j])) * (double)hsc; },
+                      p.capR + (size_t)cidx * (p.cap_a + 1) * p.cap_a, p.cap_a + 1, rot, rot + 2 * p.cap_a, &lsq, &nrot,
+                      lane);
+        if (lane == 0) {
+          if (p.factor) {
+            SlotMeta sm;
+            sm.a = a;
+            sm.has_next = hn;
+            sm.timestep = tstep;
+            sm.N = N;
+            sm.lsq = lsq;
+            sm.nrot = nrot;
+            sm.dense = sm.pad_ = 0;
+            p.slotMeta[cidx] = sm;
+          } else {
+            p.capMeta[sysi].a = a;
+            p.capMeta[sysi].has_next = hn;
+            p.capMeta[sysi].N = N;
+            p.capMeta[sysi].valid = 1;
+            p.capMeta[sysi].lsq = lsq;
+            p.capMeta[sysi].nrot = nrot;
+          }
         }
       }
       __syncthreads();
@@ -803,6 +814,7 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
         p.capMeta[sysi].has_next = 0;
         p.capMeta[sysi].N = N;
         p.capMeta[sysi].valid = 1;
+        p.capMeta[sysi].lsq = p.capMeta[sysi].nrot = 0;
       }
     }
     // (the loop ends with x in the first two slots: every exit follows a

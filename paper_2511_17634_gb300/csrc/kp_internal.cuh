@@ -70,6 +70,7 @@ struct CapMeta {
   int has_next;
   int N;
   int valid;
+  int lsq, nrot;   // as in SlotMeta
 };
 
 constexpr int kMaxM = 64;            // largest restart length / basis size
@@ -98,6 +99,9 @@ struct GmresParams {
   double* capM;     // seed cycling: [slot][cap_ld] the lagged field m~ of the
                     // solve that filled the slot (its operator), or null
   CapMeta* capMeta; // [nsys]
+  double* capR;     // [nsys][(cap_a + 1) * cap_a] projection factors of the first
+  double* capRot;   // [nsys][3 * cap_a]           cycle (store_factors); the slots'
+                    // own when factor
   int cap_a;
   int cap_ld;
   int fixed_a;      // 1: the capture cycle takes min(cap_a, m) steps before the
@@ -256,26 +260,26 @@ struct ProjParams {
   const float* slotV32;    // mixed precision: FP32 bases instead of slotV
 };
 
-struct FactorParams {
+// kp_store_basis: the captured basis and factors of system `sys` into a slot.
+struct StoreParams {
   const double* capV;
+  const float* capV32;     // mixed precision: FP32 capture and slot bases (else null)
   const double* capH;
+  const double* capR;
+  const double* capRot;
   const CapMeta* capMeta;
   int sys;
-  int cap_a;
   int cap_ld;
   double* slotV;
+  float* slotV32;
   SlotMeta* meta;
+  double* slotH;           // [max_seeds][(max_a + 1) * max_a] unrotated Hbar copy
   double* slotR;
   double* slotRot;
-  double* slotH;           // [max_seeds][(max_a + 1) * max_a] unrotated Hbar copy
-  int seed_id;             // block b stores capture sys + b into slot seed_id + b
+  int seed_id;
   int timestep;
-  int max_a;
+  int max_a;               // also the capture's
   int ld;
-  int count;               // number of (sys, slot) pairs, one block each
-  const int* step;         // if non-null, the timestep is *step
-  const float* capV32;     // mixed precision: FP32 capture and slot bases (else null)
-  float* slotV32;
 };
 
 // ---- block reductions shared by the kernels ----
@@ -429,13 +433,78 @@ __device__ __forceinline__ void cross_warp_f32(const float* red32, int nv, doubl
   }
 }
 
-// Cross-warp sum of value i (called by warp 0 lanes).
+// Cross-warp sum of value i (called by the lanes of one warp).
 template <int NT>
 __device__ __forceinline__ double cross_warp(const double* red, int i) {
   double s = 0.0;
 #pragma unroll
   for (int w = 0; w < NT / 32; ++w) s += red[w * kMaxV + i];
   return s;
+}
+
+// The same sums of values 0..nv-1 by a whole warp: fn(i, sum) on one lane for
+// every i.  An FP64 instruction holds its scheduler's pipe for 64 cycles
+// however many lanes take part, so from 8 warps on four lanes share a value
+// (a quarter of the adds each, then two butterflies: 5 adds instead of 15
+// for 16 warps).
+template <int NT, typename F>
+__device__ __forceinline__ void cross_warp_all(const double* red, int nv, int lane, F&& fn) {
+  constexpr int NW = NT / 32;
+  if (NW < 8) {
+    for (int i = lane; i < nv; i += 32) fn(i, cross_warp<NT>(red, i));
+  } else {
+    for (int i0 = 0; i0 < nv; i0 += 8) {
+      const int i = i0 + (lane >> 2);
+      double s = 0.0;
+      if (i < nv) {
+#pragma unroll
+        for (int w = 0; w < NW / 4; ++w) s += red[(4 * w + (lane & 3)) * kMaxV + i];
+      }
+      s += __shfl_xor_sync(kFull, s, 2);
+      s += __shfl_xor_sync(kFull, s, 1);
+      if ((lane & 3) == 0 && i < nv) fn(i, s);
+    }
+  }
+}
+
+// Sum of one number for each of nv >= 1 values, held by the lanes on which
+// cross_warp_all handed them out (zero elsewhere); valid on lane 0.
+template <int NT>
+__device__ __forceinline__ double value_lanes_sum(double v, int nv) {
+  constexpr int step = NT / 32 < 8 ? 1 : 4;                // lanes per value
+  const int n = nv * step;
+  for (int o = n > 16 ? 16 : n > 8 ? 8 : n > 4 ? 4 : n > 2 ? 2 : 1; o >= step; o >>= 1)
+    v += __shfl_xor_sync(kFull, v, o);
+  return v;
+}
+
+// 1 / sqrt(x), x > 0: the FP32 estimate of x scaled to [1, 4) (by an even
+// power of two, exact) and one third-order correction, y (1 + e/2 + 3 e^2/8)
+// with e = 1 - x y^2 (Taylor's series of (1 - e)^(-1/2); e is about 1e-7, so
+// what is left out is below 2^-69).  Seven FP64 instructions; the runtime
+// function takes about twice as many, on the one lane that everybody waits for.
+__device__ __forceinline__ double rsqrt_fast(double x) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(x);
+  const int e = (int)(u >> 52) - 1023;
+  if (e < -1000 || e > 1000) return rsqrt(x);              // tiny, Inf, NaN
+  const int h = e >> 1;                                    // x = 2^(2h) s, 1 <= s < 4
+  const double sx = __longlong_as_double((long long)(u - ((unsigned long long)(long long)(2 * h) << 52)));
+  // (FP64 <-> FP32 by the bit patterns: the conversions run at FP64 speed)
+  const float f = __uint_as_float((unsigned int)(__double_as_longlong(sx) >> 29) - (896u << 23));
+  const unsigned int q = __float_as_uint(rsqrtf(f));
+  const double y = __longlong_as_double(((long long)(q >> 23) + 896ll) << 52 | (long long)(q & 0x7FFFFFu) << 29);
+  const double r = fma(-sx, y * y, 1.0);
+  const double z = fma(y * r, fma(0.375, r, 0.5), y);
+  return __longlong_as_double(__double_as_longlong(z) - ((long long)h << 52));
+}
+
+// Which warp of a block does its serial FP64 work (cross-warp sums, Givens
+// steps).  Blocks that share an SM take different warps, and so different
+// schedulers: with warp 0 everywhere one scheduler's FP64 pipe had all of it.
+__device__ __forceinline__ int scalar_warp(int nwarps) {
+  unsigned n;
+  asm("mov.u32 %0, %%nsmid;" : "=r"(n));
+  return (int)((blockIdx.x / n) % (unsigned)nwarps);
 }
 
 // FP64 flops per unknown of GMRES(m) with CGS2 as implemented here, for k
@@ -450,54 +519,53 @@ __host__ __device__ __forceinline__ unsigned long long gmres_flops(int k, int m)
   return f;
 }
 
-__device__ __forceinline__ void givens_rot(double a, double b, double& c, double& s) {
-  if (b == 0.0) { c = 1.0; s = 0.0; return; }
-  const double r = hypot(a, b);
-  const double ir = 1.0 / r;
-  c = a * ir;
-  s = b * ir;
-}
-
-// Givens QR of a seed's Hessenberg matrix for the projection of Sec. 3
-// (one thread).  Hb: unrotated (a+1) x a, column-major, leading dim ld, also
-// the leading dim of R.  First tries H_a (a-1 rotations); if a pivot is below
-// 1e-14 max|H_a| and v_{a+1} exists, factors Hbar instead (a rotations,
-// least squares).  Writes R, rot (c, s pairs), rinv (reciprocal pivots, 0 for
-// a zero pivot) and returns lsq / nrot.
-__device__ __forceinline__ void factor_hessenberg(const double* Hb, int ld, int a, int has_next,
-                                                  double* R, double* rot, double* rinv,
-                                                  int* lsq_out, int* nrot_out) {
-  double hmax = 0.0;
-  for (int j = 0; j < a; ++j)
-    for (int i = 0; i < a && i <= j + 1; ++i) hmax = fmax(hmax, fabs(Hb[i + j * ld]));
-  int lsq = 0, nrot = 0;
-  for (int pass = 0; pass < 2; ++pass) {
-    lsq = pass;
-    const int nr = lsq ? a + 1 : a;
-    for (int j = 0; j < a; ++j)
-      for (int i = 0; i <= a; ++i) R[i + j * ld] = (i < nr && i <= j + 1) ? Hb[i + j * ld] : 0.0;
-    nrot = 0;
-    for (int j = 0; j < a && j + 1 < nr; ++j) {
-      double c, s;
-      givens_rot(R[j + j * ld], R[(j + 1) + j * ld], c, s);
-      for (int l = j; l < a; ++l) {
-        const double t1 = R[j + l * ld], t2 = R[(j + 1) + l * ld];
-        R[j + l * ld] = c * t1 + s * t2;
-        R[(j + 1) + l * ld] = -s * t1 + c * t2;
-      }
-      rot[2 * j] = c;
-      rot[2 * j + 1] = s;
-      ++nrot;
+// The projection factors of Sec. 3 from a captured GMRES cycle, by one warp:
+// the Givens QR of H_a is the cycle's own (R: rotated columns, c, s: rotations,
+// rinv: reciprocal pivots, read by index), except that H_a's last column is not
+// rotated against row a + 1.  If a pivot of that R is below 1e-14 max|H_a| and
+// v_{a+1} exists, the least-squares factor of Hbar (a rotations) is kept
+// instead.  Hb: unrotated Hbar, column-major, leading dim hld.  Writes R (a + 1
+// rows, leading dim ld), rot (c, s pairs) and ri (0 for a zero pivot).
+// (Refactoring Hbar on one thread took 15-60 us of every seed solve.)
+template <typename FR, typename FC, typename FS, typename FI>
+__device__ __forceinline__ void store_factors(int a, int has_next, const double* Hb, int hld, FR&& getR, FC&& getC,
+                                              FS&& getS, FI&& getI, double* R, int ld, double* rot, double* ri,
+                                              int* lsq_out, int* nrot_out, int lane) {
+  __syncwarp();
+  unsigned long long hm = 0;                               // max|H_a| as bits
+  for (int e = lane; e < a * a; e += 32) {
+    const int i = e % a, j = e / a;
+    if (i <= j + 1) {
+      const unsigned long long v = (unsigned long long)__double_as_longlong(Hb[i + j * hld]) & 0x7FFFFFFFFFFFFFFFull;
+      hm = v > hm ? v : hm;
     }
-    int singular = 0;
-    for (int j = 0; j < a; ++j)
-      if (!(fabs(R[j + j * ld]) > 1e-14 * hmax)) singular = 1;
-    if (singular && !lsq && has_next) continue;
-    break;
   }
-  for (int j = 0; j < a; ++j) rinv[j] = (R[j + j * ld] != 0.0) ? 1.0 / R[j + j * ld] : 0.0;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long v = __shfl_xor_sync(kFull, hm, o);
+    hm = v > hm ? v : hm;
+  }
+  const double least = 1e-14 * __longlong_as_double((long long)hm);
+  const double last = a > 0 ? getC(a - 1) * getR(a - 1, a - 1) : 0.0;
+  int small = 0;
+  for (int j = lane; j < a; j += 32) small |= !(fabs(j == a - 1 ? last : getR(j, j)) > least);
+  const int lsq = __any_sync(kFull, small) && has_next;
+  const int nrot = lsq ? a : (a > 0 ? a - 1 : 0);
+  for (int e = lane; e < a * (a + 1); e += 32) {
+    const int i = e % (a + 1), j = e / (a + 1);
+    R[i + j * ld] = i > j ? 0.0 : (j == a - 1 && i == j && !lsq) ? last : getR(i, j);
+  }
+  for (int j = lane; j < a; j += 32) {
+    if (j < nrot) {
+      rot[2 * j] = getC(j);
+      rot[2 * j + 1] = getS(j);
+    }
+    const double d = (j == a - 1 && !lsq) ? last : getR(j, j);
+    ri[j] = d == 0.0 ? 0.0 : (j == a - 1 && !lsq) ? 1.0 / last : getI(j);
+  }
   *lsq_out = lsq;
   *nrot_out = nrot;
+  __syncwarp();
 }
 
 // alpha from c in place, c <- R^{-1} (G c), by one warp: the rotations on lane
@@ -566,8 +634,11 @@ cudaError_t launch_gmres_cluster(const GmresParams& p, int ept, int nt, int cs, 
 // the kernel strides over systems, block b using Krylov workspace slice b.
 cudaError_t launch_gmres_fp64_1k_grid(const GmresParams& p, size_t smem, int grid,
                                       cudaStream_t st);
-cudaError_t launch_apply(const SysDesc* sys, int nsys, int mode, cudaStream_t st);
-cudaError_t launch_factor(const FactorParams& p, cudaStream_t st);
+// y = A x (b: x, x: y), b = m^{n-1}/dt - Div_h f (b: m^{n-1}, x: b) or
+// r = b - A x (b: x, score: b, x: r) of every system; nmax: largest N
+enum { kApply = 0, kRhs = 1, kResidual = 2 };
+cudaError_t launch_apply(const SysDesc* sys, int nsys, int nmax, int mode, cudaStream_t st);
+cudaError_t launch_store(const StoreParams& p, cudaStream_t st);
 cudaError_t launch_project_fp64(const ProjParams& p, int ept, int nt, cudaStream_t st);
 cudaError_t launch_advance(int* step, cudaStream_t st, int by = 1, int* zero = nullptr, int nzero = 1);
 

@@ -193,6 +193,8 @@ kp::GmresParams solver_params(kp_march_plan* P, bool seeds, int par, int offset,
       g.capV = c->slotV;
     }
     g.capH = c->slotH;
+    g.capR = c->slotR;
+    g.capRot = c->slotRot;
     g.cap_a = c->opt.max_a;
     g.cap_ld = c->opt.max_n;
     g.fixed_a = c->opt.fixed_a;

@@ -10,52 +10,45 @@
 namespace kp {
 namespace {
 
-// Copies the captured basis of system p.sys into slot p.seed_id and factors
-// its Hessenberg matrix.  One block; thread 0 does the (tiny) factorisation.
-__global__ void factor_kernel(FactorParams p) {
-  p.sys += blockIdx.x;
-  p.seed_id += blockIdx.x;
-  if (p.step) p.timestep = *p.step;
+// The captured basis and factors of system p.sys into slot p.seed_id: block k
+// copies vector k, the last block the small matrices and the metadata.  (One
+// block with the factorisation on one thread took 28 us at 32x32 with six
+// vectors, 3 us now: a caller stores seed after seed.)
+__global__ void __launch_bounds__(256) store_kernel(const StoreParams p) {
   const CapMeta cm = p.capMeta[p.sys];
   const int a = cm.valid ? cm.a : 0;
   const int hn = cm.valid ? cm.has_next : 0;
-  const int N = cm.N;
-  const double* cv = p.capV + (size_t)p.sys * (p.cap_a + 1) * p.cap_ld;
-  double* sv = p.slotV + (size_t)p.seed_id * (p.max_a + 1) * p.ld;
-  const int nvec = a + hn;
-  if (p.capV32) {
-    const float* cv32 = p.capV32 + (size_t)p.sys * (p.cap_a + 1) * p.cap_ld;
-    float* sv32 = p.slotV32 + (size_t)p.seed_id * (p.max_a + 1) * p.ld;
-    for (int idx = threadIdx.x; idx < nvec * N; idx += blockDim.x) {
-      const int k = idx / N, q = idx - k * N;
-      sv32[(size_t)k * p.ld + q] = cv32[(size_t)k * p.cap_ld + q];
+  const int N = cm.N, k = blockIdx.x;
+  if (k <= p.max_a) {
+    if (k >= a + hn) return;
+    const size_t from = ((size_t)p.sys * (p.max_a + 1) + k) * p.cap_ld, to = ((size_t)p.seed_id * (p.max_a + 1) + k) * p.ld;
+    for (int q = threadIdx.x; q < N; q += blockDim.x) {
+      if (p.capV32) p.slotV32[to + q] = p.capV32[from + q];
+      else p.slotV[to + q] = p.capV[from + q];
     }
-  } else {
-    for (int idx = threadIdx.x; idx < nvec * N; idx += blockDim.x) {
-      const int k = idx / N, q = idx - k * N;
-      sv[(size_t)k * p.ld + q] = cv[(size_t)k * p.cap_ld + q];
-    }
+    return;
   }
-  if (threadIdx.x != 0) return;
-  const int cld = p.cap_a + 1;
-  const int sld = p.max_a + 1;
-  const double* ch = p.capH + (size_t)p.sys * cld * p.cap_a;
-  double* sh = p.slotH + (size_t)p.seed_id * sld * p.max_a;
-  double* R = p.slotR + (size_t)p.seed_id * sld * p.max_a;   // (a+1) x a, ld max_a+1
-  double* rot = p.slotRot + (size_t)p.seed_id * 3 * p.max_a;
-  for (int j = 0; j < a; ++j)
-    for (int i = 0; i <= a; ++i) sh[i + j * sld] = (i <= j + 1) ? ch[i + j * cld] : 0.0;
-  int lsq = 0, nrot = 0;
-  factor_hessenberg(sh, sld, a, hn, R, rot, rot + 2 * p.max_a, &lsq, &nrot);
-  SlotMeta mt;
-  mt.a = a;
-  mt.has_next = hn;
-  mt.timestep = p.timestep;
-  mt.N = N;
-  mt.lsq = lsq;
-  mt.nrot = nrot;
-  mt.dense = mt.pad_ = 0;
-  p.meta[p.seed_id] = mt;
+  const int ld = p.max_a + 1;
+  const size_t cm0 = (size_t)p.sys * ld * p.max_a, sm0 = (size_t)p.seed_id * ld * p.max_a;
+  for (int e = threadIdx.x; e < a * (a + 1); e += blockDim.x) {
+    const int i = e % (a + 1), j = e / (a + 1);
+    p.slotH[sm0 + i + j * ld] = i <= j + 1 ? p.capH[cm0 + i + j * ld] : 0.0;
+    p.slotR[sm0 + i + j * ld] = p.capR[cm0 + i + j * ld];
+  }
+  const size_t cr = (size_t)p.sys * 3 * p.max_a, sr = (size_t)p.seed_id * 3 * p.max_a;
+  for (int e = threadIdx.x; e < 2 * cm.nrot; e += blockDim.x) p.slotRot[sr + e] = p.capRot[cr + e];
+  for (int e = threadIdx.x; e < a; e += blockDim.x) p.slotRot[sr + 2 * p.max_a + e] = p.capRot[cr + 2 * p.max_a + e];
+  if (threadIdx.x == 0) {
+    SlotMeta mt;
+    mt.a = a;
+    mt.has_next = hn;
+    mt.timestep = p.timestep;
+    mt.N = N;
+    mt.lsq = a ? cm.lsq : 0;
+    mt.nrot = a ? cm.nrot : 0;
+    mt.dense = mt.pad_ = 0;
+    p.meta[p.seed_id] = mt;
+  }
 }
 
 template <int EPT, int NT>
@@ -156,8 +149,8 @@ cudaError_t launch_widen(const float* src, size_t src_ld, double* dst, size_t ds
   return cudaGetLastError();
 }
 
-cudaError_t launch_factor(const FactorParams& p, cudaStream_t st) {
-  factor_kernel<<<p.count > 0 ? p.count : 1, 256, 0, st>>>(p);
+cudaError_t launch_store(const StoreParams& p, cudaStream_t st) {
+  store_kernel<<<p.max_a + 2, 256, 0, st>>>(p);
   return cudaGetLastError();
 }
 
