@@ -584,8 +584,6 @@ kp_status kp_project_gemm_bf16(kp_ctx* c, int nt, int nv, int K, const void* B, 
     tiles[t].count = std::min(128, nt - 128 * t);
     tiles[t].nv = nv;
     tiles[t].ccol0 = 0;
-    tiles[t].kc0 = tiles[t].kc1 = 0;
-    tiles[t].atomic = 0;
   }
   cudaError_t e = grow(&c->d_tiles, &c->d_tiles_bytes, tiles.size() * sizeof(kp::ProjTile));
   if (e == cudaSuccess && !c->d_err) {

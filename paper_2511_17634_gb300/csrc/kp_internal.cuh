@@ -602,8 +602,6 @@ __device__ __forceinline__ void solve_projected_warp(double* c, int a, int nrot,
 struct ProjTile {
   int row0, vrow0, crow0, count, nv;
   int ccol0;        // first C column of this tile
-  int kc0, kc1;     // K range in 64-element chunks; kc1 == 0: the whole K
-  int atomic;       // accumulate into C with atomicAdd (split K) instead of storing
 };
 
 // Launchers (defined in the .cu files; return a cudaError_t of the launch).
@@ -685,6 +683,12 @@ cudaError_t launch_planes_to_padded(const float* X, int B, int C, int chunks, co
 cudaError_t launch_conv3x3(const __nv_bfloat16* in, int B, int cic, const __nv_bfloat16* wf, const float* bias,
                            int cout, int nout, const ConvGeom& g, __nv_bfloat16* out_pad, float* out_f32,
                            int* err, int sms, cudaStream_t st);
+// Training convolutions (kp_conv_train.cu), FP32 planes, 1..32 channels.
+cudaError_t launch_train_conv(const float* X, int B, int C, int H, int W, const __nv_bfloat16* Wb, int ldw, int N,
+                              const float* bias, int relu, const float* gate, int sign, float* Y, int* err, int sms,
+                              cudaStream_t st);
+cudaError_t launch_train_wgrad(const float* X, const float* dZ, int B, int C, int N, int H, int W, float* dW, float* db,
+                               int* err, int sms, cudaStream_t st);
 // Resident blocks per SM of the FP64 solver shape (0 if unknown).
 int gmres_fp64_blocks_per_sm(int ept, int nt, int minb, size_t smem);
 // dst[q] = src[perm[q]] (gather) or dst[perm[q]] = src[q] (scatter), planes of n doubles

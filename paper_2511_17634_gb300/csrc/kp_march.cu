@@ -803,8 +803,6 @@ kp_status kp_march_create(kp_ctx* c, int ngroups, const kp_group* groups, const 
             t.count = std::min(128, end - q);
             t.nv = kp::kVbRows;
             t.ccol0 = 0;
-            t.kc0 = t.kc1 = 0;
-            t.atomic = 0;
             tl[par].push_back(t);
           }
         k = end;
@@ -864,8 +862,6 @@ kp_status kp_march_create(kp_ctx* c, int ngroups, const kp_group* groups, const 
               t.count = std::min(128, end - q);
               t.nv = std::min(48, (int)pairs - pb);
               t.ccol0 = pb;
-              t.kc0 = t.kc1 = 0;
-              t.atomic = 0;
               tl[par].push_back(t);
             }
         k = end;

@@ -165,23 +165,21 @@ proj_gemm_bf16_kernel(const __grid_constant__ CUtensorMap mapB, const __grid_con
   for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
     const ProjTile tile = tiles[t];
     const int round = (t - (int)blockIdx.x) / (int)gridDim.x;   // tiles already done by this CTA
-    const int kc0 = tile.kc1 > 0 ? tile.kc0 : 0;
-    const int nkt = tile.kc1 > 0 ? tile.kc1 - tile.kc0 : nk;
     if (warp == 0 && lane == 0) {
       // TMA producer
-      for (int kc = 0; kc < nkt; ++kc) {
+      for (int kc = 0; kc < nk; ++kc) {
         const uint32_t it = base_phase + kc;
         const int s = it % kStages;
         const uint32_t use = it / kStages;
         if (use > 0 && !mbar_wait(&sm.empty[s], (use - 1) & 1)) { sm.abort = 1; break; }
         mbar_expect_tx(&sm.full[s], kBytesA + kBytesB);
-        tma_load_2d(sm.A[s], &mapB, (kc0 + kc) * kTileK, tile.row0, &sm.full[s]);
-        tma_load_2d(sm.B[s], &mapV, (kc0 + kc) * kTileK, tile.vrow0, &sm.full[s]);
+        tma_load_2d(sm.A[s], &mapB, kc * kTileK, tile.row0, &sm.full[s]);
+        tma_load_2d(sm.B[s], &mapV, kc * kTileK, tile.vrow0, &sm.full[s]);
         issued = it + 1;
       }
     } else if (warp == 1 && lane == 0) {
       // MMA issuer
-      for (int kc = 0; kc < nkt; ++kc) {
+      for (int kc = 0; kc < nk; ++kc) {
         const uint32_t it = base_phase + kc;
         const int s = it % kStages;
         const uint32_t use = it / kStages;
@@ -216,14 +214,13 @@ proj_gemm_bf16_kernel(const __grid_constant__ CUtensorMap mapB, const __grid_con
 #pragma unroll
         for (int i = 0; i < 16; ++i)
           if (c0 + i < tile.nv) {
-            if (tile.atomic) atomicAdd(crow + i, v[i]);
-            else crow[i] = v[i];
+            crow[i] = v[i];
           }
       }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    base_phase += (uint32_t)nkt;
+    base_phase += (uint32_t)nk;
   }
   __syncthreads();
   if (sm.abort && warp == 0 && lane == 0) {
