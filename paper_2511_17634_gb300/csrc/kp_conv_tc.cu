@@ -74,7 +74,8 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv3x3_tc_kernel(const ConvA
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 6);
   volatile int* abort = reinterpret_cast<volatile int*>(bars + 7);
   constexpr uint32_t kCols = 2 * kMT * NOUT;   // 512 or 256 TMEM columns
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // (uniform, and known to be)
   const int total = a.B * a.nst;
 
   if (tid == 0) {
@@ -131,7 +132,8 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv3x3_tc_kernel(const ConvA
       }
     }
   } else if (warp == 5) {
-    if (lane == 0) {
+    {
+      const bool issue = lane == 0;
       constexpr uint32_t idesc = idesc_f16(128, NOUT);
       uint32_t committed = 0;
       int it = 0;
@@ -153,11 +155,12 @@ __global__ void __launch_bounds__(kConvThreads, 1) conv3x3_tc_kernel(const ConvA
             for (int kc = 0; kc < CIC / 2; ++kc) {
               const uint64_t ad = desc_plain(sa + (uint32_t)(2 * kc) * L * 16 + (uint32_t)row * 16, L * 16, 128);
               const uint64_t bd = desc_plain(sw + (uint32_t)((t * CIC + 2 * kc) * NOUT * 16), NOUT * 16, 128);
-              mma_f16(d, ad, bd, idesc, (t > 0 || kc > 0) ? 1u : 0u);
+              mma_f16_one(issue, d, ad, bd, idesc, (t > 0 || kc > 0) ? 1u : 0u);
             }
           }
         }
-        mma_commit_to(&mdone[s]);
+        if (issue) mma_commit_to(&mdone[s]);
+        __syncwarp();
         committed = (uint32_t)it + 1;
       }
       if (*abort && committed > 0) {
@@ -287,7 +290,8 @@ __global__ void __launch_bounds__(kColThreads, 1) conv3x3_col_kernel(const ConvA
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * NS + 4);
   volatile int* abort = reinterpret_cast<volatile int*>(bars + 2 * NS + 5);
   constexpr uint32_t kCols = 2 * kCT * NOUT;   // 512 or 256 TMEM columns
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // (uniform, and known to be)
   const int HP = a.H + 2;
   const int nct = (a.W + kCT - 1) / kCT;
   const int total = a.B * nct;
@@ -366,7 +370,8 @@ __global__ void __launch_bounds__(kColThreads, 1) conv3x3_col_kernel(const ConvA
       }
     }
   } else if (warp == kColEpiWarps + 1) {
-    if (lane == 0) {
+    {
+      const bool issue = lane == 0;
       uint32_t committed = 0;
       int it = 0;
       for (int st = blockIdx.x; st < total; st += gridDim.x, ++it) {
@@ -404,12 +409,15 @@ __global__ void __launch_bounds__(kColThreads, 1) conv3x3_col_kernel(const ConvA
             for (int kc = 0; kc < CIC / 2; ++kc) {
               const uint64_t ad = acol + (uint64_t)(2 * kc * L + dj);
               const uint64_t bd = bbase + (uint64_t)((dj * CIC + 2 * kc) * 3 * NOUT + g0 * NOUT);
-              mma_f16(d, ad, bd, idesc, 1u);
+              mma_f16_one(issue, d, ad, bd, idesc, 1u);
             }
           }
         }
-        mma_commit_to(&sfree[s]);                   // the input stage may be refilled
-        mma_commit_to(&tfull[tb]);                  // the accumulators are ready
+        if (issue) {
+          mma_commit_to(&sfree[s]);                 // the input stage may be refilled
+          mma_commit_to(&tfull[tb]);                // the accumulators are ready
+        }
+        __syncwarp();
         committed = (uint32_t)it + 1;
       }
       if (*abort && committed > 0) {

@@ -81,7 +81,8 @@ __global__ void __launch_bounds__(kTrainThreads, 1) train_conv_kernel(const Trai
   __shared__ uint32_t tmem_slot;
   __shared__ int abort_s;
   volatile int* abort = &abort_s;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(kFull, tid >> 5, 0);   // (uniform, and known to be)
   const int P = a.H * a.W, K = 9 * a.C;
   const int total = a.B * P;                       // (at most 2^30)
   const int ntiles = (total + 127) / 128;
@@ -240,16 +241,17 @@ __global__ void __launch_bounds__(kTrainThreads, 1) train_conv_kernel(const Trai
     }
     __syncthreads();                               // tile staged; TMEM buffer it & 1 read (epilogue of it - 2)
     if (!stager) {
-      if (lane == 0 && !*abort) {
+      if (!*abort) {
         tc_fence_after();
+        const bool issue = lane == 0;
         const uint32_t idesc = idesc_f16(128, nout);
         const uint64_t ad0 = desc_sw128(su32(As)), bd0 = desc_sw128(su32(Ws));
         for (int ks = 0; ks < ksteps; ++ks) {
           const int c = ks >> 2, kk = ks & 3;
-          mma_f16(tmem + (uint32_t)((it & 1) * 32), ad0 + (uint64_t)(c * 1024 + kk * 2),
+          mma_f16_one(issue, tmem + (uint32_t)((it & 1) * 32), ad0 + (uint64_t)(c * 1024 + kk * 2),
                   bd0 + (uint64_t)(c * 256 + kk * 2), idesc, ks > 0 ? 1u : 0u);
         }
-        mma_commit_to(&done[it & 1]);
+        if (issue) mma_commit_to(&done[it & 1]);
       }
       __syncwarp();
     } else if (it > 0) {
@@ -294,7 +296,8 @@ __global__ void __launch_bounds__(kWgThreads, 1) train_wgrad_kernel(const WgradA
   __shared__ uint32_t tmem_slot;
   __shared__ int abort_s;
   volatile int* abort = &abort_s;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(kFull, tid >> 5, 0);   // (uniform, and known to be)
   const int P = a.H * a.W, rows = 9 * a.C, mi = blockIdx.y;
   const int r0 = mi * 128, rn = min(128, rows - r0);
   const int total = a.B * P;                       // (at most 2^30)
@@ -440,15 +443,16 @@ __global__ void __launch_bounds__(kWgThreads, 1) train_wgrad_kernel(const WgradA
     }
     __syncthreads();
     if (!stager) {
-      if (lane == 0 && !*abort) {
+      if (!*abort) {
         tc_fence_after();
+        const bool issue = lane == 0;
         const uint32_t idesc = idesc_f16(128, nout);
         const uint64_t ad0 = desc_sw128(su32(As)), bd0 = desc_sw128(su32(Bs));
         const int nk = ch + 1 < ch1 ? 8 : 4;       // K steps of 16 pixels
         for (int kk = 0; kk < nk; ++kk)
-          mma_f16(tmem, ad0 + (uint64_t)((kk >> 2) * 1024 + (kk & 3) * 2), bd0 + (uint64_t)((kk >> 2) * 256 + (kk & 3) * 2),
+          mma_f16_one(issue, tmem, ad0 + (uint64_t)((kk >> 2) * 1024 + (kk & 3) * 2), bd0 + (uint64_t)((kk >> 2) * 256 + (kk & 3) * 2),
                   idesc, (it > 0 || kk > 0) ? 1u : 0u);
-        mma_commit_to(&done[s]);
+        if (issue) mma_commit_to(&done[s]);
       }
       __syncwarp();
     }

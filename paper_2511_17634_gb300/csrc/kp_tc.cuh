@@ -83,6 +83,17 @@ __device__ __forceinline__ void mma_f16(uint32_t d, uint64_t a, uint64_t b, uint
       "l"(a), "l"(b), "r"(idesc), "r"(acc));
 }
 
+// The same from warp-uniform code: every lane of the issuing warp runs it, one
+// issues.  The descriptors then stay in uniform registers; computed by one
+// lane in a divergent branch they are moved there for every MMA, which took
+// about 118 cycles per MMA where the tensor core needs 46 (N = 48) to 56 (96).
+__device__ __forceinline__ void mma_f16_one(bool issue, uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+  asm volatile(
+      "{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n"
+      " @q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
+      "l"(a), "l"(b), "r"(idesc), "r"(acc), "r"((uint32_t)issue));
+}
+
 __device__ __forceinline__ void mma_commit_to(uint64_t* b) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(su32(b))
                : "memory");
