@@ -56,11 +56,11 @@ kp_status gmres_shape(kp_ctx* c, int nmax, int m, Shape* out, bool mixed, int wm
                                                              : sh.nt == 64 ? 4 : 2);
     if (mixed) {                                 // the FP32 solver has the 256- and 128-thread shapes
       if (sh.nt == 64) { sh.nt = 128; sh.ept = 8; }
-      sh.minb = sh.nt == 128 ? 6 : 4;
+      sh.minb = 4;
     }
   } else if (nmax <= 4096 && !(mixed && c->opt.cluster_size)) {
-    sh.ept = 8;
-    sh.nt = 512;
+    sh.ept = mixed ? 16 : 8;
+    sh.nt = mixed ? 256 : 512;
     if (mixed) sh.minb = 2;
   } else if (mixed) {
     // a cluster of CTAs, each holding whole columns: on request 2, 4 or 8 of
@@ -79,17 +79,16 @@ kp_status gmres_shape(kp_ctx* c, int nmax, int m, Shape* out, bool mixed, int wm
     sh.minb = c->opt.cluster_blocks_per_sm ? c->opt.cluster_blocks_per_sm : (sh.cs == 16 ? 4 : 2);
     if (sh.cs == 16 ? (sh.minb != 2 && sh.minb != 4) : sh.minb > 2)
       return set_error(c, KP_ERR_UNSUPPORTED, "cluster of %d CTAs: %d CTAs per SM not built", sh.cs, sh.minb);
-    if (!c->opt.cluster_size) { sh.cs /= 2; sh.nt = 512; }
+    if (!c->opt.cluster_size) { sh.cs /= 2; sh.ept = 16; }
   } else {
     return set_error(c, KP_ERR_UNSUPPORTED, "N=%d: FP64 grids above 4096 unknowns are not supported (use the mixed-precision mode)", nmax);
   }
   const int npad = sh.ept * sh.nt;
   sh.vld = npad;
   if (mixed) {
-    // full CTAs, columns that divide the threads of a sub-block (half a CTA
-    // of the default clusters); the shapes on request have no such kernel
-    const int ns = sh.cs ? 256 : sh.nt;
-    sh.reg = one_size && nmax == sh.ctas() * npad && hmax > 0 && ns % hmax == 0 && !c->opt.cluster_size && sh.nt != 128;
+    // full CTAs, columns that divide the CTA's threads; the shapes on request
+    // have no such kernel
+    sh.reg = one_size && nmax == sh.ctas() * npad && hmax > 0 && sh.nt % hmax == 0 && !c->opt.cluster_size && sh.nt == 256;
     sh.hmax = sh.cs || sh.reg ? hmax : 0;
     sh.vld += 2 * sh.hmax;
   }
@@ -102,8 +101,8 @@ kp_status gmres_shape(kp_ctx* c, int nmax, int m, Shape* out, bool mixed, int wm
   const size_t budget = mixed ? c->smem_optin / sh.minb - (sh.minb >= 2 ? 1024 : 0)
                       : npad <= 1024 ? c->smem_optin / sh.minb - (sh.minb > 2 ? 1024 : 0)
                                      : c->smem_optin;
-  // the mixed-precision solver keeps x (hi, lo) in two slots between cycles
-  const int smin = mixed ? 2 : 1;
+  // the mixed-precision solver keeps x (hi, lo) and r in three slots between cycles
+  const int smin = mixed ? 3 : 1;
   int S = c->opt.smem_vectors;
   if (S <= 0) {
     S = smin;
@@ -114,8 +113,8 @@ kp_status gmres_shape(kp_ctx* c, int nmax, int m, Shape* out, bool mixed, int wm
   if (bytes(S) > c->smem_optin) return set_error(c, KP_ERR_UNSUPPORTED, "shared memory too small");
   sh.S = S;
   sh.smem = bytes(S);
-  sh.ws = (size_t)std::max(m + 1 - S, 0) * sh.vld + (mixed ? 2 * (size_t)sh.vld + 2 * (size_t)npad : 0);
-  sh.ws = (sh.ws + 1) / 2 * 2;                   // (x and the coefficients are float pairs)
+  sh.ws = (size_t)std::max(m + 1 - S, 0) * sh.vld + (mixed ? 2 * (size_t)(sh.vld + sh.vld % 2) + 4 * (size_t)npad : 0);
+  sh.ws = (sh.ws + 3) / 4 * 4;                   // (the coefficients are read as float4)
   *out = sh;
   return KP_OK;
 }

@@ -101,15 +101,21 @@ __device__ __forceinline__ void split_hi_lo(float f, __nv_bfloat16& hi, __nv_bfl
 // cancellation of the two large 1/dt terms.  Evaluated in double-float on the
 // FP32 pipe (kp_dd.cuh; about 2^-44 of c |m| absolute), the FP64 field split
 // without FP64 instructions.
-__device__ __forceinline__ dd step_residual_at(const double* m, int p, int H, int W, dd c, dd e) {
-  const int i = p / H, j = p - i * H;
-  const dd z = {0.f, 0.f};
-  const dd mC = dd_from_double(m[p]);
-  const dd mE = i + 1 < W ? dd_from_double(m[p + H]) : z, mW = i > 0 ? dd_from_double(m[p - H]) : z;
-  const dd mN = j + 1 < H ? dd_from_double(m[p + 1]) : z, mS = j > 0 ? dd_from_double(m[p - 1]) : z;
-  const dd lap = dd_sub(dd_add(dd_add(mE, mW), dd_add(mN, mS)), dd{4.f * mC.hi, 4.f * mC.lo});
-  const dd dx = dd_sub(mE, mW), dy = dd_sub(mN, mS);
-  return dd_add(dd_mul(c, lap), dd_mul(e, dd_add(dd_mul(dx, dx), dd_mul(dy, dy))));
+__device__ __forceinline__ dd step_residual(dd C, dd E, dd W, dd N, dd S, dd c, dd e) {
+  auto mul = [](float ah, float al, float bh, float bl) -> dd {   // a b, unnormalised
+    const float t = __fmul_rn(ah, bh);
+    return {t, fmaf(al, bh, fmaf(ah, bl, fmaf(ah, bh, -t)))};
+  };
+  const dd s1 = kp::dd_two_sum(E.hi, W.hi), s2 = kp::dd_two_sum(N.hi, S.hi), s = kp::dd_two_sum(s1.hi, s2.hi);
+  const dd l = kp::dd_two_sum(s.hi, -4.f * C.hi);
+  const float ll = (((E.lo + W.lo) + (N.lo + S.lo)) + ((s1.lo + s2.lo) + (s.lo + l.lo))) - 4.f * C.lo;
+  const dd dx = kp::dd_two_sum(E.hi, -W.hi), dy = kp::dd_two_sum(N.hi, -S.hi);
+  const float xl = dx.lo + (E.lo - W.lo), yl = dy.lo + (N.lo - S.lo);
+  const dd x2 = mul(dx.hi, xl, dx.hi, xl), y2 = mul(dy.hi, yl, dy.hi, yl);
+  const dd q = kp::dd_two_sum(x2.hi, y2.hi);
+  const dd t1 = mul(c.hi, c.lo, l.hi, ll), t2 = mul(e.hi, e.lo, q.hi, q.lo + (x2.lo + y2.lo));
+  const dd r = kp::dd_two_sum(t1.hi, t2.hi);
+  return kp::dd_fast_two_sum(r.hi, r.lo + (t1.lo + t2.lo));
 }
 
 // rho_b = ||r_b|| / sqrt(P), one block per sample; g2 = g2v, or g2s[*step +
@@ -119,33 +125,87 @@ __device__ __forceinline__ dd step_residual_at(const double* m, int p, int H, in
 // (the FP64 pipe, not HBM, bounds this part on GB300).  Blocks of 1024
 // threads: with one block per plane, fewer and larger blocks keep the last
 // wave short (1536 planes are 5 waves of 2 blocks per SM, not 1.3 waves of 8).
+//
+// The plane is split into double-float once per point, in shared memory, strip
+// by strip of columns (five splits per point straight from memory and sums
+// renormalised at every step were 300 instructions per point: 95 us for 512
+// planes of 128x128).  Columns too long for a strip are read directly.
 constexpr int kRmsThreads = 1024;
+constexpr int kRmsStrip = 8192;                    // points of a strip and the columns beside it
+constexpr size_t kRmsSmem = kRmsStrip * sizeof(float2);
 
-__global__ void step_residual_rms_kernel(const double* const* m, int H, int W, double dt, double g2v,
-                                         const double* g2s, const int* step, int step_offset, double* rho,
-                                         float* rout, size_t rld) {
+__global__ void __launch_bounds__(kRmsThreads) step_residual_rms_kernel(const double* const* m, int H, int W, double g2v,
+                                                                        const double* g2s, const int* step,
+                                                                        int step_offset, double* rho, float* rout,
+                                                                        size_t rld) {
+  extern __shared__ float2 strip[];
   __shared__ double red[32];
   const int b = blockIdx.x, P = H * W;
   const double g2 = g2s ? g2s[*step + step_offset] : g2v;
   const double hh = (double)H * (double)H;
   const dd c = dd_from_double(0.5 * g2 * hh), e = dd_from_double(0.125 * g2 * hh);
+  const double* mp = m[b];
   float* ro = rout + (size_t)b * rld;
-  dd acc = {0.f, 0.f};
-  for (int p = threadIdx.x; p < P; p += blockDim.x) {
-    const dd r = step_residual_at(m[b], p, H, W, c, e);
-    acc = dd_add(acc, dd_mul(r, r));
-    ro[p] = r.hi;
+  float ah = 0.f, al = 0.f;                        // this thread's sum of r^2, unnormalised
+  auto add = [&](dd r) {
+    const float t = __fmul_rn(r.hi, r.hi), te = fmaf(2.f * r.hi, r.lo, fmaf(r.hi, r.hi, -t));
+    const dd s = kp::dd_two_sum(ah, t);
+    ah = s.hi;
+    al += s.lo + te;
+  };
+  const int cols = kRmsStrip / H - 2;              // columns of a strip
+  if (cols >= 1) {
+    for (int i0 = 0; i0 < W; i0 += cols) {
+      const int nc = min(cols, W - i0);
+      __syncthreads();
+      for (int q = threadIdx.x; q < (nc + 2) * H; q += kRmsThreads) {
+        const int p = (i0 - 1) * H + q;
+        const dd v = p >= 0 && p < P ? dd_from_double(mp[p]) : dd{0.f, 0.f};
+        strip[q] = make_float2(v.hi, v.lo);
+      }
+      __syncthreads();
+      for (int q = H + threadIdx.x; q < (nc + 1) * H; q += kRmsThreads) {
+        const int j = q % H;
+        const float2 z = make_float2(0.f, 0.f);
+        const float2 C = strip[q], E = strip[q + H], V = strip[q - H];
+        const float2 N = j + 1 < H ? strip[q + 1] : z, S = j > 0 ? strip[q - 1] : z;
+        const dd r = step_residual({C.x, C.y}, {E.x, E.y}, {V.x, V.y}, {N.x, N.y}, {S.x, S.y}, c, e);
+        add(r);
+        ro[(i0 - 1) * H + q] = r.hi;
+      }
+    }
+  } else {
+    const dd z = {0.f, 0.f};
+    for (int p = threadIdx.x; p < P; p += kRmsThreads) {
+      const int i = p / H, j = p - i * H;
+      const dd r = step_residual(dd_from_double(mp[p]), i + 1 < W ? dd_from_double(mp[p + H]) : z,
+                                 i > 0 ? dd_from_double(mp[p - H]) : z, j + 1 < H ? dd_from_double(mp[p + 1]) : z,
+                                 j > 0 ? dd_from_double(mp[p - 1]) : z, c, e);
+      add(r);
+      ro[p] = r.hi;
+    }
   }
-  double s = dd_to_double(acc);
+  double s = dd_to_double(kp::dd_fast_two_sum(ah, al));
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
-    rho[b] = sqrt(t / P);
+  if (threadIdx.x < 32) {
+    double t = red[threadIdx.x];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (threadIdx.x == 0) rho[b] = sqrt(t / P);
   }
+}
+
+cudaError_t launch_step_residual(int B, const double* const* m, int H, int W, double g2v, const double* g2s,
+                                 const int* step, int step_offset, double* rho, float* rout, size_t rld,
+                                 cudaStream_t st) {
+  cudaError_t e = cudaFuncSetAttribute(step_residual_rms_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)kRmsSmem);
+  if (e != cudaSuccess) return e;
+  step_residual_rms_kernel<<<B, kRmsThreads, kRmsSmem, st>>>(m, H, W, g2v, g2s, step, step_offset, rho, rout, rld);
+  return cudaGetLastError();
 }
 
 // Network input planes of sample b: the target's plane (its lagged field
@@ -523,12 +583,11 @@ kp_status kp_cnn_pack_inputs(kp_cnn* n, int B, const double* const* img, const d
   cudaError_t e = cudaMallocAsync((void**)&d, h.size() * sizeof(double*), n->ctx->stream);
   if (e == cudaSuccess) e = cudaMemcpyAsync(d, h.data(), h.size() * sizeof(double*), cudaMemcpyHostToDevice, n->ctx->stream);
   if (e == cudaSuccess) {
-    const double dt = 1.0 / T;
-    step_residual_rms_kernel<<<B, kRmsThreads, 0, n->ctx->stream>>>(d, n->H, n->W, dt, g2n, nullptr, nullptr, 0, rho,
-                                                            in + 8 * (size_t)n->P, 10 * (size_t)n->P);
+    e = launch_step_residual(B, d, n->H, n->W, g2n, nullptr, nullptr, 0, rho, in + 8 * (size_t)n->P,
+                             10 * (size_t)n->P, n->ctx->stream);
     pack_inputs_kernel<<<dim3(grid_for(n->P), B), 256, 0, n->ctx->stream>>>(d, d + B, (float)step / (float)T,
                                                                            rho, n->P, in);
-    e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaGetLastError();
   }
   if (d) cudaFreeAsync(d, n->ctx->stream);
   return e == cudaSuccess ? KP_OK : kp::cuda_error(n->ctx, e, "CNN pack");
@@ -597,11 +656,11 @@ cudaError_t cnn_enqueue_guess(kp_cnn* n, int B, const double* const* mprev, cons
   const dim3 grid(std::min((n->P + 255) / 256, 1024), B);
   // the FP32 residual goes through the network's output buffer, which the
   // packing kernel has read before any layer runs
-  step_residual_rms_kernel<<<B, kRmsThreads, 0, st>>>(mprev, n->H, n->W, 1.0 / T, 0.0, g2, step, step_offset, rho,
-                                              n->dout, (size_t)n->P);
+  cudaError_t e = launch_step_residual(B, mprev, n->H, n->W, 0.0, g2, step, step_offset, rho, n->dout, (size_t)n->P, st);
+  if (e != cudaSuccess) return e;
   march_pack_kernel<<<grid, 256, 0, st>>>(mprev, mseed, n->dout, step, step_offset, rho, T, n->H, n->W,
                                           n->geo.halo, n->geo.Rp, n->pin);
-  cudaError_t e = cudaGetLastError();
+  e = cudaGetLastError();
   if (e == cudaSuccess) e = conv_layers(n, B, delta, st);
   return e;
 }

@@ -428,66 +428,74 @@ __global__ void __launch_bounds__(kColThreads, 1) conv3x3_col_kernel(const ConvA
     }
   } else {
     // epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31 = pixel rows j of
-    // every (kColEpiWarps / 4)-th output column, starting at column w / 4
+    // every (kColEpiWarps / 4)-th output column, starting at column w / 4, and
+    // returns them to zero for the MMAs of tile it + 2.  Two warps per
+    // scheduler take turns here, so the chain of one column is kept short: the
+    // biases are in registers (loaded per value behind stores that may alias
+    // they were a round of latency per 8 channels), one TMEM load per column
+    // (of one value for a single output).
+    const int quad = warp & 3;
+    const int j = quad * 32 + lane;
+    const bool valid_j = j < a.H;
+    float bias[NOUT];
+#pragma unroll
+    for (int c = 0; c < NOUT; ++c) bias[c] = c < a.cout ? a.bias[c] : 0.f;
+    const size_t plane = (size_t)a.Rp * 8;         // BF16 values of a chunk plane
     int it = 0;
     for (int st = blockIdx.x; st < total; st += gridDim.x, ++it) {
       const int tb = it & 1;
       const uint32_t ut = (uint32_t)it >> 1;
       if (!bar_wait(&tfull[tb], ut & 1, abort)) { *abort = 1; break; }
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      tc_fence_after();
       const int b = st / nct;
       const int i0 = (st - b * nct) * kCT;
       const int kv = min(kCT, a.W - i0);
-      const int quad = warp & 3;
-      const int j = quad * 32 + lane;
-      const bool valid_j = j < a.H;
+      __nv_bfloat16* op = F32OUT ? nullptr
+                                 : a.out_pad + (size_t)b * (NOUT / 8) * plane + ((size_t)a.halo + (size_t)i0 * HP + 1 + j) * 8;
+      float* of = F32OUT ? a.out_f32 + (size_t)b * a.cout * a.H * a.W + (size_t)i0 * a.H + j : nullptr;
 #pragma unroll 1
       for (int q = warp >> 2; q < kv; q += kColEpiWarps / 4) {
-        const int o = i0 + q;
         const uint32_t taddr =
             tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(tb * kCT * NOUT + NOUT * (kCT - 1 - q));
-        float v[NOUT];
-#pragma unroll
-        for (int c0 = 0; c0 < NOUT; c0 += 16) {
-          float w16[16];
-          tmem_ld_x16(taddr + (uint32_t)c0, w16);
-#pragma unroll
-          for (int k = 0; k < 16; ++k) v[c0 + k] = w16[k];
+        if (F32OUT && a.cout == 1) {
+          const float v = tmem_ld_x1(taddr) + bias[0];
+          tmem_zero_x16(taddr);
+          if (valid_j) of[(size_t)q * a.H] = v;
+          continue;
         }
+        float v[NOUT];
+        if constexpr (NOUT == 32) tmem_ld_x32(taddr, v);
+        else tmem_ld_x16(taddr, v);
+#pragma unroll
+        for (int c0 = 0; c0 < NOUT; c0 += 16) tmem_zero_x16(taddr + (uint32_t)c0);
         if (!valid_j) continue;
         if (F32OUT) {
 #pragma unroll
           for (int co = 0; co < NOUT; ++co)
-            if (co < a.cout)
-              a.out_f32[((size_t)b * a.cout + co) * a.H * a.W + (size_t)o * a.H + j] = v[co] + a.bias[co];
+            if (co < a.cout) of[((size_t)co * a.W + q) * a.H] = v[co] + bias[co];
         } else {
-          const size_t prow = (size_t)a.halo + (size_t)o * HP + 1 + j;
+          if (a.cout < NOUT)                       // channels past cout stay zero whatever the input
+#pragma unroll
+            for (int c = 0; c < NOUT; ++c) v[c] = c < a.cout ? v[c] : 0.f;
+          uint4 pk[NOUT / 8];
 #pragma unroll
           for (int cc = 0; cc < NOUT / 8; ++cc) {
-            uint32_t pk[4];
+            uint32_t w[4];
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
               const int c0 = cc * 8 + 2 * e;
-              const float x0 = c0 < a.cout ? fmaxf(v[c0] + a.bias[c0], 0.f) : 0.f;
-              const float x1 = c0 + 1 < a.cout ? fmaxf(v[c0 + 1] + a.bias[c0 + 1], 0.f) : 0.f;
-              __nv_bfloat162 h2 = __floats2bfloat162_rn(x0, x1);
-              pk[e] = *reinterpret_cast<uint32_t*>(&h2);
+              __nv_bfloat162 h2 = __floats2bfloat162_rn(fmaxf(v[c0] + bias[c0], 0.f), fmaxf(v[c0 + 1] + bias[c0 + 1], 0.f));
+              w[e] = *reinterpret_cast<uint32_t*>(&h2);
             }
-            *reinterpret_cast<uint4*>(a.out_pad + (((size_t)b * (NOUT / 8) + cc) * a.Rp + prow) * 8) =
-                make_uint4(pk[0], pk[1], pk[2], pk[3]);
+            pk[cc] = make_uint4(w[0], w[1], w[2], w[3]);
           }
+#pragma unroll
+          for (int cc = 0; cc < NOUT / 8; ++cc)
+            *reinterpret_cast<uint4*>(op + cc * plane + (size_t)q * HP * 8) = pk[cc];
         }
       }
-      // return the columns this warp read to zero for the MMAs of tile it + 2
-#pragma unroll 1
-      for (int q = warp >> 2; q < kv; q += kColEpiWarps / 4) {
-        const uint32_t taddr =
-            tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(tb * kCT * NOUT + NOUT * (kCT - 1 - q));
-#pragma unroll
-        for (int c0 = 0; c0 < NOUT; c0 += 16) tmem_zero_x16(taddr + (uint32_t)c0);
-      }
       asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      tc_fence_before();
       __syncwarp();
       if (lane == 0) bar_arrive(&tempty[tb]);
     }

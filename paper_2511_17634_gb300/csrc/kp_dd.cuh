@@ -65,17 +65,16 @@ __device__ __forceinline__ dd dd_mul(dd x, dd y) {
 }
 
 __device__ __forceinline__ dd dd_from_double(double x) {
-  const unsigned long long u = (unsigned long long)__double_as_longlong(x);
-  const unsigned int uh = (unsigned int)(u >> 32), ul = (unsigned int)u;
-  const unsigned int sign = uh & 0x80000000u;
-  const int e = (int)((uh >> 20) & 0x7FFu);          // biased FP64 exponent
-  if (e < 1023 - 100) return {0.f, 0.f};
+  const unsigned int uh = (unsigned int)__double2hiint(x), ul = (unsigned int)__double2loint(x);
+  const unsigned int sign = uh & 0x80000000u, mag = uh ^ sign;
+  const int e = (int)(mag >> 20);                    // biased FP64 exponent
   // top 24 significant bits -> float (exponent rebiased by 1023 - 127 = 896)
-  const float hi = __uint_as_float(sign | ((unsigned int)(e - 896) << 23) | ((uh & 0xFFFFFu) << 3) | (ul >> 29));
-  if (e < 949) return {hi, 0.f};
-  // the 29 bits below: an integer times 2^(e - 1075)
-  const float scale = __uint_as_float(sign | ((unsigned int)(e - 948) << 23));
-  return {hi, __uint2float_rn(ul & 0x1FFFFFFFu) * scale};
+  const float hi = __uint_as_float(sign | __funnelshift_l(ul, mag - (896u << 20), 3));
+  // the 29 bits below: an integer times 2^(e - 1075), zero for e < 949
+  const float scale = __uint_as_float(sign | ((unsigned int)max(e - 948, 0) << 23));
+  const float lo = __uint2float_rn(ul & 0x1FFFFFFFu) * scale;
+  const bool tiny = e < 1023 - 100;
+  return {tiny ? 0.f : hi, tiny ? 0.f : lo};
 }
 
 // 1 / sqrt(x) for x > 0: the FP32 estimate y and one correction from the
@@ -99,6 +98,9 @@ __device__ __forceinline__ dd dd_sqrt(dd x) {
   return dd_fast_two_sum(y, r * (0.5f / y));
 }
 
+// (out of line, or its FP64 instructions are speculated for every value)
+static __device__ __noinline__ double dd_to_double_slow(dd x) { return (double)x.hi + (double)x.lo; }
+
 // hi + lo rounded to FP64.  A conversion and an add on the FP64 pipe cost
 // three warp instructions of 64 cycles each; this composes the bit pattern
 // with integer operations: hi's pattern plus lo as a signed count of units in
@@ -108,7 +110,7 @@ __device__ __forceinline__ dd dd_sqrt(dd x) {
 __device__ __forceinline__ double dd_to_double(dd x) {
   const unsigned int u = __float_as_uint(x.hi);
   const unsigned int e = (u >> 23) & 0xFFu;
-  if (e < 56 || e > 254) return (double)x.hi + (double)x.lo;   // small, zero, Inf, NaN
+  if (e < 56 || e > 254) return dd_to_double_slow(x);          // small, zero, Inf, NaN
   const float lo = (u >> 31) ? -x.lo : x.lo;                   // relative to |hi|
   const unsigned int below = (u & 0x7FFFFFu) == 0u && lo < 0.f;
   const int t = __float2int_rn(lo * __uint_as_float((306u + below - e) << 23));

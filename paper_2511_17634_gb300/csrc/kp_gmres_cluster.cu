@@ -8,17 +8,16 @@ namespace kp {
 
 cudaError_t launch_gmres_cluster(const GmresParams& p, int ept, int nt, int cs, bool reg, size_t smem,
                                  cudaStream_t st) {
-  if (ept != 8) return cudaErrorInvalidValue;
-  if (nt == 512) {                               // the default: 4096 points per CTA
-    if (cs == 4) return reg ? launch_mx<8, 512, 4, 2, 2, true>(p, smem, st) : launch_mx<8, 512, 4, 2, 2, false>(p, smem, st);
-    if (cs == 2) return reg ? launch_mx<8, 512, 2, 2, 2, true>(p, smem, st) : launch_mx<8, 512, 2, 2, 2, false>(p, smem, st);
+  if (ept == 16 && nt == 256) {                  // the default: 4096 points per CTA
+    if (cs == 4) return reg ? launch_mx<16, 256, 4, 2, 2, true>(p, smem, st) : launch_mx<16, 256, 4, 2, 2, false>(p, smem, st);
+    if (cs == 2) return reg ? launch_mx<16, 256, 2, 2, 2, true>(p, smem, st) : launch_mx<16, 256, 2, 2, 2, false>(p, smem, st);
   }
-  if (nt == 256) {                               // cluster_size 2, 4, 8: 2048 points per CTA
-    if (cs == 8) return launch_mx<8, 256, 8, 2, 1, false>(p, smem, st);
-    if (cs == 4) return launch_mx<8, 256, 4, 2, 1, false>(p, smem, st);
-    if (cs == 2) return launch_mx<8, 256, 2, 2, 1, false>(p, smem, st);
+  if (ept == 8 && nt == 256) {                   // cluster_size 2, 4, 8: 2048 points per CTA
+    if (cs == 8) return launch_mx<8, 256, 8, 2, 0, false>(p, smem, st);
+    if (cs == 4) return launch_mx<8, 256, 4, 2, 0, false>(p, smem, st);
+    if (cs == 2) return launch_mx<8, 256, 2, 2, 0, false>(p, smem, st);
   }
-  if (nt == 128 && cs == 16) return launch_mx<8, 128, 16, 4, 1, false>(p, smem, st);   // 1024 points per CTA
+  if (ept == 8 && nt == 128 && cs == 16) return launch_mx<8, 128, 16, 4, 0, false>(p, smem, st);   // 1024 points per CTA
   return cudaErrorInvalidValue;
 }
 

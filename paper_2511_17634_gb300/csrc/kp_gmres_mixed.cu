@@ -8,7 +8,7 @@ namespace kp {
 
 size_t gmres_mixed_smem_bytes(int nt, int cs, int hmax, int vld, int S, int m) {
   const size_t nw = nt / 32, f = sizeof(float), f2 = sizeof(float2);
-  const size_t fixed = (4 * (size_t)m + 1) * f2 + nw * kMaxV * f2 + 2 * kRedV * nw * cs * f + kMaxV * f +
+  const size_t fixed = (4 * (size_t)m + 2) * f2 + nw * kMaxV * f2 + 4 * kRedV * nw * cs * f + kMaxV * f +
                        8 * sizeof(int) + 4 * (size_t)hmax * f;
   const size_t hess = (size_t)m * (m + 1) / 2 * f2;
   // exact Galerkin lays its a x a FP64 matrix over the Hessenberg matrix and the slots
@@ -17,10 +17,10 @@ size_t gmres_mixed_smem_bytes(int nt, int cs, int hmax, int vld, int S, int m) {
 
 cudaError_t launch_gmres_mixed(const GmresParams& p, int ept, int nt, bool reg, size_t smem, cudaStream_t st) {
   if (ept == 4 && nt == 256)
-    return reg ? launch_mx<4, 256, 1, 4, 1, true>(p, smem, st) : launch_mx<4, 256, 1, 4, 1, false>(p, smem, st);
-  if (ept == 8 && nt == 128) return launch_mx<8, 128, 1, 6, 1, false>(p, smem, st);
-  if (ept == 8 && nt == 512)
-    return reg ? launch_mx<8, 512, 1, 2, 1, true>(p, smem, st) : launch_mx<8, 512, 1, 2, 1, false>(p, smem, st);
+    return reg ? launch_mx<4, 256, 1, 4, 0, true>(p, smem, st) : launch_mx<4, 256, 1, 4, 0, false>(p, smem, st);
+  if (ept == 8 && nt == 128) return launch_mx<8, 128, 1, 4, 0, false>(p, smem, st);
+  if (ept == 16 && nt == 256)
+    return reg ? launch_mx<16, 256, 1, 2, 1, true>(p, smem, st) : launch_mx<16, 256, 1, 2, 1, false>(p, smem, st);
   return cudaErrorInvalidValue;
 }
 

@@ -69,26 +69,37 @@ constexpr int kRedV = 16;
 __device__ __forceinline__ float2 as_f2(dd x) { return make_float2(x.hi, x.lo); }
 __device__ __forceinline__ dd as_dd(float2 x) { return {x.x, x.y}; }
 
-// Warp reduce-scatter of 4 FP32 values per lane: every lane ends with the
-// warp sum of value lane >> 3.
-__device__ __forceinline__ float warp_reduce4f(float (&a)[4], int lane) {
+// Warp reduce-scatter of 4 FP32 values per lane, each in NH parts: every lane
+// ends with the warp sum of value lane >> 3 (NH = 1), or of part lane >> 4 of
+// value (lane >> 2) & 3 (NH = 2).
+template <int NH>
+__device__ __forceinline__ float warp_reduce4f(float (&a)[NH][4], int lane) {
+  if (NH == 2) {
+    const bool up = lane & 16;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const float send = up ? a[0][k] : a[NH - 1][k];
+      const float keep = up ? a[NH - 1][k] : a[0][k];
+      a[0][k] = keep + __shfl_xor_sync(kFull, send, 16);
+    }
+  }
+  constexpr int o = NH == 2 ? 8 : 16;
 #pragma unroll
   for (int k = 0; k < 2; ++k) {
-    const bool up = lane & 16;
-    const float send = up ? a[k] : a[k + 2];
-    const float keep = up ? a[k + 2] : a[k];
-    a[k] = keep + __shfl_xor_sync(kFull, send, 16);
+    const bool up = lane & o;
+    const float send = up ? a[0][k] : a[0][k + 2];
+    const float keep = up ? a[0][k + 2] : a[0][k];
+    a[0][k] = keep + __shfl_xor_sync(kFull, send, o);
   }
   {
-    const bool up = lane & 8;
-    const float send = up ? a[0] : a[1];
-    const float keep = up ? a[1] : a[0];
-    a[0] = keep + __shfl_xor_sync(kFull, send, 8);
+    const bool up = lane & (o / 2);
+    const float send = up ? a[0][0] : a[0][1];
+    const float keep = up ? a[0][1] : a[0][0];
+    a[0][0] = keep + __shfl_xor_sync(kFull, send, o / 2);
   }
-  a[0] += __shfl_xor_sync(kFull, a[0], 4);
-  a[0] += __shfl_xor_sync(kFull, a[0], 2);
-  a[0] += __shfl_xor_sync(kFull, a[0], 1);
-  return a[0];
+#pragma unroll
+  for (int q = o / 4; q > 0; q /= 2) a[0][0] += __shfl_xor_sync(kFull, a[0][0], q);
+  return a[0][0];
 }
 
 // alpha = R^{-1} (G c) in double-float by one warp (the double-float form of
@@ -144,35 +155,38 @@ __device__ __forceinline__ void solve_projected_dd(float2* c, int a, int nrot, c
   __syncwarp();
 }
 
-// SUB: sub-blocks of a CTA, each with its own half of the slice (SUB = 2: the
-// sums then have the bits of twice as many CTAs of half the threads, whose
-// FP32 sums stop at the CTA).  REG: every system of the launch fills its CTAs
-// (N = CS EPT NT) and its columns divide a sub-block's threads, so that all of
-// a thread's points share one row j: two neighbour flags per thread instead of
-// four bits per point, no guards, and zero halo columns beside the grid (66
-// against 89 instructions per point and step; the launcher decides).
-template <int EPT, int NT, int CS, int MINB, int SUB, bool REG>
+// HALF: a thread's EPT points in two halves, each with its own FP32 sums, so
+// that a sum has the bits of twice as many threads (HALF = 1: even and odd k)
+// or CTAs (HALF = 2: the two halves of the slice) with EPT / 2 points each;
+// 0: one chain.  REG: every system of the launch fills its CTAs (N = CS EPT
+// NT) and its columns divide the CTA's threads, so that all of a thread's
+// points share one row j: two neighbour flags per thread instead of four bits
+// per point, no guards, and zero halo columns beside the grid (the launcher
+// decides).
+template <int EPT, int NT, int CS, int MINB, int HALF, bool REG>
 __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams p) {
   namespace cg = cooperative_groups;
-  constexpr int NS = NT / SUB;                   // threads of a sub-block
-  constexpr int VC = CS * SUB;                   // sub-blocks of a system
-  constexpr int P = (NS / 32) * VC;              // per-warp partials of one value
-  constexpr int PL = P < 32 ? P : 32;            // lanes that add them
+  constexpr int NH = HALF ? 2 : 1;
+  constexpr int NWS = NT / 32 * (HALF == 1 ? 2 : 1);   // warps (HALF 1: half-warps' worth) of FP32 partials
+  constexpr int VC = CS * (HALF == 2 ? 2 : 1);   // blocks above them, added in double-float
+  constexpr int P = NWS * VC;                    // partials of one value
+  // four lanes add a value's partials: the lanes take blocks (VC >= 4), a
+  // block bit and a warp bit (2), or two warp bits (1)
+  constexpr int VL = VC >= 4 ? VC / 4 : 1;       // blocks in a lane
+  constexpr int NWL = P / 4 / VL;                // warps of each in a lane
   constexpr bool HALO = CS > 1 || REG;
-  static_assert(EPT <= 8, "the neighbour bits of a thread fill one word");
   extern __shared__ __align__(16) unsigned char smem_mx[];
   cg::cluster_group cluster = cg::this_cluster();
   const int rank = CS > 1 ? (int)cluster.block_rank() : 0;
   const int m = p.m;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int sub = SUB > 1 ? tid / NS : 0, st = SUB > 1 ? tid % NS : tid;
   // shared-memory carve (identical offsets in every CTA of the cluster);
   // gmres_mixed_smem_bytes counts the same pieces
   float2* cs = reinterpret_cast<float2*>(smem_mx);            // [m]
   float2* sn = cs + m;                                        // [m]
   float2* rinv = sn + m;                                      // [m]
-  float2* gv = rinv + m;                                      // [m + 1]
-  float2* hball = gv + m + 1;                                 // [NT / 32][kMaxV] sums, a copy per warp
+  float2* gv = rinv + m;                                      // [m + 2]
+  float2* hball = gv + m + 2;                                 // [NT / 32][kMaxV] sums, a copy per warp
   float2* hb = hball + warp * kMaxV;
   float* red = reinterpret_cast<float*>(hball + (NT / 32) * kMaxV);   // [2][kRedV][P]
   float* yf = red + 2 * kRedV * P;                            // [kMaxV] combination coefficients
@@ -181,11 +195,11 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
   float2* Hr = reinterpret_cast<float2*>(whalo + 4 * p.hmax); // packed columns of R: j at j (j + 1) / 2
   float* V = reinterpret_cast<float*>(Hr + m * (m + 1) / 2);  // [S][vld]
   const int vld = p.vld;
-  // workspace of this CTA: x (hi, lo) over the extended slice, the low parts
-  // of q_x, q_y, then the Krylov vectors past the shared-memory window
+  // workspace of this CTA: x (hi, lo) over the extended slice, q_x and q_y
+  // (hi, lo each), then the Krylov vectors past the shared-memory window
   float2* xs = reinterpret_cast<float2*>(p.spill32 + (size_t)blockIdx.x * p.ws_ld);
-  float2* ql = xs + vld;
-  float* Vg = reinterpret_cast<float*>(ql + EPT * NT);
+  float4* qc = reinterpret_cast<float4*>(xs + vld + (vld & 1));
+  float* Vg = reinterpret_cast<float*>(qc + EPT * NT);
   auto slot = [&](int i) -> float* {
     return i < p.S ? V + (size_t)i * vld : Vg + (size_t)(i - p.S) * vld;
   };
@@ -202,14 +216,16 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
     const SysDesc d = p.sys[sysi];
     const int H = d.H, W = d.W, N = H * W;
     const int SL = N / CS;                       // slice length (whole columns)
-    const int SH = SL / SUB;                     // a sub-block's part
+    const int SH = SL / 2;                       // its halves (HALF = 2)
     const int base = rank * SL;
     const int hal = HALO ? H : 0;                // halo columns before and after the slice
-    const int l0 = sub * SH + st;                // this thread's points l0 + k NS of the slice
-    auto inside = [&](int k) { return REG || st + k * NS < SH; };
+    // this thread's point k of the slice, whether it lies inside, its chain
+    auto lp = [&](int k) { return !REG && HALF == 2 && k >= EPT / 2 ? SH + tid + (k - EPT / 2) * NT : tid + k * NT; };
+    auto inside = [&](int k) { return REG || (HALF == 2 ? tid + (k % (EPT / 2)) * NT < SH : tid + k * NT < SL); };
+    auto chain = [](int k) { return HALF == 1 ? k & 1 : HALF == 2 ? (k >= EPT / 2) : 0; };
     // points past the slice (w = 0 there): on one CTA their slots hold zeros;
     // on a cluster that space is the halo's, so short slices are guarded
-    const bool full = REG || CS == 1 || SH == EPT * NS;
+    const bool full = REG || CS == 1 || SL == EPT * NT;
     // the operator constants c = g^2/(2h^2), e = c/4, c_d = 1/dt + 4c from the
     // descriptor's quotients: a division is a dozen FP64 instructions on
     // every warp.  Solved as (A / s) x = b / s with s = b_scale: the scale is
@@ -223,16 +239,26 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
     float* capV = capture ? p.capV32 + (size_t)cidx * (p.cap_a + 1) * p.cap_ld : nullptr;
     double* capH = capture ? p.capH + (size_t)cidx * (p.cap_a + 1) * p.cap_a : nullptr;
 
-    // fn(index in a vector slot, point of the grid or -1 outside) over this
-    // thread's points of the slice and of its halo columns
-    auto each_ext = [&](auto&& fn) {
+    // put(at, get(at, pp)) over this thread's points of the slice and of its
+    // halo columns (at: index in a vector slot, pp: point of the grid or -1
+    // outside), values read in groups ahead of their stores
+    // (rolled: see the residual below)
+    auto each_ext = [&](auto&& get, auto&& put) {
+      constexpr int B = !REG ? 2 : EPT < 8 ? EPT : 8;
+#pragma unroll 1
+      for (int k0 = 0; k0 < EPT; k0 += B) {
+        dd v[B];
 #pragma unroll
-      for (int k = 0; k < EPT; ++k)
-        if (inside(k)) fn(hal + l0 + k * NS, base + l0 + k * NS);
+        for (int u = 0; u < B; ++u)
+          if (inside(k0 + u)) v[u] = get(hal + lp(k0 + u), base + lp(k0 + u));
+#pragma unroll
+        for (int u = 0; u < B; ++u)
+          if (inside(k0 + u)) put(hal + lp(k0 + u), v[u]);
+      }
       if (CS > 1)
         for (int q = tid; q < 2 * H; q += NT) {
-          const int pp = q < H ? base - H + q : base + SL + q - H;
-          fn(q < H ? q : SL + q, (unsigned)pp < (unsigned)N ? pp : -1);
+          const int pp = q < H ? base - H + q : base + SL + q - H, at = q < H ? q : SL + q;
+          put(at, get(at, (unsigned)pp < (unsigned)N ? pp : -1));
         }
     };
     // x (hi, lo) lives in the workspace and, outside the Krylov phases, in the
@@ -246,15 +272,15 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
     };
     // x = u + yf-combination of the nc rows U (indexed by grid point)
     auto add_basis = [&](const float* U, int nc, bool from_zero) {
-      each_ext([&](int at, int pp) {
+      each_ext([&](int at, int pp) -> dd {
         float xv = 0.f;
         if (pp >= 0)
           for (int i = 0; i < nc; ++i) xv = fmaf(yf[i], U[(size_t)i * p.slot_ld + pp], xv);
-        put_x(at, from_zero ? dd{xv, 0.f} : dd_add_f(dd{xh[at], xl[at]}, xv));
-      });
+        return from_zero ? dd{xv, 0.f} : dd_add_f(dd{xh[at], xl[at]}, xv);
+      }, put_x);
     };
     auto load_x = [&](const double* src) {
-      each_ext([&](int at, int pp) { put_x(at, src && pp >= 0 ? dd_from_double(src[pp]) : dd{0.f, 0.f}); });
+      each_ext([&](int, int pp) -> dd { return src && pp >= 0 ? dd_from_double(src[pp]) : dd{0.f, 0.f}; }, put_x);
     };
     // zero columns beside the grid, in the shared-memory slots (REG on one CTA)
     auto zero_halo = [&]() {
@@ -267,30 +293,31 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
 
     // neighbours of this thread's points: 1 E, 2 W, 4 N, 8 S per point (REG:
     // N and S of all its points).  With halo columns E and W are always there.
-    unsigned msk = 0;
+    unsigned long long msk = 0;
     if (REG) {
-      const int j = l0 % H;
+      const int j = tid % H;
       msk = (j + 1 < H ? 4u : 0u) | (j > 0 ? 8u : 0u);
     } else {
 #pragma unroll
       for (int k = 0; k < EPT; ++k)
         if (inside(k)) {
-          const int pp = base + l0 + k * NS;
+          const int pp = base + lp(k);
           const int i = pp / H, j = pp - i * H;
-          msk |= ((CS > 1 || i + 1 < W ? 1u : 0u) | (CS > 1 || i > 0 ? 2u : 0u) | (j + 1 < H ? 4u : 0u) |
-                  (j > 0 ? 8u : 0u)) << (4 * k);
+          msk |= (unsigned long long)((CS > 1 || i + 1 < W ? 1u : 0u) | (CS > 1 || i > 0 ? 2u : 0u) |
+                                      (j + 1 < H ? 4u : 0u) | (j > 0 ? 8u : 0u)) << (4 * k);
         }
     }
     const bool rN = msk & 4u, rS = msk & 8u;
-    auto nbE = [&](const float* v, int at, int k) { return REG || (msk & (1u << (4 * k))) ? v[at + H] : 0.f; };
-    auto nbW = [&](const float* v, int at, int k) { return REG || (msk & (2u << (4 * k))) ? v[at - H] : 0.f; };
+    auto nb = [&](int k, unsigned bit) { return ((unsigned)(msk >> (4 * k)) & bit) != 0u; };
+    auto nbE = [&](const float* v, int at, int k) { return REG || nb(k, 1u) ? v[at + H] : 0.f; };
+    auto nbW = [&](const float* v, int at, int k) { return REG || nb(k, 2u) ? v[at - H] : 0.f; };
     auto nbN = [&](const float* v, int at, int k) {
       if (REG) { const float t = v[at + 1]; return rN ? t : 0.f; }
-      return (msk & (4u << (4 * k))) ? v[at + 1] : 0.f;
+      return nb(k, 4u) ? v[at + 1] : 0.f;
     };
     auto nbS = [&](const float* v, int at, int k) {
       if (REG) { const float t = v[at - 1]; return rS ? t : 0.f; }
-      return (msk & (8u << (4 * k))) ? v[at - 1] : 0.f;
+      return nb(k, 8u) ? v[at - 1] : 0.f;
     };
 
     // the lagged field, then q_x, q_y (hi parts in registers for the Krylov
@@ -301,35 +328,48 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
     load_x(d.mt);
     if (CS == 1) __syncthreads();
     else cluster.sync();                         // (every CTA runs and its halo buffer is zero)
-    float qx[EPT], qy[EPT];
+    // (kA, kB): the pair u of this thread's points, one of each half where the
+    // sums keep two chains
+    auto kA = [](int u) { return HALF == 2 ? u : 2 * u; };
+    auto kB = [](int u) { return HALF == 2 ? u + EPT / 2 : 2 * u + 1; };
     {
       const dd eed = {0.25f * ccd.hi, 0.25f * ccd.lo};
       const dd i2hd = dd_from_double(d.ki);
-#pragma unroll
-      for (int k = 0; k < EPT; ++k) {
-        const int at = hal + l0 + k * NS;
-        qx[k] = qy[k] = 0.f;
-        if (inside(k)) {
-          const dd mE = {nbE(xh, at, k), nbE(xl, at, k)}, mW = {nbW(xh, at, k), nbW(xl, at, k)};
-          const dd mN = {nbN(xh, at, k), nbN(xl, at, k)}, mS = {nbS(xh, at, k), nbS(xl, at, k)};
-          dd x = dd_mul(eed, dd_sub(mW, mE)), y = dd_mul(eed, dd_sub(mS, mN));
-          const int pp = base + l0 + k * NS;
-          if (d.fx) x = dd_add(x, dd_mul(dd_from_double(d.fx[pp]), i2hd));
-          if (d.fy) y = dd_add(y, dd_mul(dd_from_double(d.fy[pp]), i2hd));
-          qx[k] = x.hi;
-          qy[k] = y.hi;
-          ql[l0 + k * NS] = make_float2(x.lo, y.lo);
-        }
+      auto coeff = [&](int k) -> float4 {
+        const int at = hal + lp(k);
+        const dd mE = {nbE(xh, at, k), nbE(xl, at, k)}, mW = {nbW(xh, at, k), nbW(xl, at, k)};
+        const dd mN = {nbN(xh, at, k), nbN(xl, at, k)}, mS = {nbS(xh, at, k), nbS(xl, at, k)};
+        dd x = dd_mul(eed, dd_sub(mW, mE)), y = dd_mul(eed, dd_sub(mS, mN));
+        const int pp = base + lp(k);
+        if (d.fx) x = dd_add(x, dd_mul(dd_from_double(d.fx[pp]), i2hd));
+        if (d.fy) y = dd_add(y, dd_mul(dd_from_double(d.fy[pp]), i2hd));
+        return make_float4(x.hi, x.lo, y.hi, y.lo);
+      };
+#pragma unroll 1
+      for (int u = 0; u < EPT / 2; ++u) {
+        const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+        const float4 a = inside(kA(u)) ? coeff(kA(u)) : z, b = inside(kB(u)) ? coeff(kB(u)) : z;
+        qc[tid + kA(u) * NT] = a;
+        qc[tid + kB(u) * NT] = b;
       }
+    }
+    float qx[EPT], qy[EPT];                      // the hi parts, for the Krylov operator
+#pragma unroll
+    for (int k = 0; k < EPT; ++k) {
+      const float4 q = qc[tid + k * NT];
+      qx[k] = q.x;
+      qy[k] = q.z;
     }
 
     float w[EPT];                                // r, then w = A v_j
-    float bb = 0.f, sw = 0.f;                    // this thread's part of ||b||^2, of the warm start's ||r||^2
-    auto sumsq = [&]() {
-      float s = 0.f;
+    float bb[NH], sw[NH];                        // this thread's part of ||b||^2, of the warm start's ||r||^2
 #pragma unroll
-      for (int k = 0; k < EPT; ++k) s = fmaf(w[k], w[k], s);
-      return s;
+    for (int h = 0; h < NH; ++h) bb[h] = sw[h] = 0.f;
+    auto sumsq = [&](float (&s)[NH]) {
+#pragma unroll
+      for (int h = 0; h < NH; ++h) s[h] = 0.f;
+#pragma unroll
+      for (int k = 0; k < EPT; ++k) s[chain(k)] = fmaf(w[k], w[k], s[chain(k)]);
     };
     // push this CTA's edge columns of w to the neighbours' halo buffers
     // (visible after the next cluster barrier)
@@ -339,52 +379,82 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
       float* wr = rank + 1 < CS ? cluster.map_shared_rank(whalo, rank + 1) + hbuf * 2 * p.hmax : nullptr;
 #pragma unroll
       for (int k = 0; k < EPT; ++k) {
-        const int l = l0 + k * NS;
+        const int l = lp(k);
         if (wl && inside(k) && l < H) wl[l] = w[k];
         if (wr && inside(k) && l >= SL - H) wr[l - (SL - H)] = w[k];
       }
     };
-    // sums over the system of nv values part(0..nv-1) -> hb[0..nv) of every
-    // warp of every CTA, identical bits; ends with __syncwarp
+    // sums over the system of nv values -> hb[0..nv) of every warp of every
+    // CTA, identical bits; part(i0, nv, a) gives this thread's chains of values
+    // i0 .. i0 + 3.  Ends with __syncwarp.
     auto reduce = [&](int nv, auto&& part) {
       for (int c0 = 0; c0 < nv; c0 += kRedV) {
         const int nc = min(kRedV, nv - c0);
         float* rb = red + buf * kRedV * P;
 #pragma unroll 1
         for (int i0 = 0; i0 < nc; i0 += 4) {
-          float a[4];
+          float a[NH][4];
           part(c0 + i0, nv, a);
-          const float s = warp_reduce4f(a, lane);
-          const int v = i0 + (lane >> 3);
-          const int q = (warp % (NS / 32)) * VC + rank * SUB + sub;
+          const float s = warp_reduce4f<NH>(a, lane);
+          // value v of this lane, one of the 8 / NH lanes that hold it, and
+          // where the four adding lanes expect it
+          const int v = i0 + (NH == 2 ? (lane >> 2) & 3 : lane >> 3), h = NH == 2 ? lane >> 4 : 0;
+          const int r0 = NH == 2 ? lane & 3 : lane & 7;
+          const int w = warp + (HALF == 1 ? h * (NT / 32) : 0), vc = HALF == 2 ? 2 * rank + h : rank;
+          const int la = VC >= 4 ? vc & 3 : VC == 2 ? vc * 2 + (w & 1) : w & 3;
+          const int wl = VC >= 4 ? w : VC == 2 ? w >> 1 : w >> 2;
+          const int at = ((v * 4 + la) * VL + (VC >= 4 ? vc >> 2 : 0)) * NWL + wl;
           if (v < nc) {
             if (CS == 1) {
-              if ((lane & 7) == 0) rb[v * P + q] = s;
+              if (r0 == 0) rb[at] = s;
             } else {
-              for (int r = lane & 7; r < CS; r += 8) cluster.map_shared_rank(rb, r)[v * P + q] = s;
+              for (int r = r0; r < CS; r += 8 / NH) cluster.map_shared_rank(rb, r)[at] = s;
             }
           }
         }
         if (CS == 1) __syncthreads();
         else cluster.sync();
 #pragma unroll 1
-        for (int i0 = 0; i0 < nc; i0 += 32 / PL) {
-          const int i = i0 + lane / PL, q = lane % PL;
+        for (int i0 = 0; i0 < nc; i0 += 8) {
+          const int i = i0 + (lane >> 2);
           float s = 0.f, e = 0.f;
           if (i < nc) {
-            s = rb[i * P + q];
-            if (P > 32) s += rb[i * P + (q + 32) % P];
+            const float* f = rb + (i * 4 + (lane & 3)) * VL * NWL;
+#pragma unroll
+            for (int u = 0; u < VL; ++u) {
+              float x[NWL];
+#pragma unroll
+              for (int n = 0; n < NWL; ++n) x[n] = f[u * NWL + n];
+#pragma unroll
+              for (int n = NWL / 2; n > 0; n /= 2)           // warps of a block: FP32
+#pragma unroll
+                for (int q = 0; q < n; ++q) x[q] += x[q + n];
+              if (u == 0) {
+                s = x[0];
+              } else {
+                const dd t = dd_two_sum(s, x[0]);
+                s = t.hi;
+                e += t.lo;
+              }
+            }
           }
-#pragma unroll
-          for (int o = PL / 2; o >= VC; o /= 2) s += __shfl_xor_sync(kFull, s, o);   // warps of a sub-block
-#pragma unroll
-          for (int o = VC / 2; o > 0; o /= 2) {                                      // sub-blocks
+          auto blocks = [&](int o) {                         // double-float butterfly
             const float so = __shfl_xor_sync(kFull, s, o), eo = __shfl_xor_sync(kFull, e, o);
             const dd t = dd_two_sum(s, so);
             s = t.hi;
             e = (e + eo) + t.lo;
+          };
+          if (VC >= 4) {
+            blocks(2);
+            blocks(1);
+          } else if (VC == 2) {
+            s += __shfl_xor_sync(kFull, s, 1);
+            blocks(2);
+          } else {
+            s += __shfl_xor_sync(kFull, s, 2);
+            s += __shfl_xor_sync(kFull, s, 1);
           }
-          if (q == 0 && i < nc) hb[c0 + i] = as_f2(dd_fast_two_sum(s, e));
+          if ((lane & 3) == 0 && i < nc) hb[c0 + i] = VC > 1 ? as_f2(dd_fast_two_sum(s, e)) : make_float2(s, 0.f);
         }
         buf ^= 1;
       }
@@ -408,9 +478,9 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
       if (p.gdelta) {
         const float sg = (float)(p.grho[sysi] * p.gmul);
         const float* dl = p.gdelta + (size_t)sysi * p.gdelta_ld;
-        each_ext([&](int at, int pp) {
-          put_x(at, pp >= 0 ? dd_add_f(dd_from_double(d.mt[pp]), sg * dl[pp]) : dd{0.f, 0.f});
-        });
+        each_ext([&](int, int pp) -> dd {
+          return pp >= 0 ? dd_add_f(dd_from_double(d.mt[pp]), sg * dl[pp]) : dd{0.f, 0.f};
+        }, put_x);
       } else {
         load_x(d.x);
       }
@@ -468,44 +538,63 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
     for (;;) {
       __syncthreads();                           // x complete for the stencil
       const bool no_x = phase == kProject || (p.x0_mode == X0_ZERO && outer == 0);
-      // w = b - A x in double-float: the hi parts of the terms are added by
-      // TwoSum and all low parts and errors in FP32; w is its FP32 value,
-      // which is all the Krylov process and the norms need (no_x: w = b)
+      // r = b - A x in double-float: the hi parts of the terms are added by
+      // TwoSum and all low parts and errors in FP32; the FP32 value of r,
+      // which is all the Krylov process and the norms need, goes through the
+      // third vector slot to w (no_x: r = b).  The loop is rolled, two points
+      // at a time with the next ones' b and q on their way: unrolled over a
+      // thread's points, this and the loops above were 70 KB of straight code
+      // and instruction fetch was the kernel's first stall (4.3 of 12 cycles
+      // between two instructions of a warp).
       {
-        float sb = 0.f;
+        float* rs = V + 2 * vld + hal;
         auto mul = [](float ah, float al, float bh, float bl) -> dd {   // a b, unnormalised
           const float t = __fmul_rn(ah, bh);
           return {t, fmaf(al, bh, fmaf(ah, bl, fmaf(ah, bh, -t)))};
         };
-#pragma unroll
-        for (int k = 0; k < EPT; ++k) {
-          const int at = hal + l0 + k * NS;
-          w[k] = 0.f;
-          if (inside(k)) {
-            const dd b = dd_from_double(d.b[base + l0 + k * NS]);
-            sb = fmaf(b.hi, b.hi, sb);
-            w[k] = b.hi;
-            if (!no_x) {
-              const float2 q = ql[l0 + k * NS];
-              const dd x = {xh[at], xl[at]};
-              const dd xE = {nbE(xh, at, k), nbE(xl, at, k)}, xW = {nbW(xh, at, k), nbW(xl, at, k)};
-              const dd xN = {nbN(xh, at, k), nbN(xl, at, k)}, xS = {nbS(xh, at, k), nbS(xl, at, k)};
-              const dd s1 = dd_two_sum(xE.hi, xW.hi), s2 = dd_two_sum(xN.hi, xS.hi), s = dd_two_sum(s1.hi, s2.hi);
-              const float sl_ = ((xE.lo + xW.lo) + (xN.lo + xS.lo)) + ((s1.lo + s2.lo) + s.lo);
-              const dd dx = dd_two_sum(xE.hi, -xW.hi), dy = dd_two_sum(xN.hi, -xS.hi);
-              const float dxl = dx.lo + (xE.lo - xW.lo), dyl = dy.lo + (xN.lo - xS.lo);
-              const dd t1 = mul(cdd.hi, cdd.lo, x.hi, x.lo), t2 = mul(ccd.hi, ccd.lo, s.hi, sl_);
-              const dd t3 = mul(qx[k], q.x, dx.hi, dxl), t4 = mul(qy[k], q.y, dy.hi, dyl);
-              const dd a1 = dd_two_sum(b.hi, -t1.hi), a2 = dd_two_sum(a1.hi, t2.hi);
-              const dd a3 = dd_two_sum(a2.hi, -t3.hi), a4 = dd_two_sum(a3.hi, -t4.hi);
-              w[k] = a4.hi + (((b.lo - t1.lo) + (t2.lo - t3.lo)) + ((a1.lo + a2.lo) + (a3.lo + a4.lo)) - t4.lo);
-            }
-          }
+        auto point = [&](int k, double bv, float4 q, float& sum) -> float {
+          const dd b = dd_from_double(bv);
+          sum = fmaf(b.hi, b.hi, sum);
+          if (no_x) return b.hi;
+          const int at = hal + lp(k);
+          const dd x = {xh[at], xl[at]};
+          const dd xE = {nbE(xh, at, k), nbE(xl, at, k)}, xW = {nbW(xh, at, k), nbW(xl, at, k)};
+          const dd xN = {nbN(xh, at, k), nbN(xl, at, k)}, xS = {nbS(xh, at, k), nbS(xl, at, k)};
+          const dd s1 = dd_two_sum(xE.hi, xW.hi), s2 = dd_two_sum(xN.hi, xS.hi), s = dd_two_sum(s1.hi, s2.hi);
+          const float sl_ = ((xE.lo + xW.lo) + (xN.lo + xS.lo)) + ((s1.lo + s2.lo) + s.lo);
+          const dd dx = dd_two_sum(xE.hi, -xW.hi), dy = dd_two_sum(xN.hi, -xS.hi);
+          const float dxl = dx.lo + (xE.lo - xW.lo), dyl = dy.lo + (xN.lo - xS.lo);
+          const dd t1 = mul(cdd.hi, cdd.lo, x.hi, x.lo), t2 = mul(ccd.hi, ccd.lo, s.hi, sl_);
+          const dd t3 = mul(q.x, q.y, dx.hi, dxl), t4 = mul(q.z, q.w, dy.hi, dyl);
+          const dd a1 = dd_two_sum(b.hi, -t1.hi), a2 = dd_two_sum(a1.hi, t2.hi);
+          const dd a3 = dd_two_sum(a2.hi, -t3.hi), a4 = dd_two_sum(a3.hi, -t4.hi);
+          return a4.hi + (((b.lo - t1.lo) + (t2.lo - t3.lo)) + ((a1.lo + a2.lo) + (a3.lo + a4.lo)) - t4.lo);
+        };
+        float sA = 0.f, sB = 0.f;
+        double bA = 0.0, bB = 0.0;
+        float4 qA, qB;
+        auto fetch = [&](int u) {
+          if (inside(kA(u))) { bA = d.b[base + lp(kA(u))]; qA = qc[tid + kA(u) * NT]; }
+          if (inside(kB(u))) { bB = d.b[base + lp(kB(u))]; qB = qc[tid + kB(u) * NT]; }
+        };
+        fetch(0);
+#pragma unroll 1
+        for (int u = 0; u < EPT / 2; ++u) {
+          const double cA = bA, cB = bB;
+          const float4 eA = qA, eB = qB;
+          if (u + 1 < EPT / 2) fetch(u + 1);
+          const float r0 = inside(kA(u)) ? point(kA(u), cA, eA, sA) : 0.f;
+          const float r1 = inside(kB(u)) ? point(kB(u), cB, eB, HALF ? sB : sA) : 0.f;
+          if (full || inside(kA(u))) rs[lp(kA(u))] = r0;
+          if (full || inside(kB(u))) rs[lp(kB(u))] = r1;
         }
-        bb = sb;
+        bb[0] = sA;
+        if (HALF) bb[NH - 1] = sB;
+#pragma unroll
+        for (int k = 0; k < EPT; ++k) w[k] = full || inside(k) ? rs[lp(k)] : 0.f;
       }
       if (phase == kWarm) {
-        sw = sumsq();
+        sumsq(sw);
         __syncthreads();                         // every read of the warm start in the slots is done
         load_guess();
         phase = kGuess;
@@ -514,11 +603,16 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
       bool project = phase == kProject;
       if (!project) {
         push_edges();
-        reduce(first_norm ? 3 : 1, [&](int, int, float (&a)[4]) {
-          a[0] = sumsq();
-          a[1] = bb;
-          a[2] = sw;
-          a[3] = 0.f;
+        reduce(first_norm ? 3 : 1, [&](int, int, float (&a)[NH][4]) {
+          float s[NH];
+          sumsq(s);
+#pragma unroll
+          for (int h = 0; h < NH; ++h) {
+            a[h][0] = s[h];
+            a[h][1] = bb[h];
+            a[h][2] = sw[h];
+            a[h][3] = 0.f;
+          }
         });
         if (phase == kGuess) {
           // the judge of a given guess (the learned one): its true residual
@@ -545,15 +639,16 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
             __syncwarp();
           }
         } else {
-          reduce(nv, [&](int i0, int n, float (&s)[4]) {
+          reduce(nv, [&](int i0, int n, float (&s)[NH][4]) {
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-              s[u] = 0.f;
+#pragma unroll
+              for (int h = 0; h < NH; ++h) s[h][u] = 0.f;
               if (i0 + u < n) {
-                const float* ui = U + (size_t)(i0 + u) * p.slot_ld + base + l0;
+                const float* ui = U + (size_t)(i0 + u) * p.slot_ld + base;
 #pragma unroll
                 for (int k = 0; k < EPT; ++k)
-                  if (inside(k)) s[u] = fmaf(ui[k * NS], w[k], s[u]);
+                  if (inside(k)) s[chain(k)][u] = fmaf(ui[lp(k)], w[k], s[chain(k)][u]);
               }
             }
           });
@@ -597,7 +692,7 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
         const bool keep = capture && first && n <= p.cap_a;
 #pragma unroll
         for (int k = 0; k < EPT; ++k) {
-          const int l = l0 + k * NS;
+          const int l = lp(k);
           const float v = w[k] * scale;
           if (full || inside(k)) vn[hal + l] = v;
           if (keep && inside(k)) {
@@ -624,7 +719,7 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
           auto apply = [&](const float* v) {
 #pragma unroll
             for (int k = 0; k < EPT; ++k) {
-              const int at = hal + l0 + k * NS;
+              const int at = hal + lp(k);
               float xE = 0.f, xW = 0.f, xN = 0.f, xS = 0.f;
               if (full || inside(k)) {
                 xE = nbE(v, at, k);
@@ -649,28 +744,39 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
         // only measures the norm, after a large correction in pass 1
 #pragma unroll 1
         for (int pass = 0;; ++pass) {
-          reduce(nh + 1, [&](int i0, int n, float (&s)[4]) {
+          reduce(nh + 1, [&](int i0, int n, float (&s)[NH][4]) {
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-              s[u] = 0.f;
+#pragma unroll
+              for (int h = 0; h < NH; ++h) s[h][u] = 0.f;
               const int i = i0 + u;
               if (i < n - 1) {
                 auto dot = [&](const float* vi) {
 #pragma unroll
                   for (int k = 0; k < EPT; ++k)
-                    if (full || inside(k)) s[u] = fmaf(vi[k * NS], w[k], s[u]);
+                    if (full || inside(k)) s[chain(k)][u] = fmaf(vi[lp(k)], w[k], s[chain(k)][u]);
                 };
-                if (i < p.S) dot(V + (size_t)i * vld + hal + l0);
-                else dot(Vg + (size_t)(i - p.S) * vld + hal + l0);
+                if (i < p.S) dot(V + (size_t)i * vld + hal);
+                else dot(Vg + (size_t)(i - p.S) * vld + hal);
               } else if (i == n - 1) {
-                s[u] = sumsq();
+                float q[NH];
+                sumsq(q);
+#pragma unroll
+                for (int h = 0; h < NH; ++h) s[h][u] = q[h];
               }
             }
           });
           const dd ww = as_dd(hb[nh]);
           if (pass == 2) { hn2 = ww; break; }
-          dd sq = {0.f, 0.f};                    // sum of the squared coefficients
-          for (int i = 0; i < nh; ++i) sq = dd_add(sq, dd_mul(as_dd(hb[i]), as_dd(hb[i])));
+          float sqh = 0.f, sql = 0.f;            // sum of the squared coefficients
+          for (int i = 0; i < nh; ++i) {
+            const float2 h = hb[i];
+            const float t = __fmul_rn(h.x, h.x);
+            const dd a = dd_two_sum(sqh, t);
+            sqh = a.hi;
+            sql += a.lo + fmaf(2.f * h.x, h.y, fmaf(h.x, h.x, -t));
+          }
+          const dd sq = dd_fast_two_sum(sqh, sql);
           hn2 = dd_sub(ww, sq);
           if (warp == 0)
             for (int i = lane; i < nh; i += 32) col[i] = pass ? as_f2(dd_add(as_dd(col[i]), as_dd(hb[i]))) : hb[i];
@@ -681,10 +787,10 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
             auto sub_ = [&](const float* vi) {
 #pragma unroll
               for (int k = 0; k < EPT; ++k)
-                if (full || inside(k)) w[k] = fmaf(-hi, vi[k * NS], w[k]);
+                if (full || inside(k)) w[k] = fmaf(-hi, vi[lp(k)], w[k]);
             };
-            if (i < p.S) sub_(V + (size_t)i * vld + hal + l0);
-            else sub_(Vg + (size_t)(i - p.S) * vld + hal + l0);
+            if (i < p.S) sub_(V + (size_t)i * vld + hal);
+            else sub_(Vg + (size_t)(i - p.S) * vld + hal);
           }
           if (CS > 1)
             for (int q = tid; q < 2 * H; q += NT) {
@@ -795,12 +901,12 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
       __syncthreads();
       // d = V y in FP32, x += d in double-float; x goes to the first two slots
       // (each thread has read its own points of every vector by then)
-      each_ext([&](int at, int) {
+      each_ext([&](int at, int) -> dd {
         const dd x = as_dd(xs[at]);
         float dv = 0.f;
         for (int i = 0; i < kdone; ++i) dv = fmaf(yf[i], slot(i)[at], dv);
-        put_x(at, dd_add_f(x, dv));
-      });
+        return dd_add_f(x, dv);
+      }, put_x);
       ++outer;
     }
     if (capture && outer == 0 && tid == 0 && rank == 0) {
@@ -819,10 +925,10 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
     }
     // (the loop ends with x in the first two slots: every exit follows a
     // residual of x, or x0 = 0 put there)
-#pragma unroll
+#pragma unroll 4
     for (int k = 0; k < EPT; ++k)
       if (inside(k)) {
-        const int at = hal + l0 + k * NS, pp = base + l0 + k * NS;
+        const int at = hal + lp(k), pp = base + lp(k);
         const dd x = {xh[at], xl[at]};
         d.x[pp] = dd_to_double(x);
         if (p.bnext) p.bnext[(size_t)sysi * p.bnext_ld + pp] = __float2bfloat16_rn(x.hi);
@@ -861,9 +967,9 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
   if (CS > 1) cluster.sync();                    // no CTA leaves while others write its memory
 }
 
-template <int EPT, int NT, int CS, int MINB, int SUB, bool REG>
+template <int EPT, int NT, int CS, int MINB, int HALF, bool REG>
 cudaError_t launch_mx(const GmresParams& p, size_t smem, cudaStream_t st) {
-  auto k = gmres_mixed_kernel<EPT, NT, CS, MINB, SUB, REG>;
+  auto k = gmres_mixed_kernel<EPT, NT, CS, MINB, HALF, REG>;
   int dev = 0, optin = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
