@@ -130,8 +130,8 @@ __device__ __forceinline__ dd step_residual(dd C, dd E, dd W, dd N, dd S, dd c, 
 // by strip of columns (five splits per point straight from memory and sums
 // renormalised at every step were 300 instructions per point: 95 us for 512
 // planes of 128x128).  Columns too long for a strip are read directly.
-constexpr int kRmsThreads = 1024;
-constexpr int kRmsStrip = 8192;                    // points of a strip and the columns beside it
+constexpr int kRmsThreads = 512;
+constexpr int kRmsStrip = 4096;                    // points of a strip and the columns beside it
 constexpr size_t kRmsSmem = kRmsStrip * sizeof(float2);
 
 __global__ void __launch_bounds__(kRmsThreads) step_residual_rms_kernel(const double* const* m, int H, int W, double g2v,
@@ -139,7 +139,7 @@ __global__ void __launch_bounds__(kRmsThreads) step_residual_rms_kernel(const do
                                                                         int step_offset, double* rho, float* rout,
                                                                         size_t rld) {
   extern __shared__ float2 strip[];
-  __shared__ double red[32];
+  __shared__ double red[kRmsThreads / 32];
   const int b = blockIdx.x, P = H * W;
   const double g2 = g2s ? g2s[*step + step_offset] : g2v;
   const double hh = (double)H * (double)H;
@@ -158,14 +158,24 @@ __global__ void __launch_bounds__(kRmsThreads) step_residual_rms_kernel(const do
     for (int i0 = 0; i0 < W; i0 += cols) {
       const int nc = min(cols, W - i0);
       __syncthreads();
-      for (int q = threadIdx.x; q < (nc + 2) * H; q += kRmsThreads) {
-        const int p = (i0 - 1) * H + q;
-        const dd v = p >= 0 && p < P ? dd_from_double(mp[p]) : dd{0.f, 0.f};
-        strip[q] = make_float2(v.hi, v.lo);
+      {                                            // loads ahead of their splits
+        constexpr int L = kRmsStrip / kRmsThreads;
+        double v[L];
+#pragma unroll
+        for (int u = 0; u < L; ++u) {
+          const int q = threadIdx.x + u * kRmsThreads, p = (i0 - 1) * H + q;
+          v[u] = q < (nc + 2) * H && p >= 0 && p < P ? mp[p] : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < L; ++u) {
+          const dd x = dd_from_double(v[u]);
+          strip[threadIdx.x + u * kRmsThreads] = make_float2(x.hi, x.lo);
+        }
       }
       __syncthreads();
-      for (int q = H + threadIdx.x; q < (nc + 1) * H; q += kRmsThreads) {
-        const int j = q % H;
+      int j = threadIdx.x % H;                     // row of point q
+      const int dj = kRmsThreads % H;
+      for (int q = H + threadIdx.x; q < (nc + 1) * H; q += kRmsThreads, j += dj, j -= j >= H ? H : 0) {
         const float2 z = make_float2(0.f, 0.f);
         const float2 C = strip[q], E = strip[q + H], V = strip[q - H];
         const float2 N = j + 1 < H ? strip[q + 1] : z, S = j > 0 ? strip[q - 1] : z;
@@ -191,7 +201,7 @@ __global__ void __launch_bounds__(kRmsThreads) step_residual_rms_kernel(const do
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
   __syncthreads();
   if (threadIdx.x < 32) {
-    double t = red[threadIdx.x];
+    double t = threadIdx.x < kRmsThreads / 32 ? red[threadIdx.x] : 0.0;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
     if (threadIdx.x == 0) rho[b] = sqrt(t / P);
