@@ -90,6 +90,7 @@ kp_status gmres_shape(kp_ctx* c, int nmax, int m, Shape* out, bool mixed, int wm
     // have no such kernel
     sh.reg = one_size && nmax == sh.ctas() * npad && hmax > 0 && sh.nt % hmax == 0 && !c->opt.cluster_size && sh.nt == 256;
     sh.hmax = sh.cs || sh.reg ? hmax : 0;
+    if (sh.reg && sh.ept == 16 && !c->opt.cluster_blocks_per_sm) sh.minb = 3;
     sh.vld += 2 * sh.hmax;
   }
   auto bytes = [&](int S) {
@@ -235,7 +236,7 @@ kp_status run_gmres(kp_ctx* c, int nsys, const kp_op* ops, const double* const* 
   if (st != KP_OK) return st;
   cudaError_t e;
   if (sh.ws) {
-    const size_t need = (size_t)nsys * sh.ctas() * sh.ws * (mixed ? sizeof(float) : sizeof(double));
+    const size_t need = (mixed ? (size_t)sh.grid(nsys, c->sms) : (size_t)nsys) * sh.ws * (mixed ? sizeof(float) : sizeof(double));
     e = mixed ? grow(&c->spill32, &c->spill32_bytes, need) : grow(&c->spill, &c->spill_bytes, need);
     if (e != cudaSuccess) return kp::cuda_error(c, e, "cudaMalloc(Krylov workspace)");
   }
@@ -279,6 +280,8 @@ kp_status run_gmres(kp_ctx* c, int nsys, const kp_op* ops, const double* const* 
   p.x0_mode = kp::X0_READ;
   p.spill = (!mixed && sh.ws) ? c->spill : nullptr;
   p.spill32 = mixed ? c->spill32 : nullptr;
+  p.grid = mixed ? sh.grid(nsys, c->sms) : 0;
+  p.claim = c->claim;
   p.info = info;
   if (capture) {
     p.capV = c->capV;
@@ -362,6 +365,10 @@ kp_status kp_create(kp_ctx** out, const kp_options* opt, void* stream) {
     if (e == cudaSuccess)   // rows past a basis are read by the GEMM: keep them finite
       e = cudaMemset(c->slotVb, 0, (size_t)o.max_seeds * kp::kVbRows * c->vb_ld * sizeof(__nv_bfloat16));
   }
+  if (e == cudaSuccess && o.precision == KP_PREC_MIXED) {
+    e = cudaMalloc((void**)&c->claim, 2 * sizeof(int));
+    if (e == cudaSuccess) e = cudaMemset(c->claim, 0, 2 * sizeof(int));
+  }
   if (e == cudaSuccess) e = cudaMalloc((void**)&c->slotMeta, (size_t)o.max_seeds * sizeof(SlotMeta));
   if (e == cudaSuccess) e = cudaMalloc((void**)&c->slotR, (size_t)o.max_seeds * (a + 1) * a * sizeof(double));
   if (e == cudaSuccess) e = cudaMalloc((void**)&c->slotRot, (size_t)o.max_seeds * 3 * a * sizeof(double));
@@ -400,6 +407,7 @@ kp_status kp_destroy(kp_ctx* c) {
   cudaFree(c->slotVb);
   cudaFree(c->capV32);
   cudaFree(c->spill32);
+  cudaFree(c->claim);
   cudaFree(c->slotMeta);
   cudaFree(c->slotR);
   cudaFree(c->slotRot);

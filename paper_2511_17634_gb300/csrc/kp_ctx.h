@@ -3,6 +3,7 @@
 
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <vector>
 
 #include "kp.h"
@@ -64,6 +65,7 @@ struct kp_ctx {
   int* d_err = nullptr;               // device error flag of bounded waits
   float* spill32 = nullptr;
   size_t spill32_bytes = 0;
+  int* claim = nullptr;       // mixed precision: the solver's claim counters
   size_t spill_bytes = 0;
 };
 
@@ -84,6 +86,9 @@ struct Shape {
   int hmax = 0;   // longest column of the systems (mixed precision with halo columns)
   bool reg = false;   // mixed precision: see launch_gmres_mixed
   int ctas() const { return cs ? cs : 1; }
+  // mixed precision: CTAs of a launch over nsys systems (as many as are
+  // resident; they claim systems) and so slices of workspace
+  int grid(int nsys, int sms) const { return std::max(1, std::min(nsys, sms * minb / ctas())) * ctas(); }
 };
 
 kp_status set_error(kp_ctx* c, kp_status s, const char* fmt, ...);

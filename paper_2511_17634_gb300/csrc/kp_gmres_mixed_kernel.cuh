@@ -63,8 +63,8 @@ namespace kp {
 namespace {
 
 // Values per reduction round: longer Gram-Schmidt sums take several rounds
-// (and barriers), which keeps the partials of 32 warps within 4 KB.
-constexpr int kRedV = 16;
+// (and barriers), which keeps the partials of 64 warps within 4 KB (two sets).
+constexpr int kRedV = 8;
 
 __device__ __forceinline__ float2 as_f2(dd x) { return make_float2(x.hi, x.lo); }
 __device__ __forceinline__ dd as_dd(float2 x) { return {x.x, x.y}; }
@@ -212,7 +212,28 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
   const float kEta = p.inner_eta > 0.0 ? (float)p.inner_eta : 1e-5f;
   int buf = 0, hbuf = 0;                         // parities of the reductions and of the halo pushes
 
-  for (int sysi = blockIdx.x / CS; sysi < p.nsys; sysi += gridDim.x / CS) {
+  // resident CTAs claim systems until none is left: the workspace is then as
+  // large as the GPU holds CTAs and stays in L2 (a slice per system was 7 GB
+  // written back to memory per timestep of 12288 systems of 128x128)
+  // The next system is claimed while the current one's first residual runs and
+  // reaches the cluster's CTAs with that residual's sums.
+  auto tell_claim = [&](int sys) {
+    if (CS > 1) {
+#pragma unroll
+      for (int r = 0; r < CS; ++r) *cluster.map_shared_rank(fl + 4, r) = sys;
+    } else {
+      fl[4] = sys;
+    }
+  };
+  const bool claimer = rank == 0 && tid == 0;
+  if (CS > 1) cluster.sync();                    // every CTA of the cluster runs
+  if (claimer) tell_claim(atomicAdd(p.claim, 1));
+  if (CS > 1) cluster.sync();
+  else __syncthreads();
+#pragma unroll 1
+  for (;;) {
+    const int sysi = fl[4];
+    if (sysi >= p.nsys) break;                   // uniform over the cluster
     const SysDesc d = p.sys[sysi];
     const int H = d.H, W = d.W, N = H * W;
     const int SL = N / CS;                       // slice length (whole columns)
@@ -327,7 +348,9 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
     zero_halo();
     load_x(d.mt);
     if (CS == 1) __syncthreads();
-    else cluster.sync();                         // (every CTA runs and its halo buffer is zero)
+    else cluster.sync();                         // (every CTA's halo buffer is zero, and it has read its claim)
+    int next_sys = 0;
+    if (claimer) next_sys = atomicAdd(p.claim, 1);
     // (kA, kB): the pair u of this thread's points, one of each half where the
     // sums keep two chains
     auto kA = [](int u) { return HALF == 2 ? u : 2 * u; };
@@ -602,6 +625,7 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
       }
       bool project = phase == kProject;
       if (!project) {
+        if (claimer && first_norm) tell_claim(next_sys);
         push_edges();
         reduce(first_norm ? 3 : 1, [&](int, int, float (&a)[NH][4]) {
           float s[NH];
@@ -964,6 +988,10 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
     }
     __syncthreads();                             // shared memory is reused by the next system
   }
+  if (tid == 0 && rank == 0 && atomicAdd(p.claim + 1, 1) == (int)gridDim.x / CS - 1) {
+    p.claim[0] = 0;                              // the last to finish: ready for the next launch
+    p.claim[1] = 0;
+  }
   if (CS > 1) cluster.sync();                    // no CTA leaves while others write its memory
 }
 
@@ -979,7 +1007,7 @@ cudaError_t launch_mx(const GmresParams& p, size_t smem, cudaStream_t st) {
   if (e == cudaSuccess && CS > 8) e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(p.nsys * CS));
+  cfg.gridDim = dim3((unsigned)p.grid);
   cfg.blockDim = dim3(NT);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;

@@ -151,7 +151,8 @@ struct GmresParams {
   int wait_bias;            // testing aid: added to every awaited count (1: never released)
   int wait_limit;           // polls before a wait gives up; 0 = kWaitLimit
   int* err;                 // bit 1: a dependency wait gave up
-  int grid;                 // blocks of the launch (0 = one per system)
+  int grid;                 // blocks of the launch (FP64: 0 = one per system)
+  int* claim;               // mixed precision: {next system, clusters done}, both 0 between launches
   size_t score_stride;      // > 0: write the score of each solved timestep to
                             // d.score + tstep * score_stride and advance d.emb
   int picard;               // > 1: Picard iterations per system (FP64 solver)

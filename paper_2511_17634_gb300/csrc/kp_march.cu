@@ -59,6 +59,7 @@ struct kp_march_plan {
   kp::StepAcc* acc = nullptr;               // [T]
   double* spill = nullptr;
   float* spill32 = nullptr;
+  int* claim = nullptr;                     // mixed precision: claim counters, seeds then targets
   bool mixed = false;
   // targets are stored sorted by seed so that a seed's targets form whole
   // tensor-core tiles: internal plane q of group g holds user plane perm[q]
@@ -136,9 +137,13 @@ kp::GmresParams solver_params(kp_march_plan* P, bool seeds, int par, int offset,
   kp::set_shape(&g, sh);
   g.reorth = c->opt.reorth;
   g.inner_eta = kp::inner_eta(c->opt);
-  const size_t spS = P->ns ? (size_t)P->ns * P->shS.ctas() * P->shS.ws : 0;
+  const size_t spS = P->ns ? (size_t)(P->mixed ? P->shS.grid(P->ns, c->sms) : P->ns) * P->shS.ws : 0;
   if (P->mixed) g.spill32 = sh.ws ? P->spill32 + (seeds ? 0 : spS + tc.spill_off) : nullptr;
   else g.spill = sh.ws ? P->spill + (seeds ? 0 : spS + tc.spill_off) : nullptr;
+  if (P->mixed) {
+    g.grid = sh.grid(g.nsys, c->sms);
+    g.claim = P->claim + (seeds ? 0 : 2);
+  }
   g.slotV32 = c->slotV32;
   g.info = nullptr;
   g.step = P->step;
@@ -430,6 +435,7 @@ kp_status kp_march_destroy(kp_march_plan* P) {
   cudaFree(P->acc);
   cudaFree(P->spill);
   cudaFree(P->spill32);
+  cudaFree(P->claim);
   cudaFree(P->cyc_prev);
   cudaFree(P->slotM);
   cudaFree(P->cycV);
@@ -671,14 +677,19 @@ kp_status kp_march_create(kp_ctx* c, int ngroups, const kp_group* groups, const 
 
   // one Krylov workspace per branch: seed blocks first, then target blocks
   size_t spS = 0, spT = 0;
-  if (ns) spS = (size_t)ns * P->shS.ctas() * P->shS.ws;
+  auto slices = [&](const kp::Shape& sh, int n) { return (size_t)(P->mixed ? sh.grid(n, c->sms) : n) * sh.ws; };
+  if (ns) spS = slices(P->shS, ns);
   for (int ci = 0; ci < P->ncls; ++ci) {
     kp_march_plan::TClass& tc = P->cls[ci];
     tc.spill_off = spT;
-    spT += (size_t)tc.count * tc.sh.ctas() * tc.sh.ws;
+    if (tc.count) spT += slices(tc.sh, tc.count);
   }
   if (e == cudaSuccess && spS + spT) {
-    if (P->mixed) e = dmalloc(&P->spill32, spS + spT);
+    if (P->mixed) {
+      e = dmalloc(&P->spill32, spS + spT);
+      if (e == cudaSuccess) e = dmalloc(&P->claim, 4);
+      if (e == cudaSuccess) e = cudaMemset(P->claim, 0, 4 * sizeof(int));
+    }
     else e = dmalloc(&P->spill, spS + spT);
   }
   for (int k = 0; k < 2 && e == cudaSuccess; ++k) e = dmalloc(&P->desc[k], (size_t)ns + nt);
