@@ -42,7 +42,7 @@ cudaError_t launch_solver(const GmresParams& p, const Shape& sh, bool mixed, cud
 }
 
 kp_status gmres_shape(kp_ctx* c, int nmax, int m, Shape* out, bool mixed, int wmin, int hmax,
-                      bool one_size) {
+                      bool one_size, int count, bool one_launch) {
   Shape sh;
   sh.minb = 1;
   if (nmax <= 1024) {
@@ -54,6 +54,20 @@ kp_status gmres_shape(kp_ctx* c, int nmax, int m, Shape* out, bool mixed, int wm
     sh.ept = 1024 / sh.nt;
     sh.minb = c->opt.blocks_per_sm ? c->opt.blocks_per_sm : (sh.nt == 128 && !c->opt.block_threads ? 4
                                                              : sh.nt == 64 ? 4 : 2);
+    if (!mixed && !c->opt.block_threads && !c->opt.blocks_per_sm && count > 0) {
+      // Few systems leave SMs with one or two blocks, whose own latency then
+      // counts: the shapes with registers to spare (126 and 224 a thread, no
+      // spills) are faster there -- 28x28, 4 targets: 10.1 -> 8.1 ms for 50
+      // timesteps (256 x 4); 192 targets and 30 seeds of 32x32: 116 -> 97 ms
+      // for 100 (128 x 8, two blocks per SM; 256 x 4: 101).  A single launch
+      // of 768 systems fills 608 slots 1.26 times but 456 slots 1.68 times, two
+      // rounds of three blocks per SM instead of two of four: 0.55 -> 0.50 ms
+      // for one 32x32x3 step.
+      const int rounds3 = (count + 3 * c->sms - 1) / (3 * c->sms), rounds4 = (count + 4 * c->sms - 1) / (4 * c->sms);
+      if (count <= c->sms) { sh.nt = 256; sh.ept = 4; sh.minb = 2; }
+      else if (count <= 2 * c->sms) { sh.minb = 2; }
+      else if (one_launch && 3 * rounds3 < 4 * rounds4) { sh.nt = 256; sh.ept = 4; sh.minb = 3; }
+    }
     if (mixed) {                                 // the FP32 solver has the 256- and 128-thread shapes
       if (sh.nt == 64) { sh.nt = 128; sh.ept = 8; }
       sh.minb = 4;
@@ -232,7 +246,7 @@ kp_status run_gmres(kp_ctx* c, int nsys, const kp_op* ops, const double* const* 
     if ((long long)ops[k].H * ops[k].W != nmax)
       return kp::set_error(c, KP_ERR_UNSUPPORTED, "grids above 4096 unknowns must share one size per call");
   kp::Shape sh;
-  st = kp::gmres_shape(c, nmax, m, &sh, mixed, wmin, hmax, one_size);
+  st = kp::gmres_shape(c, nmax, m, &sh, mixed, wmin, hmax, one_size, nsys, true);
   if (st != KP_OK) return st;
   cudaError_t e;
   if (sh.ws) {

@@ -96,9 +96,10 @@ kp_status cuda_error(kp_ctx* c, cudaError_t e, const char* what);
 // Chooses threads, elements per thread and the shared-memory Krylov window
 // (FP64 vectors, or FP32 ones for the mixed-precision solver).  wmin, hmax:
 // narrowest and longest grid of the systems, one_size: they are all hmax x
-// (nmax / hmax) (mixed precision).
+// (nmax / hmax) (mixed precision).  count: systems solved at the same time (0:
+// many), one_launch: all of them by one launch of as many blocks (FP64).
 kp_status gmres_shape(kp_ctx* c, int nmax, int m, Shape* out, bool mixed = false,
-                      int wmin = 0, int hmax = 0, bool one_size = false);
+                      int wmin = 0, int hmax = 0, bool one_size = false, int count = 0, bool one_launch = false);
 // The shape's part of the solver parameters and the CTAs' workspace.
 inline void set_shape(GmresParams* p, const Shape& sh) {
   p->S = sh.S;
