@@ -727,7 +727,7 @@ def run_learned_march(args):
     solver_roof = {"bound": "alu", "achieved": sol_eq, "peak": FP32_PEAK_TFLOPS,
                    "unit": "TFLOP/s FP32-pipe equivalent (FP32 flops + 16 x double-float flops)",
                    "frac": sol_eq / FP32_PEAK_TFLOPS, "traffic": None,
-                   "kernel": "gmres_cluster_kernel (targets: judge, projection, refine)",
+                   "kernel": "gmres_mixed_kernel (targets: judge, projection, refine)",
                    "hp_tflops": hp_fl / sec / 1e12, "fp32_tflops": f32_fl / sec / 1e12,
                    "peak_source": ALU_PEAK_SOURCE}
     # the learned guess is bound by its activations' HBM traffic (each layer

@@ -57,7 +57,7 @@ typedef enum {
                         refinement whose solution, operator coefficients and
                         true residual b - A x are double-float (a pair of FP32
                         values, about 48 bits, on the FP32 pipe; FP64 in and
-                        out); FP64 Hessenberg and Givens; BF16 tensor-core
+                        out), as are Hessenberg and Givens; BF16 tensor-core
                         projection with FP32 accumulation */
 } kp_precision;
 
@@ -75,19 +75,24 @@ typedef struct {
                         1: second pass only when the first removed more than
                         half of the vector's norm (Daniel-Gragg-Kaufman-Stewart)  */
   int block_threads; /* threads per system for grids of <= 1024 points: 256 (4
-                        points per thread), 128 (8), 64 (16); 0 = 128 with 4
-                        blocks per SM (FP64) or 256 with 2 (mixed precision) */
+                        points per thread), 128 (8), 64 (16); 0 = by the number
+                        of systems (FP64: 256 with 2 blocks per SM up to one
+                        system per SM, 128 with 2 up to two, else 128 with 4, or
+                        256 with 3 where one call then leaves fewer slots
+                        empty) or 256 with 4 (mixed precision; 64 counts as
+                        128 there)                                           */
   int blocks_per_sm; /* resident solver blocks per SM for grids of <= 1024
                         points (caps registers per thread and sizes the
                         shared-memory window): 256 threads: 2 or 3; 128: 2, 3
                         or 4; 64: 4; 0 = the default above (2 for an explicit
-                        256 or 128, 4 for 64).  Mixed precision: 2 always.   */
+                        256 or 128, 4 for 64).  Mixed precision: 4 always.   */
   int cluster_size;  /* mixed precision, grids of 1025..16384 points: solve each
                         system on a cluster of this many CTAs (2, 4 or 8 of 256
                         threads, <= 2048 points per CTA; or 16 of 128 threads,
                         <= 1024 points per CTA -- a non-portable cluster size;
                         W divisible by it); 0 = clusters only above 4096 points
-                        (one 512-thread block below), of 2, 4 or 8 CTAs      */
+                        (one 256-thread block below), of 2 or 4 CTAs of
+                        <= 4096 points, W divisible by twice as many         */
   int fixed_a;       /* basis dimension of the seed solves (Sec. 3: V_a^n spans
                         the a-dimensional Krylov space; Sec. 5.2 uses a = 20):
                         0 = the first restart cycle ends when the seed meets its
@@ -102,8 +107,9 @@ typedef struct {
                         the iterative refinement recomputes the true
                         residual; 1..7, 0 = 5                                     */
   int cluster_blocks_per_sm; /* cluster solver (grids above 4096 points): resident
-                        CTAs per SM, 1 or 2 (16-CTA clusters: 2 or 4); 0 = 2
-                        (16-CTA clusters: 4) -- several systems share the SMs,
+                        CTAs per SM, 1 or 2 (16-CTA clusters: 2 or 4); 0 = 3
+                        where a slice fills its CTA, else 2 (16-CTA clusters:
+                        4) -- several systems share the SMs,
                         each with a smaller shared-memory window of Krylov
                         vectors                                                  */
 } kp_options;
@@ -268,8 +274,8 @@ kp_status kp_residual(kp_ctx* ctx, int nsys, const kp_op* ops, const double* con
  * Learned initial guess (not in the paper): a 3x3 convolutional network with
  * zero padding and ReLU between layers, trained on the GPU with this
  * library's kernels -- every convolution, its input gradient and its weight
- * gradient is a tcgen05 GEMM over im2col operands (BF16 inputs, FP32
- * accumulation); biases, ReLU, MSE loss and Adam (FP32 master weights, BF16
+ * gradient is a tcgen05 GEMM over im2col operands staged in shared memory (BF16
+ * inputs, FP32 accumulation); biases, ReLU, MSE loss and Adam (FP32 master weights, BF16
  * copies) are elementwise kernels.  Activations are FP32 planes
  * [batch][channels][H*W] in the solver's vector order.
  * Parameters (flat FP32): for each layer l, W_l [c_{l+1}][c_l][3][3] (tap

@@ -122,9 +122,8 @@ __device__ __forceinline__ dd step_residual(dd C, dd E, dd W, dd N, dd S, dd c, 
 // step_offset] when g2s is given (the march's schedule and counter).  The FP32
 // value of r goes to rout[b * rld + p] for the packing kernels.  The squares
 // are summed in double-float per thread; no FP64 instruction runs per point
-// (the FP64 pipe, not HBM, bounds this part on GB300).  Blocks of 1024
-// threads: with one block per plane, fewer and larger blocks keep the last
-// wave short (1536 planes are 5 waves of 2 blocks per SM, not 1.3 waves of 8).
+// (the FP64 pipe, not HBM, bounds this part on GB300).  One block of
+// 512 threads per plane, three to four of them per SM.
 //
 // The plane is split into double-float once per point, in shared memory, strip
 // by strip of columns (five splits per point straight from memory and sums

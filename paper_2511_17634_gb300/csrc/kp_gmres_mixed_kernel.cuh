@@ -39,11 +39,22 @@
 // pass) and one per residual.
 //
 // Memory.  Shared memory holds the first S Krylov vectors; the others, x and
-// the low parts of the coefficients live in a per-CTA device workspace (L2).
-// During a residual the first two vector slots hold x (hi, lo): the Krylov
-// vectors are dead by then.  Two 256-thread CTAs of 4096 points share an SM,
-// so that one system's barriers and serial work overlap the other's vector
-// work.
+// q_x, q_y (hi and lo) live in a device workspace per resident CTA (L2).
+// During a residual the first three vector slots hold x (hi, lo) and r: the
+// Krylov vectors are dead by then.  Resident CTAs (or clusters) claim system
+// after system, the next one during the first residual of the one before, so
+// neither the workspace nor the last wave grows with the number of systems.
+// REG: full CTAs whose threads divide into columns; a thread's points then lie
+// in one row, its neighbours at fixed offsets, and three CTAs of 4096 points
+// share an SM (two in general), so that one system's barriers and serial work
+// overlap the others' vector work.
+//
+// What bounds it now is issue and latency: 45 % of the issue slots are used.
+// Before (one CTA per SM, FP64 scalars, halos read across the cluster) eight
+// timesteps of 3072 channels of 64x64 took 16.5 ms, now 8.4; four of 128x128
+// 38.8, now 19.0.  16 points a thread rather than 8 took the instructions per
+// system from 235 to 170 thousand; the long loops stay rolled, since unrolled
+// code of that length stalled on instruction fetch (10.2 ms against 8.9).
 //
 // The operator is applied from q_x = f_x/(2h) - e (m~_E - m~_W) and q_y per
 // point:
