@@ -199,19 +199,30 @@ def test_network_gradients_exact_on_whole_numbers(kp, H, W, B, ch):
         assert np.abs(gb - rb).max() <= 2.0 ** -20 * 9 * e.size
 
 
-@pytest.mark.parametrize("H,W,B,ch", [(7, 5, 1, (3, 5)), (64, 3, 2, (10, 32)), (65, 9, 2, (17, 8)),
-                                      (128, 16, 1, (32, 31)), (130, 4, 1, (4, 2))])
-def test_network_last_layer_with_several_outputs(kp, H, W, B, ch):
+@pytest.mark.parametrize("H,W,B,ch", [
+    (65, 1, 1, (3, 5, 1)), (65, 9, 2, (16, 16, 1)), (96, 7, 1, (10, 17, 1)), (97, 8, 3, (2, 32, 1)),
+    (98, 17, 2, (10, 32, 32, 1)), (127, 10, 2, (9, 32, 17, 1)), (128, 16, 9, (10, 32, 32, 1)),
+    (128, 20, 1, (6, 16, 16, 1)), (7, 5, 1, (3, 5, 4)), (64, 3, 2, (10, 32, 16)), (65, 9, 2, (15, 8, 2)),
+    (100, 16, 1, (16, 32, 15)), (130, 4, 1, (4, 2, 3)), (129, 5, 2, (10, 32, 1))])
+def test_network_inference_exact_on_whole_numbers(kp, H, W, B, ch):
+    # the column-aligned kernel (64 < H <= 128: one row, part of and a whole warp
+    # of 32 rows past a warp's edge, one column, a super tile of 8 columns, one
+    # less and one more), the row-tiled one, and last layers of one and several
+    # outputs
     from oracle import cnn_oracle as R
     rng = np.random.default_rng(H + W)
-    w = rng.choice([-1.0, 0.0, 1.0], size=(ch[1], ch[0], 3, 3))
-    p = R.flatten([(w, rng.integers(-2, 3, size=ch[1]).astype(np.float64))])
+    w = [rng.choice([-1.0, 0.0, 1.0], p=[0.04, 0.9, 0.06], size=(co, ci, 3, 3)) for ci, co in zip(ch[:-1], ch[1:])]
+    for v in w:
+        v[:, 0] = rng.integers(-1, 2, size=v[:, 0].shape)
+    p = R.flatten([(v, rng.integers(-1, 2, size=v.shape[0]).astype(np.float64)) for v in w])
     x = rng.integers(0, 4, size=(B, ch[0], W, H)).astype(np.float64)
+    acts = R.forward(p, ch, x)
+    assert max(a.max() for a in acts[:-1]) <= 256
     net = kp.CNN(kp.Context(max_seeds=1, max_n=16384), H, W, channels=ch, max_batch=B)
     net.set_params(p)
     xin = torch.as_tensor(x.reshape(B, ch[0], -1), dtype=torch.float32, device="cuda")
-    out = torch.zeros((B, ch[1], H * W), dtype=torch.float32, device="cuda")
-    net.forward(xin, out)
+    out = torch.zeros((B, ch[-1], H * W), dtype=torch.float32, device="cuda")
+    for _ in range(2):                            # the second pass on buffers that the first one left
+        net.forward(xin, out)
     torch.cuda.synchronize()
-    ref = R.forward(p, ch, x)[-1]
-    assert np.array_equal(out.cpu().numpy().reshape(ref.shape), ref)
+    assert np.array_equal(out.cpu().numpy().reshape(acts[-1].shape), acts[-1])
