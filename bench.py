@@ -1110,7 +1110,7 @@ def bench_small(args, dist, init=False):
                          "unit": "TFLOP/s" if not mixed else
                                  "TFLOP/s FP32-pipe equivalent (FP32 flops + 16 x double-float flops)",
                          "frac": achieved_eq / peak_eq,
-                         "traffic": 23.81e6 if captured else None,
+                         "traffic": 23.38e6 if captured else None,
                          "traffic_note": ("DRAM bytes per target launch (16 timesteps x 768 systems), ncu "
                                           "capture of the first window; the path is L2-resident"
                                           if captured else "no ncu capture of this workload and shape"),
