@@ -22,11 +22,7 @@
 namespace {
 
 using kp::dd;
-using kp::dd_add;
-using kp::dd_add_f;
 using kp::dd_from_double;
-using kp::dd_mul;
-using kp::dd_sub;
 using kp::dd_to_double;
 using kp::f32_nearest;
 
