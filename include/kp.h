@@ -92,7 +92,8 @@ typedef struct {
                         <= 1024 points per CTA -- a non-portable cluster size;
                         W divisible by it); 0 = clusters only above 4096 points
                         (one 256-thread block below), of 2 or 4 CTAs of
-                        <= 4096 points, W divisible by twice as many         */
+                        <= 4096 points, W divisible by twice as many (or that
+                        many CTAs of <= 2048 points, by the number of systems) */
   int fixed_a;       /* basis dimension of the seed solves (Sec. 3: V_a^n spans
                         the a-dimensional Krylov space; Sec. 5.2 uses a = 20):
                         0 = the first restart cycle ends when the seed meets its

@@ -93,7 +93,25 @@ kp_status gmres_shape(kp_ctx* c, int nmax, int m, Shape* out, bool mixed, int wm
     sh.minb = c->opt.cluster_blocks_per_sm ? c->opt.cluster_blocks_per_sm : (sh.cs == 16 ? 4 : 2);
     if (sh.cs == 16 ? (sh.minb != 2 && sh.minb != 4) : sh.minb > 2)
       return set_error(c, KP_ERR_UNSUPPORTED, "cluster of %d CTAs: %d CTAs per SM not built", sh.cs, sh.minb);
-    if (!c->opt.cluster_size) { sh.cs /= 2; sh.ept = 16; }
+    if (!c->opt.cluster_size) {
+      // Few systems leave SMs idle and wait for their own latency: twice the
+      // CTAs of 2048 points each then (128x128: 30 systems 449 -> 340 us, 38
+      // 478 -> 578).  Without the register form the 8-point CTAs are also
+      // faster per round of a full chip, two rounds of them against one
+      // (101x80: 56 systems 480 -> 265 us, 100 528 -> 489, 165 987 -> 668;
+      // 152, one full round against three, 541 -> 672; 110x96: 300 systems
+      // 2492 -> 2210).  Two CTAs share an SM; larger clusters leave a tenth of
+      // the places empty.
+      const long long full = (long long)count * sh.cs;
+      auto rounds = [&](long long ctas, int cs) {
+        const long long slots = cs == 2 ? 2 * c->sms : 2 * c->sms * 9 / 10;
+        return (ctas + slots - 1) / slots;
+      };
+      const bool reg = one_size && nmax == sh.cs * 2048 && hmax > 0 && sh.nt % hmax == 0;
+      const bool more = count > 0 && !c->opt.cluster_blocks_per_sm &&
+                        (reg ? 2 * full <= 3 * c->sms : 5 * rounds(full, sh.cs) < 12 * rounds(full / 2, sh.cs / 2));
+      if (!more) { sh.cs /= 2; sh.ept = 16; }
+    }
   } else {
     return set_error(c, KP_ERR_UNSUPPORTED, "N=%d: FP64 grids above 4096 unknowns are not supported (use the mixed-precision mode)", nmax);
   }
@@ -102,7 +120,8 @@ kp_status gmres_shape(kp_ctx* c, int nmax, int m, Shape* out, bool mixed, int wm
   if (mixed) {
     // full CTAs, columns that divide the CTA's threads; the shapes on request
     // have no such kernel
-    sh.reg = one_size && nmax == sh.ctas() * npad && hmax > 0 && sh.nt % hmax == 0 && !c->opt.cluster_size && sh.nt == 256;
+    sh.reg = one_size && nmax == sh.ctas() * npad && hmax > 0 && sh.nt % hmax == 0 && !c->opt.cluster_size &&
+             sh.nt == 256 && (!sh.cs || sh.ept == 16);
     sh.hmax = sh.cs || sh.reg ? hmax : 0;
     if (sh.reg && sh.ept == 16 && !c->opt.cluster_blocks_per_sm) sh.minb = 3;
     sh.vld += 2 * sh.hmax;

@@ -121,6 +121,14 @@ def test_mixed_solver_sizes_and_more_systems_than_blocks(kp, orc, H, W, n):
     _solve_copies(kp, orc, H, W, n, kp.PREC_MIXED)
 
 
+@pytest.mark.parametrize("H,W,n", [(101, 80, 1), (101, 80, 136), (101, 80, 137), (101, 80, 152), (101, 80, 153),
+                                   (110, 96, 5), (110, 96, 68), (110, 96, 69), (128, 128, 28), (128, 128, 29),
+                                   (64, 128, 57), (64, 128, 58)])
+def test_cluster_shapes_by_number_of_systems(kp, orc, H, W, n):
+    # either side of each line between twice the CTAs and twice the points
+    _solve_copies(kp, orc, H, W, n, kp.PREC_MIXED)
+
+
 def test_mixed_solver_sizes_in_one_call(kp, orc):
     rng = np.random.default_rng(5)
     sizes = [(5, 3), (31, 33), (16, 64), (32, 32), (1, 1), (63, 64), (28, 28)]
