@@ -22,7 +22,10 @@
 namespace {
 
 using kp::dd;
+using kp::dd_add;
 using kp::dd_from_double;
+using kp::dd_mul;
+using kp::dd_sub;
 using kp::dd_to_double;
 using kp::f32_nearest;
 
@@ -98,20 +101,9 @@ __device__ __forceinline__ void split_hi_lo(float f, __nv_bfloat16& hi, __nv_bfl
 // FP32 pipe (kp_dd.cuh; about 2^-44 of c |m| absolute), the FP64 field split
 // without FP64 instructions.
 __device__ __forceinline__ dd step_residual(dd C, dd E, dd W, dd N, dd S, dd c, dd e) {
-  auto mul = [](float ah, float al, float bh, float bl) -> dd {   // a b, unnormalised
-    const float t = __fmul_rn(ah, bh);
-    return {t, fmaf(al, bh, fmaf(ah, bl, fmaf(ah, bh, -t)))};
-  };
-  const dd s1 = kp::dd_two_sum(E.hi, W.hi), s2 = kp::dd_two_sum(N.hi, S.hi), s = kp::dd_two_sum(s1.hi, s2.hi);
-  const dd l = kp::dd_two_sum(s.hi, -4.f * C.hi);
-  const float ll = (((E.lo + W.lo) + (N.lo + S.lo)) + ((s1.lo + s2.lo) + (s.lo + l.lo))) - 4.f * C.lo;
-  const dd dx = kp::dd_two_sum(E.hi, -W.hi), dy = kp::dd_two_sum(N.hi, -S.hi);
-  const float xl = dx.lo + (E.lo - W.lo), yl = dy.lo + (N.lo - S.lo);
-  const dd x2 = mul(dx.hi, xl, dx.hi, xl), y2 = mul(dy.hi, yl, dy.hi, yl);
-  const dd q = kp::dd_two_sum(x2.hi, y2.hi);
-  const dd t1 = mul(c.hi, c.lo, l.hi, ll), t2 = mul(e.hi, e.lo, q.hi, q.lo + (x2.lo + y2.lo));
-  const dd r = kp::dd_two_sum(t1.hi, t2.hi);
-  return kp::dd_fast_two_sum(r.hi, r.lo + (t1.lo + t2.lo));
+  const dd lap = dd_sub(dd_add(dd_add(E, W), dd_add(N, S)), dd{4.f * C.hi, 4.f * C.lo});
+  const dd dx = dd_sub(E, W), dy = dd_sub(N, S);
+  return dd_add(dd_mul(c, lap), dd_mul(e, dd_add(dd_mul(dx, dx), dd_mul(dy, dy))));
 }
 
 // rho_b = ||r_b|| / sqrt(P), one block per sample; g2 = g2v, or g2s[*step +
@@ -119,35 +111,38 @@ __device__ __forceinline__ dd step_residual(dd C, dd E, dd W, dd N, dd S, dd c, 
 // value of r goes to rout[b * rld + p] for the packing kernels.  The squares
 // are summed in double-float per thread; no FP64 instruction runs per point
 // (the FP64 pipe, not HBM, bounds this part on GB300).  One block of
-// 512 threads per plane, three to four of them per SM.
+// 512 threads per plane, three of them per SM.
 //
 // The plane is split into double-float once per point, in shared memory, strip
-// by strip of columns (five splits per point straight from memory and sums
-// renormalised at every step were 300 instructions per point: 95 us for 512
-// planes of 128x128).  Columns too long for a strip are read directly.
+// by strip of columns (five splits per point straight from memory were most of
+// the instructions: 95 us for 512 planes of 128x128).  Columns too long for a
+// strip are read directly.
+//
+// r and the sum of squares are normalised double-float operations in a fixed
+// order that does not depend on the strips (point p goes to sum p mod
+// kRmsSums, ascending, two sums a thread): an FP32 ulp of r or a rounding of
+// rho can tip a BF16 plane and, through an activation, single points of the
+// guess.  Sums that renormalise once at the end were twice as far off (1.1e-11
+// of rho against 5.2e-12) and 14 us faster (512 planes of 128x128, whole guess
+// 965 against 979 us).
 constexpr int kRmsThreads = 512;
+constexpr int kRmsSums = 1024;
 constexpr int kRmsStrip = 4096;                    // points of a strip and the columns beside it
 constexpr size_t kRmsSmem = kRmsStrip * sizeof(float2);
 
-__global__ void __launch_bounds__(kRmsThreads) step_residual_rms_kernel(const double* const* m, int H, int W, double g2v,
-                                                                        const double* g2s, const int* step,
-                                                                        int step_offset, double* rho, float* rout,
-                                                                        size_t rld) {
+__global__ void __launch_bounds__(kRmsThreads, 3) step_residual_rms_kernel(const double* const* m, int H, int W, double g2v,
+                                                                           const double* g2s, const int* step,
+                                                                           int step_offset, double* rho, float* rout,
+                                                                           size_t rld) {
   extern __shared__ float2 strip[];
-  __shared__ double red[kRmsThreads / 32];
-  const int b = blockIdx.x, P = H * W;
+  __shared__ double red[kRmsSums / 32];
+  const int b = blockIdx.x, P = H * W, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const double g2 = g2s ? g2s[*step + step_offset] : g2v;
   const double hh = (double)H * (double)H;
   const dd c = dd_from_double(0.5 * g2 * hh), e = dd_from_double(0.125 * g2 * hh);
   const double* mp = m[b];
   float* ro = rout + (size_t)b * rld;
-  float ah = 0.f, al = 0.f;                        // this thread's sum of r^2, unnormalised
-  auto add = [&](dd r) {
-    const float t = __fmul_rn(r.hi, r.hi), te = fmaf(2.f * r.hi, r.lo, fmaf(r.hi, r.hi, -t));
-    const dd s = kp::dd_two_sum(ah, t);
-    ah = s.hi;
-    al += s.lo + te;
-  };
+  dd acc[2] = {{0.f, 0.f}, {0.f, 0.f}};            // this thread's sums tid and tid + kRmsThreads
   const int cols = kRmsStrip / H - 2;              // columns of a strip
   if (cols >= 1) {
     for (int i0 = 0; i0 < W; i0 += cols) {
@@ -158,48 +153,69 @@ __global__ void __launch_bounds__(kRmsThreads) step_residual_rms_kernel(const do
         double v[L];
 #pragma unroll
         for (int u = 0; u < L; ++u) {
-          const int q = threadIdx.x + u * kRmsThreads, p = (i0 - 1) * H + q;
+          const int q = tid + u * kRmsThreads, p = (i0 - 1) * H + q;
           v[u] = q < (nc + 2) * H && p >= 0 && p < P ? mp[p] : 0.0;
         }
 #pragma unroll
         for (int u = 0; u < L; ++u) {
           const dd x = dd_from_double(v[u]);
-          strip[threadIdx.x + u * kRmsThreads] = make_float2(x.hi, x.lo);
+          strip[tid + u * kRmsThreads] = make_float2(x.hi, x.lo);
         }
       }
       __syncthreads();
-      int j = threadIdx.x % H;                     // row of point q
-      const int dj = kRmsThreads % H;
-      for (int q = H + threadIdx.x; q < (nc + 1) * H; q += kRmsThreads, j += dj, j -= j >= H ? H : 0) {
-        const float2 z = make_float2(0.f, 0.f);
-        const float2 C = strip[q], E = strip[q + H], V = strip[q - H];
-        const float2 N = j + 1 < H ? strip[q + 1] : z, S = j > 0 ? strip[q - 1] : z;
-        const dd r = step_residual({C.x, C.y}, {E.x, E.y}, {V.x, V.y}, {N.x, N.y}, {S.x, S.y}, c, e);
-        add(r);
-        ro[(i0 - 1) * H + q] = r.hi;
+      // points p0 <= p < p1; point p of the plane is at p - (i0 - 1) H of the strip
+      const int p0 = i0 * H, p1 = (i0 + nc) * H;
+      int j[2];                                    // row of point p
+      const int dj = kRmsSums % H, ps = p0 / kRmsSums * kRmsSums + tid;
+      j[0] = ps % H;
+      j[1] = (ps + kRmsThreads) % H;
+      for (int p = ps; p - tid < p1; p += kRmsSums) {
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          const int pp = p + u * kRmsThreads, q = pp - (i0 - 1) * H;
+          if (pp >= p0 && pp < p1) {
+            const float2 z = make_float2(0.f, 0.f);
+            const float2 C = strip[q], E = strip[q + H], V = strip[q - H];
+            const float2 N = j[u] + 1 < H ? strip[q + 1] : z, S = j[u] > 0 ? strip[q - 1] : z;
+            const dd r = step_residual({C.x, C.y}, {E.x, E.y}, {V.x, V.y}, {N.x, N.y}, {S.x, S.y}, c, e);
+            acc[u] = dd_add(acc[u], dd_mul(r, r));
+            ro[pp] = r.hi;
+          }
+          j[u] += dj;
+          j[u] -= j[u] >= H ? H : 0;
+        }
       }
     }
   } else {
     const dd z = {0.f, 0.f};
-    for (int p = threadIdx.x; p < P; p += kRmsThreads) {
-      const int i = p / H, j = p - i * H;
-      const dd r = step_residual(dd_from_double(mp[p]), i + 1 < W ? dd_from_double(mp[p + H]) : z,
-                                 i > 0 ? dd_from_double(mp[p - H]) : z, j + 1 < H ? dd_from_double(mp[p + 1]) : z,
-                                 j > 0 ? dd_from_double(mp[p - 1]) : z, c, e);
-      add(r);
-      ro[p] = r.hi;
+    for (int p = tid; p < P; p += kRmsSums) {
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int pp = p + u * kRmsThreads;
+        if (pp < P) {
+          const int i = pp / H, j = pp - i * H;
+          const dd r = step_residual(dd_from_double(mp[pp]), i + 1 < W ? dd_from_double(mp[pp + H]) : z,
+                                     i > 0 ? dd_from_double(mp[pp - H]) : z, j + 1 < H ? dd_from_double(mp[pp + 1]) : z,
+                                     j > 0 ? dd_from_double(mp[pp - 1]) : z, c, e);
+          acc[u] = dd_add(acc[u], dd_mul(r, r));
+          ro[pp] = r.hi;
+        }
+      }
     }
   }
-  double s = dd_to_double(kp::dd_fast_two_sum(ah, al));
+  // 32 neighbouring sums by halves, then the groups of 32 in order.  Half of a
+  // warp takes the one group and half the other after the first step.
+  const double s0 = dd_to_double(acc[0]), s1 = dd_to_double(acc[1]);
+  const bool up = lane & 16;
+  double s = (up ? s1 : s0) + __shfl_xor_sync(0xffffffffu, up ? s0 : s1, 16);
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+  for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if ((lane & 15) == 0) red[warp + (up ? kRmsThreads / 32 : 0)] = s;
   __syncthreads();
-  if (threadIdx.x < 32) {
-    double t = threadIdx.x < kRmsThreads / 32 ? red[threadIdx.x] : 0.0;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-    if (threadIdx.x == 0) rho[b] = sqrt(t / P);
+  if (tid == 0) {
+    double t = 0.0;
+    for (int w = 0; w < kRmsSums / 32; ++w) t += red[w];
+    rho[b] = sqrt(t / P);
   }
 }
 

@@ -1,0 +1,106 @@
+"""What callers rely on beyond the tolerances: arithmetic whose bits are part
+of the result, and the outcome of calls at the edges of what a solver accepts."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def kp():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2511_17634_gb300 import build
+    build.build()
+    from paper_2511_17634_gb300 import kp as K
+    return K
+
+
+def _dev(a):
+    return torch.as_tensor(np.ascontiguousarray(a, dtype=np.float64), device="cuda")
+
+
+# ---- double-float arithmetic (pairs of FP32 arrays) with FP32's own rounding
+
+def _fma(a, b, c):
+    """round32(a b + c): the FP64 sum of the exact product and c, rounded to odd
+    where it is inexact, so that the second rounding is the only one."""
+    p, c = a.astype(np.float64) * b.astype(np.float64), np.broadcast_to(c, a.shape).astype(np.float64)
+    s = p + c
+    t = s - p
+    e = (p - (s - t)) + (c - t)
+    odd = (s.view(np.int64) & 1) == 1
+    s = np.where((e != 0) & ~odd, np.nextafter(s, np.where(e > 0, np.inf, -np.inf)), s)
+    return s.astype(np.float32)
+
+
+def _fast_two_sum(a, b):
+    s = a + b
+    return s, b - (s - a)
+
+
+def _add(x, y):
+    s = x[0] + y[0]
+    t = s - x[0]
+    e = (x[0] - (s - t)) + (y[0] - t)
+    return _fast_two_sum(s, e + (x[1] + y[1]))
+
+
+def _sub(x, y):
+    return _add(x, (-y[0], -y[1]))
+
+
+def _mul(x, y):
+    p = x[0] * y[0]
+    return _fast_two_sum(p, _fma(x[1], y[0], _fma(x[0], y[1], _fma(x[0], y[0], -p))))
+
+
+def _split(v):
+    """FP64 -> hi (truncated to 24 bits) and lo (the rest, rounded)."""
+    hi = (np.asarray(v, dtype=np.float64).view(np.int64) & ~np.int64(0x1FFFFFFF)).view(np.float64)
+    return hi.astype(np.float32), (v - hi).astype(np.float32)
+
+
+def _rho(m, H, W, g2):
+    """Root mean square of the step's residual in double-float: point p in sum
+    p mod 1024, the sums by halves of 32 and then in order."""
+    f = np.zeros((W + 2, H + 2))
+    f[1:-1, 1:-1] = m.reshape(W, H)
+    f = _split(f)
+    at = lambda i, j: tuple(v[1 + i:1 + i + W, 1 + j:1 + j + H].reshape(-1) for v in f)
+    C, E, V, N, S = at(0, 0), at(1, 0), at(-1, 0), at(0, 1), at(0, -1)
+    hh = float(H) * float(H)
+    one = np.ones(H * W, np.float64)
+    c, e = _split(0.5 * g2 * hh * one), _split(0.125 * g2 * hh * one)
+    lap = _sub(_add(_add(E, V), _add(N, S)), (np.float32(4) * C[0], np.float32(4) * C[1]))
+    dx, dy = _sub(E, V), _sub(N, S)
+    r = _add(_mul(c, lap), _mul(e, _add(_mul(dx, dx), _mul(dy, dy))))
+    sq = _mul(r, r)
+    pad = -len(m) % 1024
+    sq = tuple(np.concatenate([v, np.zeros(pad, np.float32)]).reshape(-1, 1024) for v in sq)
+    acc = (np.zeros(1024, np.float32), np.zeros(1024, np.float32))
+    for k in range(sq[0].shape[0]):
+        acc = _add(acc, (sq[0][k], sq[1][k]))
+    s = (acc[0].astype(np.float64) + acc[1].astype(np.float64)).reshape(32, 32)
+    for o in (16, 8, 4, 2, 1):
+        s = s[:, :o] + s[:, o:2 * o]
+    t = 0.0
+    for v in s[:, 0]:
+        t += v
+    return np.sqrt(t / len(m))
+
+
+@pytest.mark.parametrize("H,W", [(128, 128), (33, 125), (24, 24), (7, 700), (1000, 5), (1366, 3), (1, 1500)])
+def test_step_residual_is_the_double_float_sequence(kp, H, W):
+    # the rms scale of the learned guess to the last bit: normalised
+    # double-float operations in a fixed order, whatever the strips are
+    rng = np.random.default_rng(H * 3 + W)
+    B, n, T, g2n = 3, 251, 1000, 0.0051
+    m = rng.uniform(0, 1, (B, H * W)) * 10.0 ** rng.integers(-3, 1, size=(B, H * W))
+    net = kp.CNN(kp.Context(max_seeds=1, max_n=16384), H, W, channels=(10, 1), max_batch=B)
+    out = torch.zeros((B, 10, H * W), dtype=torch.float32, device="cuda")
+    rho = torch.zeros(B, dtype=torch.float64, device="cuda")
+    net.pack_inputs(_dev(m), _dev(m), n, T, g2n, out, rho)
+    torch.cuda.synchronize()
+    assert np.array_equal(rho.cpu().numpy(), [_rho(v, H, W, g2n) for v in m])
