@@ -354,8 +354,11 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
 
     // the lagged field, then q_x, q_y (hi parts in registers for the Krylov
     // operator, low parts in the workspace for the residual)
-    if (CS > 1)
-      for (int q = tid; q < 4 * H; q += NT) whalo[q] = 0.f;
+    if (CS > 1) {
+      // (both buffers whole: nobody pushes the halo outside the grid, and a
+      // system before this one may have had longer columns)
+      for (int q = tid; q < 4 * p.hmax; q += NT) whalo[q] = 0.f;
+    }
     zero_halo();
     load_x(d.mt);
     if (CS == 1) __syncthreads();

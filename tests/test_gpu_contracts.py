@@ -104,3 +104,39 @@ def test_step_residual_is_the_double_float_sequence(kp, H, W):
     net.pack_inputs(_dev(m), _dev(m), n, T, g2n, out, rho)
     torch.cuda.synchronize()
     assert np.array_equal(rho.cpu().numpy(), [_rho(v, H, W, g2n) for v in m])
+
+
+# ---- clusters
+
+def _check_solution(orc, H, W, mt, b, x, tol):
+    # residual and solution as in the solver tests: 1e-9 for a relative
+    # residual of 1e-10 with cond <= 2.3
+    C = orc.coeffs(H, W, 0.02, 1e-3, 1.0 / H, mt)
+    assert np.linalg.norm(b - orc.apply(H, W, C, x)) <= 1.01 * tol * np.linalg.norm(b)
+    ref = orc.gmres(H, W, C, b, tol=1e-13, m=40, maxit=800).x
+    assert np.linalg.norm(x - ref) <= 1e-9 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("sizes,cluster,n", [
+    ([(64, 128), (128, 64)], 0, 420), ([(128, 128), (256, 64), (64, 256)], 0, 200),
+    ([(32, 64), (64, 32)], 2, 700), ([(64, 40), (24, 50), (50, 24), (3, 20)], 2, 700),
+    ([(40, 40), (24, 64), (96, 16)], 8, 300), ([(20, 64), (64, 48), (48, 16)], 16, 120)])
+def test_cluster_systems_of_different_column_lengths(kp, orc, sizes, cluster, n):
+    # columns shorter and longer than those of the system before, on the same
+    # cluster (more systems than clusters are resident): the halo outside the
+    # grid stays zero
+    rng = np.random.default_rng(n + cluster)
+    ctx = kp.Context(max_n=16384, precision=kp.PREC_MIXED, cluster_size=cluster)
+    data = [(H, W, rng.uniform(0, 1, H * W), rng.normal(size=H * W)) for H, W in sizes for _ in range(3)]
+    dev = [(kp.make_ops(H, W, 1e-3, 0.02, 1.0 / H, _dev(mt[None])), _dev(b)) for H, W, mt, b in data]
+    at = rng.permutation(np.arange(n) % len(data))
+    x = [torch.zeros_like(dev[k][1]) for k in at]
+    tol = 1e-10
+    info = ctx.refine(kp.Ops.concat([dev[k][0] for k in at]), [dev[k][1] for k in at], x, tol=tol, m=30, maxit=500)
+    _, st, rr = kp.decode_info(info)
+    torch.cuda.synchronize()
+    assert (st == 0).all() and (rr <= tol).all()
+    for k, (H, W, mt, b) in enumerate(data):
+        rows = torch.stack([x[s] for s in np.flatnonzero(at == k)])
+        assert bool((rows == rows[0]).all()), (H, W)
+        _check_solution(orc, H, W, mt, b, rows[0].cpu().numpy(), tol)
