@@ -267,6 +267,12 @@ kp_status run_gmres(kp_ctx* c, int nsys, const kp_op* ops, const double* const* 
   kp::Shape sh;
   st = kp::gmres_shape(c, nmax, m, &sh, mixed, wmin, hmax, one_size, nsys, true);
   if (st != KP_OK) return st;
+  // a slice is N / cs points (it may end inside a column: the halo then holds
+  // the north and south neighbours too), so every N has to be divisible; the
+  // points past the last whole slice would stay unsolved
+  for (int k = 0; k < nsys && sh.cs; ++k)
+    if ((ops[k].H * ops[k].W) % sh.cs)
+      return kp::set_error(c, KP_ERR_UNSUPPORTED, "system %d: %d x %d is not divisible into %d slices", k, ops[k].H, ops[k].W, sh.cs);
   cudaError_t e;
   if (sh.ws) {
     const size_t need = (mixed ? (size_t)sh.grid(nsys, c->sms) : (size_t)nsys) * sh.ws * (mixed ? sizeof(float) : sizeof(double));

@@ -140,3 +140,20 @@ def test_cluster_systems_of_different_column_lengths(kp, orc, sizes, cluster, n)
         rows = torch.stack([x[s] for s in np.flatnonzero(at == k)])
         assert bool((rows == rows[0]).all()), (H, W)
         _check_solution(orc, H, W, mt, b, rows[0].cpu().numpy(), tol)
+
+
+def test_cluster_call_refuses_what_its_slices_leave_out(kp, orc):
+    # the narrowest width decides the cluster: a wider system of an odd number
+    # of points is refused, one whose slices end inside a column is solved
+    rng = np.random.default_rng(3)
+    ctx = kp.Context(max_n=4096, precision=kp.PREC_MIXED, cluster_size=2)
+    sys_ = [(H, W, rng.uniform(0, 1, H * W), rng.normal(size=H * W)) for H, W in ((64, 32), (32, 33), (47, 40), (31, 33))]
+    dev = [(kp.make_ops(H, W, 1e-3, 0.02, 1.0 / H, _dev(mt[None])), _dev(b)) for H, W, mt, b in sys_]
+    x = [torch.zeros_like(b) for _, b in dev]
+    with pytest.raises(kp.KPError) as e:
+        ctx.refine(kp.Ops.concat([o for o, _ in dev]), [b for _, b in dev], x, tol=1e-10, m=30, maxit=500)
+    assert e.value.status == kp.ERR_UNSUPPORTED
+    info = ctx.refine(kp.Ops.concat([o for o, _ in dev[:3]]), [b for _, b in dev[:3]], x[:3], tol=1e-10, m=30, maxit=500)
+    assert (kp.decode_info(info)[1] == 0).all()
+    for (H, W, mt, b), v in zip(sys_[:3], x):
+        _check_solution(orc, H, W, mt, b, v.cpu().numpy(), 1e-10)
