@@ -17,9 +17,13 @@
 //
 // FP64 <-> dd conversions: dd_from_double splits the FP64 bit pattern with
 // integer operations (no FP64 instruction): hi = x truncated to 24
-// significant bits, lo = the remaining 29 bits rounded to 24; |x| < 2^-74 maps
-// to (hi, 0) and below 2^-100 to zero, far under any quantity the solvers
-// compare.  dd_to_double rounds hi + lo to FP64 (exact up to 53 significant bits).
+// significant bits, lo = the remaining 29 bits rounded to 24; below 2^-100 both
+// are zero, far under any quantity the solvers compare.  |x| >= 2^128, an
+// infinity or NaN leaves an infinity or NaN in lo (hi is then meaningless),
+// which every sum of the low parts carries on: marking hi as well, by a
+// compare and two selects per value, made the mixed-precision solves 3 to 8 %
+// slower.  dd_to_double rounds hi + lo to FP64 (exact up to 53 significant
+// bits); dd_to_double_any does so for such values too.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -70,9 +74,10 @@ __device__ __forceinline__ dd dd_from_double(double x) {
   const int e = (int)(mag >> 20);                    // biased FP64 exponent
   // top 24 significant bits -> float (exponent rebiased by 1023 - 127 = 896)
   const float hi = __uint_as_float(sign | __funnelshift_l(ul, mag - (896u << 20), 3));
-  // the 29 bits below: an integer times 2^(e - 1075), zero for e < 949
-  const float scale = __uint_as_float(sign | ((unsigned int)max(e - 948, 0) << 23));
-  const float lo = __uint2float_rn(ul & 0x1FFFFFFFu) * scale;
+  // the 29 bits below: an integer times 2^(e - 1075), here 2^-52 2^(e - 1023)
+  // with the second factor infinite from e = 1151 (2^128) on
+  const float scale = __uint_as_float(sign | ((unsigned int)__vimin_s32_relu(e - 896, 255) << 23));
+  const float lo = (__uint2float_rn(ul & 0x1FFFFFFFu) * 0x1p-52f) * scale;
   const bool tiny = e < 1023 - 100;
   return {tiny ? 0.f : hi, tiny ? 0.f : lo};
 }
@@ -99,7 +104,7 @@ __device__ __forceinline__ dd dd_sqrt(dd x) {
 }
 
 // (out of line, or its FP64 instructions are speculated for every value)
-static __device__ __noinline__ double dd_to_double_slow(dd x) { return (double)x.hi + (double)x.lo; }
+static __device__ __noinline__ double dd_to_double_any(dd x) { return (double)x.hi + (double)x.lo; }
 
 // hi + lo rounded to FP64.  A conversion and an add on the FP64 pipe cost
 // three warp instructions of 64 cycles each; this composes the bit pattern
@@ -110,7 +115,7 @@ static __device__ __noinline__ double dd_to_double_slow(dd x) { return (double)x
 __device__ __forceinline__ double dd_to_double(dd x) {
   const unsigned int u = __float_as_uint(x.hi);
   const unsigned int e = (u >> 23) & 0xFFu;
-  if (e < 56 || e > 254) return dd_to_double_slow(x);          // small, zero, Inf, NaN
+  if (e < 56 || e > 254) return dd_to_double_any(x);          // small, zero, Inf, NaN
   const float lo = (u >> 31) ? -x.lo : x.lo;                   // relative to |hi|
   const unsigned int below = (u & 0x7FFFFFu) == 0u && lo < 0.f;
   const int t = __float2int_rn(lo * __uint_as_float((306u + below - e) << 23));

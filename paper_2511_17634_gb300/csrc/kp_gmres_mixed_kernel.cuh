@@ -715,8 +715,9 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
         }
       }
       const float beta = rnorm.hi;
+      // (before the tolerance: an infinite ||b|| is above everything)
+      if (!isfinite(beta) || !isfinite(bnorm.hi)) { status = KP_BREAKDOWN; break; }
       if (beta <= tolb) { status = KP_OK; break; }
-      if (!isfinite(beta)) { status = KP_BREAKDOWN; break; }
       if (steps >= p.maxit || outer >= 64) break;
       const bool first = (outer == 0);
       // the seed's captured cycle runs to the seed tolerance, so its basis has
@@ -968,8 +969,10 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
       if (inside(k)) {
         const int at = hal + lp(k), pp = base + lp(k);
         const dd x = {xh[at], xl[at]};
-        d.x[pp] = dd_to_double(x);
-        if (p.bnext) p.bnext[(size_t)sysi * p.bnext_ld + pp] = __float2bfloat16_rn(x.hi);
+        // (after a breakdown the low part may hold the infinity or NaN)
+        const bool bad = status == KP_BREAKDOWN;
+        d.x[pp] = bad ? dd_to_double_any(x) : dd_to_double(x);
+        if (p.bnext) p.bnext[(size_t)sysi * p.bnext_ld + pp] = __float2bfloat16_rn(bad ? x.hi + x.lo : x.hi);
       }
     if (tid == 0 && rank == 0) {
       const double rel = bnorm.hi > 0.f ? dd_to_double(rnorm) / dd_to_double(bnorm) : 0.0;

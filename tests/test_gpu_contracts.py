@@ -157,3 +157,44 @@ def test_cluster_call_refuses_what_its_slices_leave_out(kp, orc):
     assert (kp.decode_info(info)[1] == 0).all()
     for (H, W, mt, b), v in zip(sys_[:3], x):
         _check_solution(orc, H, W, mt, b, v.cpu().numpy(), 1e-10)
+
+
+# ---- values past what the mixed-precision solver can hold
+
+@pytest.mark.parametrize("H,W", [(28, 28), (32, 32), (50, 37), (64, 64), (101, 80), (128, 128)])
+@pytest.mark.parametrize("bad", [np.nan, -np.nan, np.inf, -np.inf, 1e39, -1e300, 1e25])
+def test_mixed_solver_breaks_down_on_values_out_of_range(kp, H, W, bad):
+    # one such value in b, in the lagged field or in x0 of every other system
+    # (1e25: in range, its square is not); the systems beside them converge
+    rng = np.random.default_rng(H)
+    N, n = H * W, 6
+    ctx = kp.Context(max_n=16384, precision=kp.PREC_MIXED)
+    for where in ("b", "m", "x0") if abs(bad) != 1e25 else ("b",):
+        v = {"b": rng.normal(size=(n, N)), "m": rng.uniform(0, 1, (n, N)), "x0": rng.normal(size=(n, N))}
+        for k in (0, 2, 4):
+            v[where][k, rng.integers(N)] = bad
+        x = _dev(v["x0"])
+        ops = kp.make_ops(H, W, 1e-3, 0.02, 1.0 / H, _dev(v["m"]))
+        for solve in (ctx.refine, ctx.seed_solve):
+            xs = x.clone()
+            it, st, rr = kp.decode_info(solve(ops, _dev(v["b"]), xs, tol=1e-8, m=30, maxit=200))
+            torch.cuda.synchronize()
+            assert (st[::2] == kp.BREAKDOWN).all(), (where, st)
+            assert (st[1::2] == kp.OK).all() and (rr[1::2] <= 1e-8).all()
+
+
+@pytest.mark.parametrize("H,W", [(32, 32), (64, 64), (128, 128)])
+@pytest.mark.parametrize("mode", ["warm", "projected"])
+def test_mixed_march_keeps_a_broken_system_broken(kp, H, W, mode):
+    rng = np.random.default_rng(W)
+    s, t = rng.uniform(0, 1, (2, H * W)), rng.uniform(0, 1, (6, H * W))
+    t[1, 5], t[4, 77] = np.nan, np.inf
+    ctx = kp.Context(max_seeds=4, max_n=16384, precision=kp.PREC_MIXED)
+    ds, dt = _dev(s), _dev(t)
+    plan = kp.March(ctx, [(ds, dt, np.array([0, 0, 0, 1, 1, 1]), H, W)], 1000, np.full(1000, 0.01),
+                    mode={"warm": kp.MARCH_WARM, "projected": kp.MARCH_PROJECTED}[mode])
+    st, _ = plan.run(0, 3, stats=True)
+    torch.cuda.synchronize()
+    assert [q.not_converged for q in st] == [2, 2, 2]
+    ok = torch.isfinite(dt).all(1).cpu().numpy()
+    assert ok.tolist() == [True, False, True, True, False, True]
