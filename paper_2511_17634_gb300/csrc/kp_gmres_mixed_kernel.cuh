@@ -717,7 +717,15 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
       const float beta = rnorm.hi;
       // (before the tolerance: an infinite ||b|| is above everything)
       if (!isfinite(beta) || !isfinite(bnorm.hi)) { status = KP_BREAKDOWN; break; }
-      if (beta <= tolb) { status = KP_OK; break; }
+      // ||r|| <= tol ||b||: by the FP32 values, or in double-float where they
+      // are too close (with a margin above its rounding), so that the rel_res
+      // of a converged system is not above tol
+      bool met = beta <= tolb * (1.f - 0x1p-20f);
+      if (!met && beta <= tolb * (1.f + 0x1p-20f)) {
+        const dd t = dd_mul(dd_from_double(p.tol), bnorm);
+        met = (t.hi - rnorm.hi) + (t.lo - rnorm.lo) >= t.hi * 0x1p-40f;
+      }
+      if (met) { status = KP_OK; break; }
       if (steps >= p.maxit || outer >= 64) break;
       const bool first = (outer == 0);
       // the seed's captured cycle runs to the seed tolerance, so its basis has

@@ -198,3 +198,20 @@ def test_mixed_march_keeps_a_broken_system_broken(kp, H, W, mode):
     assert [q.not_converged for q in st] == [2, 2, 2]
     ok = torch.isfinite(dt).all(1).cpu().numpy()
     assert ok.tolist() == [True, False, True, True, False, True]
+
+
+@pytest.mark.parametrize("H,W", [(28, 28), (50, 37), (64, 64), (101, 80), (128, 128)])
+def test_converged_means_rel_res_within_tol(kp, H, W):
+    # tolerances just below and above each system's own residual, closer than
+    # FP32 can tell apart: no iteration is allowed, so only the test decides
+    rng = np.random.default_rng(H + W)
+    N, n = H * W, 24
+    ctx = kp.Context(max_n=16384, precision=kp.PREC_MIXED)
+    b, x0 = _dev(rng.normal(size=(n, N))), _dev(1e-3 * rng.normal(size=(n, N)))
+    ops = kp.make_ops(H, W, 1e-3, 0.02, 1.0 / H, _dev(rng.uniform(0, 1, (n, N))))
+    _, _, rr = kp.decode_info(ctx.refine(ops, b, x0.clone(), tol=0.0, m=30, maxit=0))
+    for k in range(n):
+        for f, status in ((1 - 2.0 ** -27, kp.NOT_CONVERGED), (1 + 2.0 ** -27, kp.OK), (1.01, kp.OK), (0.99, kp.NOT_CONVERGED)):
+            _, st, rk = kp.decode_info(ctx.refine(ops, b, x0.clone(), tol=rr[k] * f, m=30, maxit=0))
+            assert rk[k] == rr[k] and st[k] == status, (k, f)
+            assert (rk[st == kp.OK] <= rr[k] * f).all()
