@@ -77,9 +77,10 @@ typedef struct {
   int block_threads; /* threads per system for grids of <= 1024 points: 256 (4
                         points per thread), 128 (8), 64 (16); 0 = by the number
                         of systems (FP64: 256 with 2 blocks per SM up to one
-                        system per SM, 128 with 2 up to two, else 128 with 4, or
-                        256 with 3 where one call then leaves fewer slots
-                        empty) or 256 with 4 (mixed precision; 64 counts as
+                        system per SM, 128 with 2 up to two -- in a march's
+                        windows one per SM up to one and a half --, else 128
+                        with 4, or 256 with 3 where one call then leaves fewer
+                        slots empty) or 256 with 4 (mixed precision; 64 counts as
                         128 there)                                           */
   int blocks_per_sm; /* resident solver blocks per SM for grids of <= 1024
                         points (caps registers per thread and sizes the

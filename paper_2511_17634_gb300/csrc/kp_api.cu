@@ -42,9 +42,10 @@ cudaError_t launch_solver(const GmresParams& p, const Shape& sh, bool mixed, cud
 }
 
 kp_status gmres_shape(kp_ctx* c, int nmax, int m, Shape* out, bool mixed, int wmin, int hmax,
-                      bool one_size, int count, bool one_launch) {
+                      bool one_size, int count, bool one_launch, bool windows) {
   Shape sh;
   sh.minb = 1;
+  bool alone = false;                            // one block per SM all the same
   if (nmax <= 1024) {
     // default (FP64): 128 threads x 8 points, 4 resident blocks per SM -- more
     // independent systems per SM hide the per-step barriers and the serial
@@ -58,14 +59,19 @@ kp_status gmres_shape(kp_ctx* c, int nmax, int m, Shape* out, bool mixed, int wm
       // Few systems leave SMs with one or two blocks, whose own latency then
       // counts: the shapes with registers to spare (126 and 224 a thread, no
       // spills) are faster there -- 28x28, 4 targets: 10.1 -> 8.1 ms for 50
-      // timesteps (256 x 4); 192 targets and 30 seeds of 32x32: 116 -> 97 ms
-      // for 100 (128 x 8, two blocks per SM; 256 x 4: 101).  A single launch
-      // of 768 systems fills 608 slots 1.26 times but 456 slots 1.68 times, two
-      // rounds of three blocks per SM instead of two of four: 0.55 -> 0.50 ms
-      // for one 32x32x3 step.
+      // timesteps (256 x 4); 270 targets and 30 seeds of 32x32 with g = 0.5:
+      // 5.98 -> 5.20 ms for 16 (128 x 8, two blocks per SM; 256 x 4: 5.42).
+      // In windows of timesteps the blocks are resident and a second one on an
+      // SM slows the first: while less than half of the SMs would have two,
+      // each keeps its SM and some blocks march two systems (192 targets, 30
+      // seeds, 100 timesteps with g = 0.5: 97.2 ms against 100.5; 254 of 28x28, 16:
+      // 1.78 against 1.58, so two there).
+      // A single launch of 768 systems fills 608 slots 1.26 times but 456 slots
+      // 1.68 times, two rounds of three blocks per SM instead of two of four:
+      // 0.55 -> 0.50 ms for one 32x32x3 step.
       const int rounds3 = (count + 3 * c->sms - 1) / (3 * c->sms), rounds4 = (count + 4 * c->sms - 1) / (4 * c->sms);
       if (count <= c->sms) { sh.nt = 256; sh.ept = 4; sh.minb = 2; }
-      else if (count <= 2 * c->sms) { sh.minb = 2; }
+      else if (count <= 2 * c->sms) { sh.minb = 2; alone = windows && 2 * count <= 3 * c->sms; }
       else if (one_launch && 3 * rounds3 < 4 * rounds4) { sh.nt = 256; sh.ept = 4; sh.minb = 3; }
     }
     if (mixed) {                                 // the FP32 solver has the 256- and 128-thread shapes
@@ -133,7 +139,7 @@ kp_status gmres_shape(kp_ctx* c, int nmax, int m, Shape* out, bool mixed, int wm
   // shared memory of one CTA when minb of them share an SM (1 KB per CTA is
   // reserved by the hardware)
   const size_t budget = mixed ? c->smem_optin / sh.minb - (sh.minb >= 2 ? 1024 : 0)
-                      : npad <= 1024 ? c->smem_optin / sh.minb - (sh.minb > 2 ? 1024 : 0)
+                      : npad <= 1024 ? c->smem_optin / sh.minb - (sh.minb >= 2 ? 1024 : 0)
                                      : c->smem_optin;
   // the mixed-precision solver keeps x (hi, lo) and r in three slots between cycles
   const int smin = mixed ? 3 : 1;
@@ -143,6 +149,8 @@ kp_status gmres_shape(kp_ctx* c, int nmax, int m, Shape* out, bool mixed, int wm
     while (S < m + 1 && bytes(S + 1) <= budget) ++S;
   }
   S = std::max(std::min(S, m + 1), smin);
+  // (no larger than it takes to keep the SM: what is left of it is L1 cache)
+  while (alone && c->opt.smem_vectors <= 0 && S < m + 1 && 2 * (bytes(S) + 1024) <= c->smem_optin + 1024) ++S;
   while (S > smin && bytes(S) > c->smem_optin) --S;
   if (bytes(S) > c->smem_optin) return set_error(c, KP_ERR_UNSUPPORTED, "shared memory too small");
   sh.S = S;

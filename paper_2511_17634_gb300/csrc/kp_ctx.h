@@ -100,7 +100,8 @@ kp_status cuda_error(kp_ctx* c, cudaError_t e, const char* what);
 // many), one_launch: all of them by one launch of as many blocks (FP64).
 // Mixed precision: the systems of one launch.
 kp_status gmres_shape(kp_ctx* c, int nmax, int m, Shape* out, bool mixed = false,
-                      int wmin = 0, int hmax = 0, bool one_size = false, int count = 0, bool one_launch = false);
+                      int wmin = 0, int hmax = 0, bool one_size = false, int count = 0, bool one_launch = false,
+                      bool windows = false);
 // The shape's part of the solver parameters and the CTAs' workspace.
 inline void set_shape(GmresParams* p, const Shape& sh) {
   p->S = sh.S;

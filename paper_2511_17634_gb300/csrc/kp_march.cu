@@ -516,10 +516,11 @@ kp_status kp_march_create(kp_ctx* c, int ngroups, const kp_group* groups, const 
   }
   P->mixed = c->opt.precision == KP_PREC_MIXED;
   kp_status s = KP_OK;
+  const bool windows = !P->mixed && o.window != 1 && o.T > 1 && P->nt > 0 && (!P->ns || c->opt.max_seeds / (2 * P->ns) > 1);
   if (P->ns) s = kp::gmres_shape(c, nmaxS, o.m_seed, &P->shS, P->mixed, wminS, hmaxS, ngroups == 1,
-                                  P->mixed ? P->ns : P->ns + P->nt);
+                                  P->mixed ? P->ns : P->ns + P->nt, false, windows);
   if (s == KP_OK && P->nt) s = kp::gmres_shape(c, nmaxT, o.m, &P->shT, P->mixed, wminT, hmaxT, ngroups == 1,
-                                                 P->mixed ? P->nt : P->ns + P->nt);
+                                                 P->mixed ? P->nt : P->ns + P->nt, false, windows);
   if (s == KP_OK && ((P->shS.cs && ngroups > 1) || (P->shT.cs && ngroups > 1))) {
     kp_march_destroy(P);
     return kp::set_error(c, KP_ERR_UNSUPPORTED, "grids above 4096 unknowns: one grid size per plan");
