@@ -109,11 +109,14 @@ typedef struct {
                         the iterative refinement recomputes the true
                         residual; 1..7, 0 = 5                                     */
   int cluster_blocks_per_sm; /* cluster solver (grids above 4096 points): resident
-                        CTAs per SM, 1 or 2 (16-CTA clusters: 2 or 4); 0 = 3
-                        where a slice fills its CTA, else 2 (16-CTA clusters:
-                        4) -- several systems share the SMs,
-                        each with a smaller shared-memory window of Krylov
-                        vectors                                                  */
+                        CTAs per SM, 1 or 2 (16-CTA clusters: 2 or 4); 0 = 2
+                        (16-CTA clusters: 4), or 3 on clusters of 4 whose slices
+                        fill their CTAs with columns of H points, H dividing
+                        256 -- several systems share the SMs, each with a
+                        smaller shared-memory window of Krylov vectors.  1 (2 of
+                        16-CTA clusters) only makes the window larger and
+                        launches fewer CTAs: the kernels are compiled for the
+                        default                                               */
 } kp_options;
 
 /* Operator of one system (Sec. 2.3): A(m~; g^2, dt, h, f).  `mtilde` is the

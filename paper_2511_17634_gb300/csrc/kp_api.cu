@@ -123,22 +123,31 @@ kp_status gmres_shape(kp_ctx* c, int nmax, int m, Shape* out, bool mixed, int wm
   }
   const int npad = sh.ept * sh.nt;
   sh.vld = npad;
+  int share = 0;                                 // mixed precision: CTAs that the window leaves room for
   if (mixed) {
     // full CTAs, columns that divide the CTA's threads; the shapes on request
     // have no such kernel
     sh.reg = one_size && nmax == sh.ctas() * npad && hmax > 0 && sh.nt % hmax == 0 && !c->opt.cluster_size &&
              sh.nt == 256 && (!sh.cs || sh.ept == 16);
     sh.hmax = sh.cs || sh.reg ? hmax : 0;
-    if (sh.reg && sh.ept == 16 && !c->opt.cluster_blocks_per_sm) sh.minb = 3;
+    if (sh.reg && sh.ept == 16 && !c->opt.cluster_blocks_per_sm) {
+      // the window of three CTAs per SM also where two are resident (clusters
+      // of two): the rest of the SM is L1 cache for the workspace (64x128, 900
+      // systems, warm: 1.06 ms against 1.11 with the window of two; more
+      // vectors pay for harder systems, g = 0.5: 4.50 against 4.25)
+      sh.minb = mixed_reg_blocks(sh.ctas());
+      share = 3;
+    }
     sh.vld += 2 * sh.hmax;
+    if (!share) share = sh.minb;
   }
   auto bytes = [&](int S) {
     return mixed ? gmres_mixed_smem_bytes(sh.nt, sh.ctas(), sh.hmax, sh.vld, S, m)
                  : gmres_fp64_smem_bytes(sh.ept, sh.nt, S, m);
   };
-  // shared memory of one CTA when minb of them share an SM (1 KB per CTA is
-  // reserved by the hardware)
-  const size_t budget = mixed ? c->smem_optin / sh.minb - (sh.minb >= 2 ? 1024 : 0)
+  // shared memory of one CTA when minb (share) of them are on an SM (1 KB per
+  // CTA is reserved by the hardware)
+  const size_t budget = mixed ? c->smem_optin / share - (share >= 2 ? 1024 : 0)
                       : npad <= 1024 ? c->smem_optin / sh.minb - (sh.minb >= 2 ? 1024 : 0)
                                      : c->smem_optin;
   // the mixed-precision solver keeps x (hi, lo) and r in three slots between cycles

@@ -9,8 +9,8 @@ namespace kp {
 cudaError_t launch_gmres_cluster(const GmresParams& p, int ept, int nt, int cs, bool reg, size_t smem,
                                  cudaStream_t st) {
   if (ept == 16 && nt == 256) {                  // the default: 4096 points per CTA
-    if (cs == 4) return reg ? launch_mx<16, 256, 4, 3, 2, true>(p, smem, st) : launch_mx<16, 256, 4, 2, 2, false>(p, smem, st);
-    if (cs == 2) return reg ? launch_mx<16, 256, 2, 2, 2, true>(p, smem, st) : launch_mx<16, 256, 2, 2, 2, false>(p, smem, st);
+    if (cs == 4) return reg ? launch_mx<16, 256, 4, mixed_reg_blocks(4), 2, true>(p, smem, st) : launch_mx<16, 256, 4, 2, 2, false>(p, smem, st);
+    if (cs == 2) return reg ? launch_mx<16, 256, 2, mixed_reg_blocks(2), 2, true>(p, smem, st) : launch_mx<16, 256, 2, 2, 2, false>(p, smem, st);
   }
   if (ept == 8 && nt == 256) {                   // cluster_size 2, 4, 8: 2048 points per CTA
     if (cs == 8) return launch_mx<8, 256, 8, 2, 0, false>(p, smem, st);

@@ -20,7 +20,7 @@ cudaError_t launch_gmres_mixed(const GmresParams& p, int ept, int nt, bool reg, 
     return reg ? launch_mx<4, 256, 1, 4, 0, true>(p, smem, st) : launch_mx<4, 256, 1, 4, 0, false>(p, smem, st);
   if (ept == 8 && nt == 128) return launch_mx<8, 128, 1, 4, 0, false>(p, smem, st);
   if (ept == 16 && nt == 256)
-    return reg ? launch_mx<16, 256, 1, 3, 1, true>(p, smem, st) : launch_mx<16, 256, 1, 2, 1, false>(p, smem, st);
+    return reg ? launch_mx<16, 256, 1, mixed_reg_blocks(1), 1, true>(p, smem, st) : launch_mx<16, 256, 1, 2, 1, false>(p, smem, st);
   return cudaErrorInvalidValue;
 }
 

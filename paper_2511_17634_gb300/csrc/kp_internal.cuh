@@ -624,6 +624,9 @@ size_t gmres_fp64_smem_bytes(int ept, int nt, int S, int m);
 // Mixed precision: shared memory of a CTA with S vector slots of vld floats
 // (cs CTAs per system, 1 for the one-block solver; hmax: longest column).
 size_t gmres_mixed_smem_bytes(int nt, int cs, int hmax, int vld, int S, int m);
+// CTAs per SM that the register form (REG) of 4096-point CTAs is compiled for,
+// by CTAs per system: its grid and workspace are sized for as many.
+constexpr int mixed_reg_blocks(int cs) { return cs == 2 ? 2 : 3; }
 // reg: every system fills its CTAs and its columns divide a sub-block (the REG kernels).
 cudaError_t launch_gmres_mixed(const GmresParams& p, int ept, int nt, bool reg, size_t smem, cudaStream_t st);
 // Cluster of cs CTAs per system (grids above 4096 unknowns, or on request).

@@ -77,3 +77,15 @@ def test_fp64_blocks_of_a_window_keep_their_sm_while_few_would_share_it(shapes):
     for r, s in zip(rows, shapes(rows)):
         assert s["status"] == 0 and s["minb"] == 2
         assert _fits(s) != (152 < r[6] <= 228), (r, s)
+
+
+def test_mixed_grid_is_what_its_kernel_keeps_resident(shapes):
+    # full CTAs of 4096 points: three of them per SM are compiled for one and
+    # four CTAs per system, two for two
+    rows = [(n, m, 1, W, H, 1, 2000, 1, 0, 0, 0, 0, 0) for m in range(1, 65)
+            for n, H, W in ((4096, 64, 64), (8192, 64, 128), (8192, 128, 64), (16384, 128, 128))]
+    for r, s in zip(rows, shapes(rows)):
+        assert s["status"] == 0 and s["reg"] and s["ept"] == 16 and s["S"] >= 3
+        assert (s["cs"], s["minb"]) == {4096: (0, 3), 8192: (2, 2), 16384: (4, 3)}[r[0]]
+        if r[1] <= 40:
+            assert _fits(s), (r, s)
