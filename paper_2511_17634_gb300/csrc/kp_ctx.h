@@ -83,6 +83,7 @@ struct Shape {
   // parts of the operator coefficients
   size_t ws = 0;
   int vld = 0;    // values of a vector slot (mixed precision on a cluster: with its halo columns)
+  int redv = 8;   // mixed precision, clusters: values per reduction round
   int hmax = 0;   // longest column of the systems (mixed precision with halo columns)
   bool reg = false;   // mixed precision: see launch_gmres_mixed
   int ctas() const { return cs ? cs : 1; }
@@ -109,6 +110,7 @@ inline void set_shape(GmresParams* p, const Shape& sh) {
   p->vld = sh.vld;
   p->hmax = sh.hmax;
   p->ws_ld = sh.ws;
+  p->red_v = sh.redv;
 }
 // Inner FP32 residual reduction of the mixed-precision solvers.
 inline double inner_eta(const kp_options& o) {

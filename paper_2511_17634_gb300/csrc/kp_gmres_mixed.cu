@@ -6,9 +6,9 @@
 
 namespace kp {
 
-size_t gmres_mixed_smem_bytes(int nt, int cs, int hmax, int vld, int S, int m) {
+size_t gmres_mixed_smem_bytes(int nt, int cs, int hmax, int vld, int S, int m, int redv) {
   const size_t nw = nt / 32, f = sizeof(float), f2 = sizeof(float2);
-  const size_t fixed = (4 * (size_t)m + 2) * f2 + nw * kMaxV * f2 + 4 * kRedV * nw * cs * f + kMaxV * f +
+  const size_t fixed = (4 * (size_t)m + 2) * f2 + nw * kMaxV * f2 + 4 * (redv > 0 ? redv : kRedV) * nw * cs * f + kMaxV * f +
                        8 * sizeof(int) + 4 * (size_t)hmax * f;
   const size_t hess = (size_t)m * (m + 1) / 2 * f2;
   // exact Galerkin lays its a x a FP64 matrix over the Hessenberg matrix and the slots

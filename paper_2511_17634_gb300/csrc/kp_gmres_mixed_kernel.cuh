@@ -75,6 +75,8 @@ namespace {
 
 // Values per reduction round: longer Gram-Schmidt sums take several rounds
 // (and barriers), which keeps the partials of 64 warps within 4 KB (two sets).
+// Clusters, whose barriers cost more, take as many more as the shared memory
+// beside the Krylov window holds (GmresParams::red_v).
 constexpr int kRedV = 8;
 
 __device__ __forceinline__ float2 as_f2(dd x) { return make_float2(x.hi, x.lo); }
@@ -199,8 +201,9 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
   float2* gv = rinv + m;                                      // [m + 2]
   float2* hball = gv + m + 2;                                 // [NT / 32][kMaxV] sums, a copy per warp
   float2* hb = hball + warp * kMaxV;
-  float* red = reinterpret_cast<float*>(hball + (NT / 32) * kMaxV);   // [2][kRedV][P]
-  float* yf = red + 2 * kRedV * P;                            // [kMaxV] combination coefficients
+  float* red = reinterpret_cast<float*>(hball + (NT / 32) * kMaxV);   // [2][redv][P]
+  const int redv = CS > 1 ? p.red_v : kRedV;
+  float* yf = red + 2 * redv * P;                             // [kMaxV] combination coefficients
   int* fl = reinterpret_cast<int*>(yf + kMaxV);               // [8]
   float* whalo = reinterpret_cast<float*>(fl + 8);            // [2][2 hmax] pushed edge columns
   float2* Hr = reinterpret_cast<float2*>(whalo + 4 * p.hmax); // packed columns of R: j at j (j + 1) / 2
@@ -222,6 +225,7 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
   const int parity_base = slot_set_base(p, tstep);
   const float kEta = p.inner_eta > 0.0 ? (float)p.inner_eta : 1e-5f;
   int buf = 0, hbuf = 0;                         // parities of the reductions and of the halo pushes
+  int zeroed = -1;                               // where the zeros of the slots begin (short slices)
 
   // resident CTAs claim systems until none is left: the workspace is then as
   // large as the GPU holds CTAs and stays in L2 (a slice per system was 7 GB
@@ -255,9 +259,18 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
     auto lp = [&](int k) { return !REG && HALF == 2 && k >= EPT / 2 ? SH + tid + (k - EPT / 2) * NT : tid + k * NT; };
     auto inside = [&](int k) { return REG || (HALF == 2 ? tid + (k % (EPT / 2)) * NT < SH : tid + k * NT < SL); };
     auto chain = [](int k) { return HALF == 1 ? k & 1 : HALF == 2 ? (k >= EPT / 2) : 0; };
-    // points past the slice (w = 0 there): on one CTA their slots hold zeros;
-    // on a cluster that space is the halo's, so short slices are guarded
+    // points past the slice: w = 0 there.  On one CTA their slots hold zeros.
+    // On a cluster that space is the halo's, so stores of short slices are
+    // guarded; the sums and updates of Gram-Schmidt read it all the same (a
+    // guard per point and vector doubled the instructions of a system of 30
+    // steps: 101x80, 270 systems with g = 0.5, 4.73 -> 3.08 ms), which takes
+    // finite values behind the halo too
     const bool full = REG || CS == 1 || SL == EPT * NT;
+    if (!full && zeroed != SL + 2 * H) {
+      zeroed = SL + 2 * H;
+      for (int i = 0; i <= m; ++i)
+        for (int q = SL + 2 * H + tid; q < vld; q += NT) slot(i)[q] = 0.f;
+    }
     // the operator constants c = g^2/(2h^2), e = c/4, c_d = 1/dt + 4c from the
     // descriptor's quotients: a division is a dozen FP64 instructions on
     // every warp.  Solved as (A / s) x = b / s with s = b_scale: the scale is
@@ -425,9 +438,9 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
     // CTA, identical bits; part(i0, nv, a) gives this thread's chains of values
     // i0 .. i0 + 3.  Ends with __syncwarp.
     auto reduce = [&](int nv, auto&& part) {
-      for (int c0 = 0; c0 < nv; c0 += kRedV) {
-        const int nc = min(kRedV, nv - c0);
-        float* rb = red + buf * kRedV * P;
+      for (int c0 = 0; c0 < nv; c0 += redv) {
+        const int nc = min(redv, nv - c0);
+        float* rb = red + buf * redv * P;
 #pragma unroll 1
         for (int i0 = 0; i0 < nc; i0 += 4) {
           float a[NH][4];
@@ -800,8 +813,7 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
               if (i < n - 1) {
                 auto dot = [&](const float* vi) {
 #pragma unroll
-                  for (int k = 0; k < EPT; ++k)
-                    if (full || inside(k)) s[chain(k)][u] = fmaf(vi[lp(k)], w[k], s[chain(k)][u]);
+                  for (int k = 0; k < EPT; ++k) s[chain(k)][u] = fmaf(vi[lp(k)], w[k], s[chain(k)][u]);   // (w = 0 outside)
                 };
                 if (i < p.S) dot(V + (size_t)i * vld + hal);
                 else dot(Vg + (size_t)(i - p.S) * vld + hal);
@@ -827,25 +839,51 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
           hn2 = dd_sub(ww, sq);
           if (warp == 0)
             for (int i = lane; i < nh; i += 32) col[i] = pass ? as_f2(dd_add(as_dd(col[i]), as_dd(hb[i]))) : hb[i];
-          // w -= sum h_i v_i on the slice and, in the halo buffer, on the halo
+          // w -= sum h_i v_i on the slice and on the halo.  A thread's first
+          // halo point goes along with its points of the slice, the others of
+          // long columns several at a time: in a loop of its own each waited a
+          // latency per vector (L2 past the window; 128x128, 300 systems, warm:
+          // 1126 -> 1097 us, 2048x8 36.6 -> 22.7 ms)
+          float* wh = whalo + hbuf * 2 * p.hmax;
+          const bool hq = CS > 1 && tid < 2 * H;
+          float hv = hq ? wh[tid] : 0.f;
 #pragma unroll 1
           for (int i = 0; i < nh; ++i) {
             const float hi = hb[i].x;
             auto sub_ = [&](const float* vi) {
 #pragma unroll
-              for (int k = 0; k < EPT; ++k)
-                if (full || inside(k)) w[k] = fmaf(-hi, vi[lp(k)], w[k]);
+              for (int k = 0; k < EPT; ++k) w[k] = fmaf(-hi, vi[hal + lp(k)], w[k]);
+              if (hq) hv = fmaf(-hi, vi[tid < H ? tid : SL + tid], hv);
             };
-            if (i < p.S) sub_(V + (size_t)i * vld + hal);
-            else sub_(Vg + (size_t)(i - p.S) * vld + hal);
+            if (i < p.S) sub_(V + (size_t)i * vld);
+            else sub_(Vg + (size_t)(i - p.S) * vld);
           }
-          if (CS > 1)
-            for (int q = tid; q < 2 * H; q += NT) {
-              float* wh = whalo + hbuf * 2 * p.hmax + q;
-              float v = *wh;
-              for (int i = 0; i < nh; ++i) v = fmaf(-hb[i].x, slot(i)[q < H ? q : SL + q], v);
-              *wh = v;
+          if (!full)
+#pragma unroll
+            for (int k = 0; k < EPT; ++k) w[k] = inside(k) ? w[k] : 0.f;
+          if (hq) wh[tid] = hv;
+          if (CS > 1) {
+            constexpr int B = REG ? 1 : 8;       // (REG: H <= NT)
+#pragma unroll 1
+            for (int q0 = tid + NT; q0 < 2 * H; q0 += B * NT) {
+              float v[B];
+#pragma unroll
+              for (int u = 0; u < B; ++u) v[u] = q0 + u * NT < 2 * H ? wh[q0 + u * NT] : 0.f;
+#pragma unroll 1
+              for (int i = 0; i < nh; ++i) {
+                const float hi = hb[i].x;
+                const float* vi = slot(i);
+#pragma unroll
+                for (int u = 0; u < B; ++u) {
+                  const int q = q0 + u * NT;
+                  if (q < 2 * H) v[u] = fmaf(-hi, vi[q < H ? q : SL + q], v[u]);
+                }
+              }
+#pragma unroll
+              for (int u = 0; u < B; ++u)
+                if (q0 + u * NT < 2 * H) wh[q0 + u * NT] = v[u];
             }
+          }
           if (pass == 0) {
             ww0 = ww.hi;
             if (p.reorth != 0 && hn2.hi >= 0.5f * ww0) break;

@@ -130,6 +130,7 @@ struct GmresParams {
   int vld;                  // floats of a vector slot: npad and two halo columns
   int hmax;                 // longest column of the launch's systems (cluster halos)
   size_t ws_ld;             // floats of a CTA's workspace
+  int red_v;                // values per reduction round (clusters)
   float* capV32;            // capture target for FP32 bases (slot layout when factor)
   const float* slotV32;     // [max_seeds][max_a + 1][slot_ld] FP32 seed bases
   const float* cproj;       // if set: c = V^T b per target, [nsys][cproj_ld] (tensor-core GEMM)
@@ -623,7 +624,8 @@ cudaError_t launch_gmres_fp64_picard(const GmresParams& p, int ept, int nt, int 
 size_t gmres_fp64_smem_bytes(int ept, int nt, int S, int m);
 // Mixed precision: shared memory of a CTA with S vector slots of vld floats
 // (cs CTAs per system, 1 for the one-block solver; hmax: longest column).
-size_t gmres_mixed_smem_bytes(int nt, int cs, int hmax, int vld, int S, int m);
+// redv: values per reduction round (0: the least).
+size_t gmres_mixed_smem_bytes(int nt, int cs, int hmax, int vld, int S, int m, int redv = 0);
 // CTAs per SM that the register form (REG) of 4096-point CTAs is compiled for,
 // by CTAs per system: its grid and workspace are sized for as many.
 constexpr int mixed_reg_blocks(int cs) { return cs == 2 ? 2 : 3; }

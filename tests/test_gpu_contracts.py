@@ -215,3 +215,32 @@ def test_converged_means_rel_res_within_tol(kp, H, W):
             _, st, rk = kp.decode_info(ctx.refine(ops, b, x0.clone(), tol=rr[k] * f, m=30, maxit=0))
             assert rk[k] == rr[k] and st[k] == status, (k, f)
             assert (rk[st == kp.OK] <= rr[k] * f).all()
+
+
+@pytest.mark.parametrize("H,W,n,m", [
+    (101, 80, 5, 40), (101, 80, 90, 12), (72, 64, 200, 64), (128, 120, 90, 40), (129, 96, 40, 40), (300, 48, 6, 40),
+    (256, 64, 5, 20), (1024, 16, 4, 40), (2048, 8, 3, 64), (8, 1024, 5, 40)])
+def test_clusters_on_systems_of_many_steps(kp, orc, H, W, n, m):
+    # short slices, columns past a block's threads and past its points, basis
+    # vectors past the shared-memory window, several reduction rounds, restarts;
+    # copies of three systems.  cond(A) <= 1 + 16 c dt with c = g^2 / (2 h^2):
+    # h is chosen so that it is 40, about 25 to 35 steps to 1e-9 (times the
+    # condition: 1e-7)
+    rng = np.random.default_rng(H + 7 * n)
+    N, dt, g2 = H * W, 1e-3, 0.25
+    h = np.sqrt(8 * g2 * dt / 39.0)
+    mt, b = rng.uniform(0, 0.05, (3, N)), rng.normal(size=(3, N))
+    at = torch.arange(n, device="cuda") % 3
+    ctx = kp.Context(max_n=16384, precision=kp.PREC_MIXED)
+    x = torch.zeros((n, N), dtype=torch.float64, device="cuda")
+    info = ctx.refine(kp.make_ops(H, W, dt, g2, h, _dev(mt)[at].contiguous()), _dev(b)[at].contiguous(), x, tol=1e-9, m=m, maxit=2000)
+    it, st, rr = kp.decode_info(info)
+    torch.cuda.synchronize()
+    assert (st == 0).all() and (rr <= 1e-9).all() and it.min() >= 15, it
+    for k in range(min(3, n)):
+        assert bool((x[k::3] == x[k]).all())
+        C = orc.coeffs(H, W, g2, dt, h, mt[k])
+        xk = x[k].cpu().numpy()
+        assert np.linalg.norm(b[k] - orc.apply(H, W, C, xk)) <= 1.01e-9 * np.linalg.norm(b[k])
+        ref = orc.gmres(H, W, C, b[k], tol=1e-12, m=60, maxit=4000).x
+        assert np.linalg.norm(xk - ref) <= 1e-7 * np.linalg.norm(ref)
