@@ -858,7 +858,7 @@ __global__ void __launch_bounds__(NT, MINB) gmres_fp64_kernel(const GmresParams 
           store_factors(a, hn, capH, p.cap_a + 1, [&](int i, int j) { return sm.Hr[i + j * ld]; },
                         [&](int j) { return sm.cs[j]; }, [&](int j) { return sm.sn[j]; },
                         [&](int j) { return sm.rinv[j]; }, p.capR + (size_t)cidx * (p.cap_a + 1) * p.cap_a,
-                        p.cap_a + 1, rot, rot + 2 * p.cap_a, &lsq, &nrot, lane);
+                        p.cap_a + 1, rot, rot + 2 * p.cap_a, &lsq, &nrot, 1e-14, lane);
           if (lane == 0) {
             if (p.factor) {
               SlotMeta mt;

@@ -961,7 +961,7 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
                       [&](int j) { return dd_to_double(as_dd(cs[j])); }, [&](int j) { return dd_to_double(as_dd(sn[j])); },
                       [&](int j) { return dd_to_double(as_dd(rinv[j])) * (double)hsc; },
                       p.capR + (size_t)cidx * (p.cap_a + 1) * p.cap_a, p.cap_a + 1, rot, rot + 2 * p.cap_a, &lsq, &nrot,
-                      lane);
+                      kDdPivot, lane);
         if (lane == 0) {
           if (p.factor) {
             SlotMeta sm;

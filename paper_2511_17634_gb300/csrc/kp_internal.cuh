@@ -521,10 +521,17 @@ __host__ __device__ __forceinline__ unsigned long long gmres_flops(int k, int m)
   return f;
 }
 
+// Pivots below this share of max|H_a| are rounding in double-float.  On singular
+// H_a along which rounding doubles every second column, the last pivot passes
+// 1e-14 at 15 columns, in FP64 at 35: 2^10 times FP64's rounding.  (H_a itself
+// holds FP32 sums, 1e-7 of it.)
+constexpr double kDdPivot = 1e-11;
+
 // The projection factors of Sec. 3 from a captured GMRES cycle, by one warp:
 // the Givens QR of H_a is the cycle's own (R: rotated columns, c, s: rotations,
 // rinv: reciprocal pivots, read by index), except that H_a's last column is not
-// rotated against row a + 1.  If a pivot of that R is below 1e-14 max|H_a| and
+// rotated against row a + 1.  If a pivot of that R is below tiny max|H_a| (the
+// rounding of the rotations: 1e-14 for FP64, kDdPivot for double-float) and
 // v_{a+1} exists, the least-squares factor of Hbar (a rotations) is kept
 // instead.  Hb: unrotated Hbar, column-major, leading dim hld.  Writes R (a + 1
 // rows, leading dim ld), rot (c, s pairs) and ri (0 for a zero pivot).
@@ -532,7 +539,7 @@ __host__ __device__ __forceinline__ unsigned long long gmres_flops(int k, int m)
 template <typename FR, typename FC, typename FS, typename FI>
 __device__ __forceinline__ void store_factors(int a, int has_next, const double* Hb, int hld, FR&& getR, FC&& getC,
                                               FS&& getS, FI&& getI, double* R, int ld, double* rot, double* ri,
-                                              int* lsq_out, int* nrot_out, int lane) {
+                                              int* lsq_out, int* nrot_out, double tiny, int lane) {
   __syncwarp();
   unsigned long long hm = 0;                               // max|H_a| as bits
   for (int e = lane; e < a * a; e += 32) {
@@ -547,7 +554,7 @@ __device__ __forceinline__ void store_factors(int a, int has_next, const double*
     const unsigned long long v = __shfl_xor_sync(kFull, hm, o);
     hm = v > hm ? v : hm;
   }
-  const double least = 1e-14 * __longlong_as_double((long long)hm);
+  const double least = tiny * __longlong_as_double((long long)hm);
   const double last = a > 0 ? getC(a - 1) * getR(a - 1, a - 1) : 0.0;
   int small = 0;
   for (int j = lane; j < a; j += 32) small |= !(fabs(j == a - 1 ? last : getR(j, j)) > least);

@@ -244,3 +244,42 @@ def test_clusters_on_systems_of_many_steps(kp, orc, H, W, n, m):
         assert np.linalg.norm(b[k] - orc.apply(H, W, C, xk)) <= 1.01e-9 * np.linalg.norm(b[k])
         ref = orc.gmres(H, W, C, b[k], tol=1e-12, m=60, maxit=4000).x
         assert np.linalg.norm(xk - ref) <= 1e-7 * np.linalg.norm(ref)
+
+
+# ---- projection factors
+
+def _singular_hessenberg(kp, a, precision, d=1.0):
+    """A seed solve (1 x W grid, b = e_1, no diffusion) whose captured H_a is
+    tridiagonal with exact entries and exactly singular: diagonal d, products
+    p_n of the off-diagonals with D_n = d D_{n-1} + p_n D_{n-2}, D_n / D_{n-1}
+    = d, -1, -1, ..., 0."""
+    p = [None, None, -2.0] + [2.0] * (a - 3) + [1.0]
+    W = a + 4
+    q = np.ones(W)
+    for n in range(2, a + 1):
+        q[n - 1] = p[n] / q[n - 2]
+    ctx = kp.Context(max_seeds=2, max_a=40, max_n=64, precision=precision)
+    ops = kp.make_ops(1, W, 1.0 / d, 0.0, 0.5, _dev(np.zeros((1, W))), _dev(q[None]), None)
+    b = np.zeros((1, W))
+    b[0, 0] = 1.0
+    ctx.seed_solve(ops, _dev(b), torch.zeros((1, W), dtype=torch.float64, device="cuda"), tol=1e-12, m=a, maxit=a)
+    ctx.store_basis(0, 1, 0)
+    return ctx, ops, W
+
+
+@pytest.mark.parametrize("a", [3, 8, 14, 15, 21, 30])
+@pytest.mark.parametrize("mixed", [False, True])
+def test_singular_basis_takes_the_least_squares(kp, orc, a, mixed):
+    # x0 is the least-squares projection of the oracle for the same basis: 1e-4
+    # of its norm in mixed precision (FP32 basis and coefficients, alpha up to
+    # 2^(a / 2) of the data), 1e-9 in FP64
+    ctx, ops, W = _singular_hessenberg(kp, a, kp.PREC_MIXED if mixed else kp.PREC_FP64)
+    n, hn, V, Hb = ctx.basis_get(0, 1, W)
+    assert n == a and hn == 1
+    r = np.ones((1, W))
+    x0 = torch.zeros((1, W), dtype=torch.float64, device="cuda")
+    ctx.project_targets(0, 1, ops, _dev(r), x0)
+    torch.cuda.synchronize()
+    ref, lsq = orc.project(V.cpu().numpy(), Hb, n, hn, r[0])
+    assert lsq
+    assert np.linalg.norm(x0.cpu().numpy()[0] - ref) <= (1e-4 if mixed else 1e-9) * np.linalg.norm(ref)
