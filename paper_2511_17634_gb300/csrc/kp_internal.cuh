@@ -555,7 +555,11 @@ __device__ __forceinline__ void store_factors(int a, int has_next, const double*
     hm = v > hm ? v : hm;
   }
   const double least = tiny * __longlong_as_double((long long)hm);
-  const double last = a > 0 ? getC(a - 1) * getR(a - 1, a - 1) : 0.0;
+  // (a zero column after its rotations has no rotation of its own: c and R are
+  // NaN there, the pivot is zero; NaN in H_a itself stays)
+  const double rl = a > 0 ? getR(a - 1, a - 1) : 0.0;
+  const bool none = isnan(rl) && hm < 0x7FF0000000000000ull;
+  const double last = a > 0 && !none ? getC(a - 1) * rl : 0.0;
   int small = 0;
   for (int j = lane; j < a; j += 32) small |= !(fabs(j == a - 1 ? last : getR(j, j)) > least);
   const int lsq = __any_sync(kFull, small) && has_next;

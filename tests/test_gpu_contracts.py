@@ -283,3 +283,21 @@ def test_singular_basis_takes_the_least_squares(kp, orc, a, mixed):
     ref, lsq = orc.project(V.cpu().numpy(), Hb, n, hn, r[0])
     assert lsq
     assert np.linalg.norm(x0.cpu().numpy()[0] - ref) <= (1e-4 if mixed else 1e-9) * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("mixed", [False, True])
+def test_singular_basis_at_a_breakdown_stays_finite(kp, orc, mixed):
+    # A = [[1, -1], [-1, 1]], b = e_1: the second column is zero after its
+    # rotation and there is no next vector; x0 as the oracle's (zero pivot:
+    # that coefficient is left out)
+    ctx = kp.Context(max_seeds=2, max_a=40, max_n=64, precision=kp.PREC_MIXED if mixed else kp.PREC_FP64)
+    q, b, r = np.array([[-1.0, 1.0]]), np.array([[1.0, 0.0]]), np.array([[0.25, 1.0]])
+    ops = kp.make_ops(1, 2, 1.0, 0.0, 0.5, _dev(np.zeros((1, 2))), _dev(q), None)
+    ctx.seed_solve(ops, _dev(b), torch.zeros((1, 2), dtype=torch.float64, device="cuda"), tol=1e-12, m=10, maxit=10)
+    ctx.store_basis(0, 1, 0)
+    n, hn, V, Hb = ctx.basis_get(0, 1, 2)
+    assert n == 2 and hn == 0
+    x0 = torch.zeros((1, 2), dtype=torch.float64, device="cuda")
+    ctx.project_targets(0, 1, ops, _dev(r), x0)
+    ref, _ = orc.project(V.cpu().numpy(), Hb, n, hn, r[0])
+    assert np.isfinite(ref).all() and np.linalg.norm(x0.cpu().numpy()[0] - ref) <= 1e-6 * np.linalg.norm(ref)
