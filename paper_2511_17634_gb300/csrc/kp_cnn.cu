@@ -50,6 +50,16 @@ __global__ void mse_kernel(const float* y, const float* t, float* dz, size_t n, 
   if (threadIdx.x == 0) atomicAdd(loss, red[0] / (double)n);
 }
 
+// Bias gradients: the FP64 sums of layer l (32 of them) rounded once
+struct BiasOffsets {
+  int off[kMaxLayers], count[kMaxLayers];
+};
+
+__global__ void bias_round_kernel(const double* sums, BiasOffsets at, float* grads) {
+  const int l = blockIdx.x;
+  if ((int)threadIdx.x < at.count[l]) grads[at.off[l] + threadIdx.x] = (float)sums[32 * l + threadIdx.x];
+}
+
 // Adam on the FP32 master parameters (Kingma & Ba 2015)
 __global__ void adam_kernel(float* w, const float* g, float* m, float* v, int n, float lr, float b1, float b2,
                             float eps, float c1, float c2) {
@@ -331,7 +341,7 @@ struct kp_cnn {
   std::vector<size_t> act_off;
   float* dz = nullptr;                 // [maxB][Cmax][P]
   float* dz2 = nullptr;
-  double* d_loss = nullptr;
+  double* d_loss = nullptr;            // the loss, then [L][32] sums of the bias gradients
   int* d_err = nullptr;
   int Cmax = 0;
   // inference on the implicit-GEMM convolutions of kp_conv_tc.cu (no im2col
@@ -433,7 +443,7 @@ kp_status backward_impl(kp_cnn* n, int B, const float* in, const float* target, 
   kp_status s = forward_impl(n, B, in);
   if (s != KP_OK) return s;
   cudaError_t e = cudaMemsetAsync(n->grads, 0, (size_t)n->nparams * sizeof(float), st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(n->d_loss, 0, sizeof(double), st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(n->d_loss, 0, (1 + 32 * (size_t)n->L) * sizeof(double), st);
   if (e != cudaSuccess) return kp::cuda_error(n->ctx, e, "CNN backward");
   const size_t nout = (size_t)B * P;
   mse_kernel<<<grid_for(nout), 256, 0, st>>>(n->act + n->act_off[n->L - 1], target, n->dz, nout, n->d_loss);
@@ -442,7 +452,7 @@ kp_status backward_impl(kp_cnn* n, int B, const float* in, const float* target, 
   for (int l = n->L - 1; l >= 0; --l) {
     const int cin = n->ch[l], cout = n->ch[l + 1];
     const float* X = l == 0 ? in : n->act + n->act_off[l - 1];
-    e = kp::launch_train_wgrad(X, dZ, B, cin, cout, n->H, n->W, n->grads + n->woff[l], n->grads + n->boff[l], n->d_err,
+    e = kp::launch_train_wgrad(X, dZ, B, cin, cout, n->H, n->W, n->grads + n->woff[l], n->d_loss + 1 + 32 * l, n->d_err,
                                n->ctx->sms, st);
     if (e != cudaSuccess) return kp::cuda_error(n->ctx, e, "CNN backward");
     if (l == 0) break;
@@ -452,6 +462,9 @@ kp_status backward_impl(kp_cnn* n, int B, const float* in, const float* target, 
     if (e != cudaSuccess) return kp::cuda_error(n->ctx, e, "CNN backward");
     std::swap(dZ, dZo);
   }
+  BiasOffsets at{};
+  for (int l = 0; l < n->L; ++l) { at.off[l] = (int)n->boff[l]; at.count[l] = n->ch[l + 1]; }
+  bias_round_kernel<<<n->L, 32, 0, st>>>(n->d_loss + 1, at, n->grads);
   e = cudaGetLastError();
   if (e == cudaSuccess && loss) {
     e = cudaMemcpyAsync(loss, n->d_loss, sizeof(double), cudaMemcpyDeviceToHost, st);
@@ -508,7 +521,7 @@ kp_status kp_cnn_create(kp_ctx* c, int H, int W, int max_batch, int nlayers, con
   if (e == cudaSuccess) e = cudaMalloc((void**)&n->act, nact * sizeof(float));
   if (e == cudaSuccess) e = cudaMalloc((void**)&n->dz, BP * n->Cmax * sizeof(float));
   if (e == cudaSuccess) e = cudaMalloc((void**)&n->dz2, BP * n->Cmax * sizeof(float));
-  if (e == cudaSuccess) e = cudaMalloc((void**)&n->d_loss, sizeof(double));
+  if (e == cudaSuccess) e = cudaMalloc((void**)&n->d_loss, (1 + 32 * (size_t)nlayers) * sizeof(double));
   if (e == cudaSuccess) e = cudaMalloc((void**)&n->d_err, sizeof(int));
   if (e == cudaSuccess) e = cudaMemset(n->d_err, 0, sizeof(int));
   if (e == cudaSuccess) e = cudaMemset(n->params, 0, np * sizeof(float));

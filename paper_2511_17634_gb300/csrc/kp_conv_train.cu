@@ -269,7 +269,7 @@ struct WgradArgs {
   const float* X;              // [B][C][P]
   const float* dZ;             // [B][N][P]
   float* dW;                   // [N][9 C], added to
-  float* db;                   // [N], added to
+  double* db;                  // [N], added to
   int B, C, N, H, W;
   int* err;
 };
@@ -380,7 +380,16 @@ __global__ void __launch_bounds__(kWgThreads, 1) train_wgrad_kernel(const WgradA
       while (xp - lane >= P) { xp -= P; ++xb; }
     }
   };
-  float bsum[2] = {0.f, 0.f};                      // this lane's part of db of outputs warp, warp + 16
+  // this lane's part of db of outputs warp, warp + 16: an FP32 sum and the
+  // errors of its additions (TwoSum, Knuth), since the chain is as long as the
+  // split; the CTAs' sums are added in FP64 (constant gradients at 128x128, batch
+  // 64: 2.2e-6 off with FP32 sums throughout, at most 6e-8 now)
+  float bsum[2] = {0.f, 0.f}, berr[2] = {0.f, 0.f};
+  auto add_b = [&](int u, float v) {
+    const float t = bsum[u] + v, w = t - bsum[u];
+    berr[u] += (bsum[u] - (t - w)) + (v - w);
+    bsum[u] = t;
+  };
   int it = 0;
   if (ch0 < ch1) {
     masks(ch0, msk);
@@ -404,7 +413,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) train_wgrad_kernel(const WgradA
 #pragma unroll
         for (int u = 0; u < 2; ++u)
           if (warp + 16 * u < a.N) {
-            bsum[u] += z[h][0][u] + z[h][1][u];
+            if (h == 0) add_b(u, (z[0][0][u] + z[0][1][u]) + (z[1][0][u] + z[1][1][u]));
             put(Bs + h * 4096, warp + 16 * u, pack(z[h][0][u], z[h][1][u]));
           }
       if (ch + 2 < ch1) load(ch + 2);
@@ -463,10 +472,13 @@ __global__ void __launch_bounds__(kWgThreads, 1) train_wgrad_kernel(const WgradA
   if (mi == 0) {
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
-      float v = bsum[u];
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
-      if (stager && lane == 0 && warp + 16 * u < a.N) atomicAdd(a.db + warp + 16 * u, v);
+      for (int o = 16; o > 0; o >>= 1) {
+        const float e = __shfl_xor_sync(kFull, berr[u], o);
+        add_b(u, __shfl_xor_sync(kFull, bsum[u], o));
+        berr[u] += e;
+      }
+      if (stager && lane == 0 && warp + 16 * u < a.N) atomicAdd(a.db + warp + 16 * u, (double)bsum[u] + (double)berr[u]);
     }
   }
   // warp w: k = lanes 32 (w % 4) .., outputs 8 (w / 4) ..
@@ -506,7 +518,7 @@ cudaError_t launch_train_conv(const float* X, int B, int C, int H, int W, const 
   return cudaGetLastError();
 }
 
-cudaError_t launch_train_wgrad(const float* X, const float* dZ, int B, int C, int N, int H, int W, float* dW, float* db,
+cudaError_t launch_train_wgrad(const float* X, const float* dZ, int B, int C, int N, int H, int W, float* dW, double* db,
                                int* err, int sms, cudaStream_t st) {
   if (C < 1 || C > 32 || N < 1 || N > 32) return cudaErrorInvalidValue;
   WgradArgs a{X, dZ, dW, db, B, C, N, H, W, err};

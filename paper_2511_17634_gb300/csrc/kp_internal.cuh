@@ -704,7 +704,7 @@ cudaError_t launch_conv3x3(const __nv_bfloat16* in, int B, int cic, const __nv_b
 cudaError_t launch_train_conv(const float* X, int B, int C, int H, int W, const __nv_bfloat16* Wb, int ldw, int N,
                               const float* bias, int relu, const float* gate, int sign, float* Y, int* err, int sms,
                               cudaStream_t st);
-cudaError_t launch_train_wgrad(const float* X, const float* dZ, int B, int C, int N, int H, int W, float* dW, float* db,
+cudaError_t launch_train_wgrad(const float* X, const float* dZ, int B, int C, int N, int H, int W, float* dW, double* db,
                                int* err, int sms, cudaStream_t st);
 // Resident blocks per SM of the FP64 solver shape (0 if unknown).
 int gmres_fp64_blocks_per_sm(int ept, int nt, int minb, size_t smem);

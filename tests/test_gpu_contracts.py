@@ -301,3 +301,27 @@ def test_singular_basis_at_a_breakdown_stays_finite(kp, orc, mixed):
     ctx.project_targets(0, 1, ops, _dev(r), x0)
     ref, _ = orc.project(V.cpu().numpy(), Hb, n, hn, r[0])
     assert np.isfinite(ref).all() and np.linalg.norm(x0.cpu().numpy()[0] - ref) <= 1e-6 * np.linalg.norm(ref)
+
+
+# ---- training
+
+@pytest.mark.parametrize("H,W,B,C", [(128, 128, 16, 32), (128, 128, 64, 10), (64, 64, 16, 8), (28, 28, 4, 10),
+                                     (100, 75, 31, 1), (192, 40, 8, 3), (1, 1, 1, 1)])
+def test_bias_gradient_is_summed_beyond_fp32(kp, H, W, B, C):
+    # one layer with zero weights: the output gradients are 2 / n (0 - t) in
+    # FP32, known exactly.  Four of them are added in FP32 (two roundings deep),
+    # everything above is exact to FP64 and rounded once: 3 2^-24 of the sum of
+    # magnitudes
+    rng = np.random.default_rng(B + C)
+    net = kp.CNN(kp.Context(max_seeds=1, max_n=16384), H, W, channels=(C, 1), max_batch=B)
+    net.set_params(np.zeros(net.nparams, np.float32))
+    x = torch.zeros((B, C, H * W), dtype=torch.float32, device="cuda")
+    grads = torch.zeros(net.nparams, dtype=torch.float32, device="cuda")
+    n = B * H * W
+    for t in (np.full(n, 1.01), np.full(n, 1 / 3), rng.normal(size=n), 3.7 + 0.01 * rng.normal(size=n)):
+        t = t.astype(np.float32)
+        for _ in range(2):                        # the second on the sums that the first left
+            net.gradients(x, torch.as_tensor(t, device="cuda").reshape(B, 1, -1), grads)
+        torch.cuda.synchronize()
+        dz = (np.float32(2) / np.float32(n) * (np.float32(0) - t)).astype(np.float64)
+        assert abs(float(grads[-1]) - dz.sum()) <= 3 * 2.0 ** -24 * np.abs(dz).sum()
