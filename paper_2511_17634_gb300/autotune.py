@@ -4,8 +4,10 @@ workload by timing a few calibration timesteps of the real march, and caches
 the choice in a JSON file keyed by (device, grid sizes, batch, precision).
 
 Candidates: m in {20, 30, 40, 60} x shared-memory window in {auto, small} x
-(threads per system, resident blocks per SM) in {(256, 2), (128, 3), (128, 4),
-(64, 4)} (FP64 grids of up to 1024 points; one shape otherwise).
+(threads per system, resident blocks per SM) in {automatic, (256, 2), (128, 2),
+(128, 3), (128, 4), (64, 4)} (FP64 grids of up to 1024 points; one shape
+otherwise).  The automatic shape depends on the number of systems, so it is a
+candidate of its own.
 The timing runs through the C ABI (kp_march_*) on the GPU; only the choice of
 the fastest candidate and the cache are host logic.
 """
@@ -15,8 +17,8 @@ import json
 import os
 
 M_CANDIDATES = (20, 30, 40, 60)
-WINDOW_CANDIDATES = (0, 6)      # 0 = automatic (two blocks per SM when N <= 1024)
-SHAPE_CANDIDATES = ((256, 2), (128, 3), (128, 4), (64, 4))   # (threads, blocks per SM), N <= 1024
+WINDOW_CANDIDATES = (0, 6)      # 0 = automatic (as many vectors as the blocks that share an SM leave room for)
+SHAPE_CANDIDATES = ((0, 0), (256, 2), (128, 2), (128, 3), (128, 4), (64, 4))   # (threads, blocks per SM), N <= 1024
 
 
 def cache_key(device: str, grids, nseed: int, ntgt: int, precision: str, mode: int) -> str:

@@ -89,3 +89,12 @@ def test_mixed_grid_is_what_its_kernel_keeps_resident(shapes):
         assert (s["cs"], s["minb"]) == {4096: (0, 3), 8192: (2, 2), 16384: (4, 3)}[r[0]]
         if r[1] <= 40:
             assert _fits(s), (r, s)
+
+
+def test_autotuner_can_choose_what_the_solver_would(shapes):
+    # the automatic shape, and every shape that a march's rule comes to
+    from paper_2511_17634_gb300 import autotune
+    assert (0, 0) in autotune.SHAPE_CANDIDATES
+    rows = [(1024, 40, 0, 32, 32, 1, count, 0, win, 0, 0, 0, 0) for count in (4, 152, 153, 230, 304, 305, 5000) for win in (0, 1)]
+    for s in shapes(rows):
+        assert (s["nt"], s["minb"]) in autotune.SHAPE_CANDIDATES, s
