@@ -36,10 +36,16 @@ kp_status cuda_error(kp_ctx* c, cudaError_t e, const char* what) {
 }
 
 cudaError_t launch_solver(const GmresParams& p, const Shape& sh, bool mixed, cudaStream_t st) {
-  if (sh.cs > 0) return launch_gmres_cluster(p, sh.ept, sh.nt, sh.cs, sh.reg, sh.smem, st);
+  if (sh.cs > 0) return launch_gmres_cluster(p, sh.ept, sh.nt, sh.cs, sh.reg, sh.long_columns, sh.smem, st);
   return mixed ? launch_gmres_mixed(p, sh.ept, sh.nt, sh.reg, sh.smem, st)
                : launch_gmres_fp64(p, sh.ept, sh.nt, sh.minb, sh.smem, st);
 }
+
+// Columns longer than this (half a block's threads: a halo point per thread
+// costs next to nothing up to there) have their halos stored by the neighbours:
+// 129x96, 270 systems, g = 0.5, 8.3 -> 7.6 ms.  See LONG in
+// kp_gmres_mixed_kernel.cuh.
+constexpr int kLongColumn = 128;
 
 kp_status gmres_shape(kp_ctx* c, int nmax, int m, Shape* out, bool mixed, int wmin, int hmax,
                       bool one_size, int count, bool one_launch, bool windows) {
@@ -139,10 +145,11 @@ kp_status gmres_shape(kp_ctx* c, int nmax, int m, Shape* out, bool mixed, int wm
       share = 3;
     }
     sh.vld += 2 * sh.hmax;
+    sh.long_columns = sh.cs && !sh.reg && hmax > kLongColumn;
     if (!share) share = sh.minb;
   }
   auto bytes = [&](int S) {
-    return mixed ? gmres_mixed_smem_bytes(sh.nt, sh.ctas(), sh.hmax, sh.vld, S, m)
+    return mixed ? gmres_mixed_smem_bytes(sh.nt, sh.ctas(), sh.long_columns ? 0 : sh.hmax, sh.vld, S, m)
                  : gmres_fp64_smem_bytes(sh.ept, sh.nt, S, m);
   };
   // shared memory of one CTA when minb (share) of them are on an SM (1 KB per
@@ -168,7 +175,7 @@ kp_status gmres_shape(kp_ctx* c, int nmax, int m, Shape* out, bool mixed, int wm
   // a time: a round of values is a cluster barrier (101x80, 27 systems with g =
   // 0.5: 4.01 -> 3.84 ms)
   for (int v = sh.redv + 4; sh.cs && v < m + 5; v += 4) {
-    const size_t need = gmres_mixed_smem_bytes(sh.nt, sh.ctas(), sh.hmax, sh.vld, S, m, v);
+    const size_t need = gmres_mixed_smem_bytes(sh.nt, sh.ctas(), sh.long_columns ? 0 : sh.hmax, sh.vld, S, m, v);
     if (need > budget) break;
     sh.redv = v;
     sh.smem = need;

@@ -86,6 +86,7 @@ struct Shape {
   int redv = 8;   // mixed precision, clusters: values per reduction round
   int hmax = 0;   // longest column of the systems (mixed precision with halo columns)
   bool reg = false;   // mixed precision: see launch_gmres_mixed
+  bool long_columns = false;   // see launch_gmres_cluster
   int ctas() const { return cs ? cs : 1; }
   // mixed precision: CTAs of a launch over nsys systems (as many as are
   // resident; they claim systems) and so slices of workspace

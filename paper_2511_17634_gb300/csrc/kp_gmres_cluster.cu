@@ -6,8 +6,9 @@
 
 namespace kp {
 
-cudaError_t launch_gmres_cluster(const GmresParams& p, int ept, int nt, int cs, bool reg, size_t smem,
-                                 cudaStream_t st) {
+cudaError_t launch_gmres_cluster(const GmresParams& p, int ept, int nt, int cs, bool reg, bool long_columns,
+                                 size_t smem, cudaStream_t st) {
+  if (long_columns) return reg ? cudaErrorInvalidValue : launch_gmres_cluster_long(p, ept, nt, cs, smem, st);
   if (ept == 16 && nt == 256) {                  // the default: 4096 points per CTA
     if (cs == 4) return reg ? launch_mx<16, 256, 4, mixed_reg_blocks(4), 2, true>(p, smem, st) : launch_mx<16, 256, 4, 2, 2, false>(p, smem, st);
     if (cs == 2) return reg ? launch_mx<16, 256, 2, mixed_reg_blocks(2), 2, true>(p, smem, st) : launch_mx<16, 256, 2, 2, 2, false>(p, smem, st);

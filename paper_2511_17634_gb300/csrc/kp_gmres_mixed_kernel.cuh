@@ -175,8 +175,12 @@ __device__ __forceinline__ void solve_projected_dd(float2* c, int a, int nrot, c
 // NT) and its columns divide the CTA's threads, so that all of a thread's
 // points share one row j: two neighbour flags per thread instead of four bits
 // per point, no guards, and zero halo columns beside the grid (the launcher
-// decides).
-template <int EPT, int NT, int CS, int MINB, int HALF, bool REG>
+// decides).  LONG (clusters, columns of more than half a block's threads): the
+// halo columns of x and of every v are stored by the neighbour that has them,
+// for one cluster barrier more per Arnoldi step; kept up here they would be
+// 2 H more points per CTA (100 systems of 1024x16, warm: 9.0 -> 7.2 ms, 50 of
+// 2048x8 20.4 -> 8.6).
+template <int EPT, int NT, int CS, int MINB, int HALF, bool REG, bool LONG = false>
 __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams p) {
   namespace cg = cooperative_groups;
   constexpr int NH = HALF ? 2 : 1;
@@ -205,8 +209,8 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
   const int redv = CS > 1 ? p.red_v : kRedV;
   float* yf = red + 2 * redv * P;                             // [kMaxV] combination coefficients
   int* fl = reinterpret_cast<int*>(yf + kMaxV);               // [8]
-  float* whalo = reinterpret_cast<float*>(fl + 8);            // [2][2 hmax] pushed edge columns
-  float2* Hr = reinterpret_cast<float2*>(whalo + 4 * p.hmax); // packed columns of R: j at j (j + 1) / 2
+  float* whalo = reinterpret_cast<float*>(fl + 8);            // [2][2 hmax] pushed edge columns (not LONG)
+  float2* Hr = reinterpret_cast<float2*>(whalo + (LONG ? 0 : 4 * p.hmax)); // packed columns of R: j at j (j + 1) / 2
   float* V = reinterpret_cast<float*>(Hr + m * (m + 1) / 2);  // [S][vld]
   const int vld = p.vld;
   // workspace of this CTA: x (hi, lo) over the extended slice, q_x and q_y
@@ -266,10 +270,16 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
     // steps: 101x80, 270 systems with g = 0.5, 4.73 -> 3.08 ms), which takes
     // finite values behind the halo too
     const bool full = REG || CS == 1 || SL == EPT * NT;
-    if (!full && zeroed != SL + 2 * H) {
-      zeroed = SL + 2 * H;
-      for (int i = 0; i <= m; ++i)
+    if ((LONG || !full) && zeroed != SL * 4096 + H) {
+      zeroed = SL * 4096 + H;                    // (H <= 2048)
+      for (int i = 0; i <= m; ++i) {
         for (int q = SL + 2 * H + tid; q < vld; q += NT) slot(i)[q] = 0.f;
+        // (LONG: nobody stores the halo outside the grid)
+        for (int q = tid; LONG && q < H; q += NT) {
+          if (rank == 0) slot(i)[q] = 0.f;
+          if (rank == CS - 1) slot(i)[H + SL + q] = 0.f;
+        }
+      }
     }
     // the operator constants c = g^2/(2h^2), e = c/4, c_d = 1/dt + 4c from the
     // descriptor's quotients: a division is a dozen FP64 instructions on
@@ -300,7 +310,7 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
         for (int u = 0; u < B; ++u)
           if (inside(k0 + u)) put(hal + lp(k0 + u), v[u]);
       }
-      if (CS > 1)
+      if (CS > 1 && !LONG)
         for (int q = tid; q < 2 * H; q += NT) {
           const int pp = q < H ? base - H + q : base + SL + q - H, at = q < H ? q : SL + q;
           put(at, get(at, (unsigned)pp < (unsigned)N ? pp : -1));
@@ -310,10 +320,24 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
     // first two vector slots
     float* xh = V;
     float* xl = V + vld;
+    // LONG: fn(r, at): point l of the slice is at index at of CTA r's halo
+    auto to_neighbours = [&](int l, auto&& fn) {
+      if (LONG && rank > 0 && l < H) fn(rank - 1, H + SL + l);
+      if (LONG && rank + 1 < CS && l >= SL - H) fn(rank + 1, l - (SL - H));
+    };
     auto put_x = [&](int at, dd v) {
       xh[at] = v.hi;
       xl[at] = v.lo;
       xs[at] = as_f2(v);
+      to_neighbours(at - hal, [&](int r, int o) {
+        float* n = cluster.map_shared_rank(V, r) + o;
+        n[0] = v.hi;
+        n[vld] = v.lo;
+      });
+    };
+    auto sync_x = [&]() {                        // every CTA's reads or stores of x on the halo are done
+      if (LONG) cluster.sync();
+      else __syncthreads();
     };
     // x = u + yf-combination of the nc rows U (indexed by grid point)
     auto add_basis = [&](const float* U, int nc, bool from_zero) {
@@ -367,7 +391,7 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
 
     // the lagged field, then q_x, q_y (hi parts in registers for the Krylov
     // operator, low parts in the workspace for the residual)
-    if (CS > 1) {
+    if (CS > 1 && !LONG) {
       // (both buffers whole: nobody pushes the halo outside the grid, and a
       // system before this one may have had longer columns)
       for (int q = tid; q < 4 * p.hmax; q += NT) whalo[q] = 0.f;
@@ -424,7 +448,7 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
     // push this CTA's edge columns of w to the neighbours' halo buffers
     // (visible after the next cluster barrier)
     auto push_edges = [&]() {
-      if (CS == 1) return;
+      if (CS == 1 || LONG) return;
       float* wl = rank > 0 ? cluster.map_shared_rank(whalo, rank - 1) + hbuf * 2 * p.hmax + H : nullptr;
       float* wr = rank + 1 < CS ? cluster.map_shared_rank(whalo, rank + 1) + hbuf * 2 * p.hmax : nullptr;
 #pragma unroll
@@ -536,7 +560,7 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
       }
     };
     if (p.x0_mode != X0_WARM && !judge) {
-      __syncthreads();                           // every read of the lagged field in the slots is done
+      sync_x();                                  // every read of the lagged field in the slots is done
       if (p.x0_mode == X0_READ) load_guess();
       else load_x(nullptr);
     }
@@ -586,7 +610,7 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
     const float hsc = (cde > 0 && cde < 254) ? __uint_as_float((254u - cde) << 23) : 1.f;
 #pragma unroll 1
     for (;;) {
-      __syncthreads();                           // x complete for the stencil
+      sync_x();                                  // x complete for the stencil
       const bool no_x = phase == kProject || (p.x0_mode == X0_ZERO && outer == 0);
       // r = b - A x in double-float: the hi parts of the terms are added by
       // TwoSum and all low parts and errors in FP32; the FP32 value of r,
@@ -645,7 +669,7 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
       }
       if (phase == kWarm) {
         sumsq(sw);
-        __syncthreads();                         // every read of the warm start in the slots is done
+        sync_x();                                // every read of the warm start in the slots is done
         load_guess();
         phase = kGuess;
         continue;
@@ -755,13 +779,17 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
           const int l = lp(k);
           const float v = w[k] * scale;
           if (full || inside(k)) vn[hal + l] = v;
+          if (LONG && inside(k))
+            to_neighbours(l, [&](int r, int o) {
+              (n < p.S ? cluster.map_shared_rank(vn, r) : vn + (r - rank) * (long long)p.ws_ld)[o] = v;
+            });
           if (keep && inside(k)) {
             capV[(size_t)n * p.cap_ld + base + l] = v;
             if (p.capVb && n < kVbRows)
               p.capVb[((size_t)cidx * kVbRows + n) * p.capVb_ld + base + l] = __float2bfloat16_rn(v);
           }
         }
-        if (CS > 1) {
+        if (CS > 1 && !LONG) {
           const float* wh = whalo + hbuf * 2 * p.hmax;
           for (int q = tid; q < 2 * H; q += NT) vn[q < H ? q : SL + q] = wh[q] * scale;
         } else if (REG && n >= p.S) {
@@ -774,7 +802,9 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
       dd gcur = rnorm;                           // running right-hand side (warp 0)
 #pragma unroll 1
       for (int j = 0; j < m; ++j) {
-        __syncthreads();                         // v_j complete (own slice and halo)
+        // v_j complete (own slice and halo; LONG: by the barrier that ends a step)
+        if (!LONG) __syncthreads();
+        else if (j == 0) cluster.sync();
         {
           auto apply = [&](const float* v) {
 #pragma unroll
@@ -845,7 +875,7 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
           // latency per vector (L2 past the window; 128x128, 300 systems, warm:
           // 1126 -> 1097 us, 2048x8 36.6 -> 22.7 ms)
           float* wh = whalo + hbuf * 2 * p.hmax;
-          const bool hq = CS > 1 && tid < 2 * H;
+          const bool hq = CS > 1 && !LONG && tid < 2 * H;
           float hv = hq ? wh[tid] : 0.f;
 #pragma unroll 1
           for (int i = 0; i < nh; ++i) {
@@ -862,7 +892,7 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
 #pragma unroll
             for (int k = 0; k < EPT; ++k) w[k] = inside(k) ? w[k] : 0.f;
           if (hq) wh[tid] = hv;
-          if (CS > 1) {
+          if (CS > 1 && !LONG) {
             constexpr int B = REG ? 1 : 8;       // (REG: H <= NT)
 #pragma unroll 1
             for (int q0 = tid + NT; q0 < 2 * H; q0 += B * NT) {
@@ -933,7 +963,7 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
           __syncwarp();
         }
         kdone = j + 1;
-        __syncthreads();
+        sync_x();
         if (fl[0]) break;
       }
       // y = R^{-1} g: column-oriented back substitution on warp 0 (lane l
@@ -1049,7 +1079,7 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
         if (status != KP_OK) atomicAdd(&a->not_converged, 1u);
       }
     }
-    __syncthreads();                             // shared memory is reused by the next system
+    sync_x();                                    // shared memory is reused by the next system
   }
   if (tid == 0 && rank == 0 && atomicAdd(p.claim + 1, 1) == (int)gridDim.x / CS - 1) {
     p.claim[0] = 0;                              // the last to finish: ready for the next launch
@@ -1058,9 +1088,9 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
   if (CS > 1) cluster.sync();                    // no CTA leaves while others write its memory
 }
 
-template <int EPT, int NT, int CS, int MINB, int HALF, bool REG>
+template <int EPT, int NT, int CS, int MINB, int HALF, bool REG, bool LONG = false>
 cudaError_t launch_mx(const GmresParams& p, size_t smem, cudaStream_t st) {
-  auto k = gmres_mixed_kernel<EPT, NT, CS, MINB, HALF, REG>;
+  auto k = gmres_mixed_kernel<EPT, NT, CS, MINB, HALF, REG, LONG>;
   int dev = 0, optin = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);

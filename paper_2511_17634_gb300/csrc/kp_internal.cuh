@@ -643,8 +643,10 @@ constexpr int mixed_reg_blocks(int cs) { return cs == 2 ? 2 : 3; }
 // reg: every system fills its CTAs and its columns divide a sub-block (the REG kernels).
 cudaError_t launch_gmres_mixed(const GmresParams& p, int ept, int nt, bool reg, size_t smem, cudaStream_t st);
 // Cluster of cs CTAs per system (grids above 4096 unknowns, or on request).
-cudaError_t launch_gmres_cluster(const GmresParams& p, int ept, int nt, int cs, bool reg, size_t smem,
-                                 cudaStream_t st);
+// long_columns: the kernels whose halos the neighbours store (LONG).
+cudaError_t launch_gmres_cluster(const GmresParams& p, int ept, int nt, int cs, bool reg, bool long_columns,
+                                 size_t smem, cudaStream_t st);
+cudaError_t launch_gmres_cluster_long(const GmresParams& p, int ept, int nt, int cs, size_t smem, cudaStream_t st);
 // The N <= 1024 instantiation (4 points x 256 threads) on an explicit grid;
 // the kernel strides over systems, block b using Krylov workspace slice b.
 cudaError_t launch_gmres_fp64_1k_grid(const GmresParams& p, size_t smem, int grid,
