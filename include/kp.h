@@ -70,7 +70,8 @@ typedef struct {
   int max_n;         /* largest N = H*W any call will pass (<= 16384)             */
   int precision;     /* kp_precision                                              */
   int smem_vectors;  /* Krylov vectors held in shared memory per system; the rest
-                        live in a device workspace (0 = choose automatically)      */
+                        live in a device workspace (0 = choose automatically;
+                        mixed precision holds at least 3)                          */
   int reorth;        /* 0: CGS2, two classical Gram-Schmidt passes every step;
                         1: second pass only when the first removed more than
                         half of the vector's norm (Daniel-Gragg-Kaufman-Stewart)  */
@@ -81,7 +82,12 @@ typedef struct {
                         windows one per SM up to one and a half --, else 128
                         with 4, or 256 with 3 where one call then leaves fewer
                         slots empty) or 256 with 4 (mixed precision; 64 counts as
-                        128 there)                                           */
+                        128 there).  The FP64 shapes add a system's partial sums
+                        in different orders, so with 0 the last bits of an FP64
+                        solve depend on how many systems share the call or plan
+                        (a shard need not equal the whole); an explicit value
+                        keeps them the same in any batch.  Mixed-precision
+                        shapes chosen by rule have the same bits.            */
   int blocks_per_sm; /* resident solver blocks per SM for grids of <= 1024
                         points (caps registers per thread and sizes the
                         shared-memory window): 256 threads: 2 or 3; 128: 2, 3

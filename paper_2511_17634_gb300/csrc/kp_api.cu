@@ -80,7 +80,12 @@ kp_status gmres_shape(kp_ctx* c, int nmax, int m, Shape* out, bool mixed, int wm
       else if (count <= 2 * c->sms) { sh.minb = 2; alone = windows && 2 * count <= 3 * c->sms; }
       else if (one_launch && 3 * rounds3 < 4 * rounds4) { sh.nt = 256; sh.ept = 4; sh.minb = 3; }
     }
-    if (mixed) {                                 // the FP32 solver has the 256- and 128-thread shapes
+    // The FP32 solver has the 256- and 128-thread shapes, four blocks per SM: 64
+    // registers a thread and spills of 700 bytes, but the blocks overlap each
+    // other's barriers.  Eight timesteps against two blocks with FP64 scalars
+    // before: 28x28, 683 targets, projected 1359 -> 1084 us, warm 1062 -> 690; 4
+    // targets 622 -> 566; 32x32x3, 768 targets 1398 -> 987 and 1085 -> 640.
+    if (mixed) {
       if (sh.nt == 64) { sh.nt = 128; sh.ept = 8; }
       sh.minb = 4;
     }
@@ -112,8 +117,9 @@ kp_status gmres_shape(kp_ctx* c, int nmax, int m, Shape* out, bool mixed, int wm
       // faster per round of a full chip, two rounds of them against one
       // (101x80: 56 systems 480 -> 265 us, 100 528 -> 489, 165 987 -> 668;
       // 152, one full round against three, 541 -> 672; 110x96: 300 systems
-      // 2492 -> 2210).  Two CTAs share an SM; larger clusters leave a tenth of
-      // the places empty.
+      // 2492 -> 2210; one size of those tried loses, 84x88, 539 systems, learned,
+      // by 1.5 %).  Two CTAs share an SM; larger clusters leave a tenth of the
+      // places empty.
       const long long full = (long long)count * sh.cs;
       auto rounds = [&](long long ctas, int cs) {
         const long long slots = cs == 2 ? 2 * c->sms : 2 * c->sms * 9 / 10;
@@ -348,7 +354,6 @@ kp_status run_gmres(kp_ctx* c, int nsys, const kp_op* ops, const double* const* 
   kp::set_shape(&p, sh);
   p.reorth = c->opt.reorth;
   p.inner_eta = kp::inner_eta(c->opt);
-  p.b_scale = 1.0;
   p.x0_mode = kp::X0_READ;
   p.spill = (!mixed && sh.ws) ? c->spill : nullptr;
   p.spill32 = mixed ? c->spill32 : nullptr;

@@ -135,10 +135,10 @@ __global__ void __launch_bounds__(NT, MINB) gmres_fp64_kernel(const GmresParams 
     const int parity_base = slot_set_base(p, tstep);
     const SysDesc d = p.sys_par[0] ? p.sys_par[(tstep + p.sys_shift) & 1][sysi] : p.sys[sysi];
     const int H = d.H, W = d.W, N = H * W;
-    // the system is solved as (A / s) x = b / s with s = b_scale (the march's
-    // 1/dt): the right-hand side is read as stored and the scale is in the
-    // descriptor's quotients, from which the four operator constants take two
-    // instructions (five FP64 divisions on every warp were 7 % of a solve)
+    // the system is solved as (A / s) x = b / s with s = 1/dt in a march, else 1:
+    // the right-hand side is read as stored and the scale is in the descriptor's
+    // quotients, from which the four operator constants take two instructions
+    // (five FP64 divisions on every warp were 7 % of a solve)
     const double g2 = p.step ? p.g2_sched[tstep] : d.g2;
     const double cc = g2 * d.kc;
     const double ee = 0.25 * cc;

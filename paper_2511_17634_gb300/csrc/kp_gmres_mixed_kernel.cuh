@@ -49,12 +49,14 @@
 // share an SM (two in general), so that one system's barriers and serial work
 // overlap the others' vector work.
 //
-// What bounds it now is issue and latency: 45 % of the issue slots are used.
-// Before (one CTA per SM, FP64 scalars, halos read across the cluster) eight
-// timesteps of 3072 channels of 64x64 took 16.5 ms, now 8.4; four of 128x128
-// 38.8, now 19.0.  16 points a thread rather than 8 took the instructions per
-// system from 235 to 170 thousand; the long loops stay rolled, since unrolled
-// code of that length stalled on instruction fetch (10.2 ms against 8.9).
+// What bounds it is issue and latency: 45 % of the issue slots are used.  Eight
+// timesteps of 3072 channels of 64x64 take 8.2 ms, four of 128x128 18.2 (with
+// one CTA per SM, FP64 scalars and halos read across the cluster 16.5 and
+// 38.8).  16 points a thread rather than 8 take 170 instead of 235 thousand
+// instructions per system; the long loops stay rolled, since unrolled code of
+// that length stalls on instruction fetch (10.2 ms against 8.9).  Systems of 30
+// and more steps are bound by the Krylov vectors past the window (L2, or memory
+// with many systems): 90 of 101x80 with g = 0.5 take 1.5 ms a timestep.
 //
 // The operator is applied from q_x = f_x/(2h) - e (m~_E - m~_W) and q_y per
 // point:
@@ -283,8 +285,8 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
     }
     // the operator constants c = g^2/(2h^2), e = c/4, c_d = 1/dt + 4c from the
     // descriptor's quotients: a division is a dozen FP64 instructions on
-    // every warp.  Solved as (A / s) x = b / s with s = b_scale: the scale is
-    // in those quotients instead of on every point of b.
+    // every warp.  Solved as (A / s) x = b / s with s = 1/dt in a march, else 1:
+    // the scale is in those quotients instead of on every point of b.
     const double g2 = p.step ? p.g2_sched[tstep] : d.g2;
     const double cc = g2 * d.kc;
     const dd ccd = dd_from_double(cc), cdd = dd_from_double(fma(4.0, cc, d.kd));

@@ -112,7 +112,6 @@ struct GmresParams {
   const double* g2_sched;   // if step: g2 = g2_sched[*step + step_offset] for every system
   int step_offset;          // seeds run one timestep ahead of the targets
   const int* step_end;      // if step: nothing to do when *step + step_offset >= *step_end
-  double b_scale;           // right-hand side = b[p] * b_scale (b = m^{n-1}/dt when f = 0)
   int x0_mode;              // X0_* below
   // seed-basis store: projection source (X0_PROJECT) and fused capture (factor)
   double* slotV;            // [max_seeds][max_a + 1][slot_ld]
@@ -135,7 +134,7 @@ struct GmresParams {
   const float* slotV32;     // [max_seeds][max_a + 1][slot_ld] FP32 seed bases
   const float* cproj;       // if set: c = V^T b per target, [nsys][cproj_ld] (tensor-core GEMM)
   int cproj_ld;
-  __nv_bfloat16* bnext;     // if set: write BF16 (x * b_scale) per system, [nsys][bnext_ld]
+  __nv_bfloat16* bnext;     // if set: write BF16 x per system, [nsys][bnext_ld] (the next b, unscaled)
   int bnext_ld;
   __nv_bfloat16* capVb;     // if set: BF16 copy of the captured basis, [slot][kVbRows][capVb_ld]
   int capVb_ld;
@@ -681,7 +680,7 @@ struct CycleParams {
   int step_offset, win;
   const int* step_end;
   const double* g2_sched;
-  double b_scale;           // the solvers' right-hand-side scale: A_proj of A / b_scale
+  double b_scale;           // the solvers' scale s (set_quotients): A_proj of A / s
   int slot_sets;            // slot of seed s at t: (t mod slot_sets) * ns + s
   float* scratch;           // [gridDim.x][max_a][ld] FP32 kept vectors
 };

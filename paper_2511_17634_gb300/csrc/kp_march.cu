@@ -150,7 +150,6 @@ kp::GmresParams solver_params(kp_march_plan* P, bool seeds, int par, int offset,
   g.g2_sched = P->g2;
   g.step_offset = offset;
   g.step_end = P->step + 1;
-  g.b_scale = (double)P->opt.T;               // b = m^{n-1} / dt with dt = 1/T
   g.slotV = c->slotV;
   g.slotMeta = c->slotMeta;
   g.slotR = c->slotR;
@@ -642,11 +641,13 @@ kp_status kp_march_create(kp_ctx* c, int ngroups, const kp_group* groups, const 
       P->cls[0].count = nbig;
       P->cls[1].first = nbig;
       P->cls[1].count = nsmall;
-      // (a point of the larger grids costs 1.2 times one of the smaller: one
+      // (a point of the larger grids costs more than one of the smaller: one
       // 512-thread block per SM hides less of its barriers and serial work
-      // than four of 128.  28x28 / 32x32 / 64x64 mix: 35.7 against 30.1 ns
-      // per point, step and SM; with equal weights the small class ended 15 %
-      // earlier and its SMs idled)
+      // than four of 128.  1.2 against equal weights, 16 timesteps, three modes
+      // each: 28x28 / 32x32 / 64x64 45.2 -> 43.8 ms, 683 of 28x28 and 100 of
+      // 64x64 6.37 -> 6.15, 32x32x3 and 300 of 48x48x3 29.6 -> 27.6, 3072 of
+      // 32x32 and 200 of 64x64 19.2 -> 17.0; 0.3 % slower at most where the
+      // larger grids have most of the work)
       wB *= 1.2;
       const int share = (int)(c->sms * wB / (wA + wB) + 0.5);
       P->cls[0].grid = std::max(1, std::min(std::min(nbig, c->sms - 1), share));
@@ -747,7 +748,7 @@ kp_status kp_march_create(kp_ctx* c, int ngroups, const kp_group* groups, const 
         const size_t off = P->seed_off[gi] + (size_t)k * N;
         SysDesc d{};
         d.H = g.H; d.W = g.W; d.dt = dt; d.g2 = 0.0; d.h = 1.0 / g.H;
-        kp::set_quotients(&d, (double)o.T);   // scaled as b (b_scale)
+        kp::set_quotients(&d, (double)o.T);   // b = m^{n-1} / dt, dt = 1 / T
         d.mt = P->S[1 - par] + off;
         d.b = d.mt;
         d.x = P->S[par] + off;
@@ -758,7 +759,7 @@ kp_status kp_march_create(kp_ctx* c, int ngroups, const kp_group* groups, const 
         const size_t off = P->tgt_off[gi] + (size_t)k * N;
         SysDesc d{};
         d.H = g.H; d.W = g.W; d.dt = dt; d.g2 = 0.0; d.h = 1.0 / g.H;
-        kp::set_quotients(&d, (double)o.T);   // scaled as b (b_scale)
+        kp::set_quotients(&d, (double)o.T);   // b = m^{n-1} / dt, dt = 1 / T
         d.mt = P->Tt[par] + off;
         d.b = d.mt;
         d.x = P->Tt[1 - par] + off;

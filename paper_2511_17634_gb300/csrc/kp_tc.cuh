@@ -76,10 +76,9 @@ __host__ __device__ constexpr uint32_t idesc_f16(int M, int N) {
 // Issued from warp-uniform code: every lane of the issuing warp runs it, one
 // issues.  (No memory clobber: the MMA reads shared memory through the async
 // proxy, and volatile asm keeps it ordered after the barrier waits and fences
-// and before the commit that publishes its completion.)  The descriptors then
-// stay in uniform registers; computed by one lane in a divergent branch they
-// are moved there for every MMA, which took about 118 cycles per MMA where the
-// tensor core needs 46 (N = 48) to 56 (N = 96).
+// and before the commit that publishes its completion.)  Issued by one lane in
+// a divergent branch the convolutions took about 118 cycles per MMA; the tensor
+// core needs 46 (N = 48) to 56 (N = 96).
 __device__ __forceinline__ void mma_f16_one(bool issue, uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
   asm volatile(
       "{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n"

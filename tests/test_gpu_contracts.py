@@ -325,3 +325,25 @@ def test_bias_gradient_is_summed_beyond_fp32(kp, H, W, B, C):
         torch.cuda.synchronize()
         dz = (np.float32(2) / np.float32(n) * (np.float32(0) - t)).astype(np.float64)
         assert abs(float(grads[-1]) - dz.sum()) <= 3 * 2.0 ** -24 * np.abs(dz).sum()
+
+
+# ---- bits and batches
+
+@pytest.mark.parametrize("H,W,counts,opt", [
+    (32, 32, (1, 160, 400, 700), {"block_threads": 128}), (28, 28, (3, 200), {"block_threads": 256}),
+    (28, 28, (1, 700), {"mixed": 1}), (48, 40, (1, 400), {"mixed": 1}), (64, 64, (1, 500), {"mixed": 1}),
+    (101, 80, (1, 90, 150), {"mixed": 1}), (128, 128, (1, 28, 29, 120), {"mixed": 1}), (129, 96, (1, 150), {"mixed": 1})])
+def test_a_system_has_the_same_bits_in_any_batch(kp, H, W, counts, opt):
+    # an explicit FP64 shape; the mixed-precision shapes that the rule chooses
+    opt = dict(opt)
+    prec = kp.PREC_MIXED if opt.pop("mixed", 0) else kp.PREC_FP64
+    rng = np.random.default_rng(H)
+    mt, b = _dev(rng.uniform(0, 1, (1, H * W))), _dev(rng.normal(size=(1, H * W)))
+    ref = None
+    for n in counts:
+        ctx = kp.Context(max_n=16384, precision=prec, **opt)
+        x = torch.zeros((n, H * W), dtype=torch.float64, device="cuda")
+        ctx.refine(kp.make_ops(H, W, 1e-3, 0.02, 1.0 / H, mt.repeat(n, 1)), b.repeat(n, 1), x, tol=1e-9, m=30)
+        torch.cuda.synchronize()
+        ref = x[0].clone() if ref is None else ref
+        assert bool((x == ref).all()), n
