@@ -231,7 +231,7 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
   const int parity_base = slot_set_base(p, tstep);
   const float kEta = p.inner_eta > 0.0 ? (float)p.inner_eta : 1e-5f;
   int buf = 0, hbuf = 0;                         // parities of the reductions and of the halo pushes
-  int zeroed = -1;                               // where the zeros of the slots begin (short slices)
+  int geometry = -1, zeroed = 0;                 // slots whose space behind the halo is zero, for these slices
 
   // resident CTAs claim systems until none is left: the workspace is then as
   // large as the GPU holds CTAs and stays in L2 (a slice per system was 7 GB
@@ -272,16 +272,18 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
     // steps: 101x80, 270 systems with g = 0.5, 4.73 -> 3.08 ms), which takes
     // finite values behind the halo too
     const bool full = REG || CS == 1 || SL == EPT * NT;
-    if ((LONG || !full) && zeroed != SL * 4096 + H) {
-      zeroed = SL * 4096 + H;                    // (H <= 2048)
-      for (int i = 0; i <= m; ++i) {
-        for (int q = SL + 2 * H + tid; q < vld; q += NT) slot(i)[q] = 0.f;
-        // (LONG: nobody stores the halo outside the grid)
-        for (int q = tid; LONG && q < H; q += NT) {
-          if (rank == 0) slot(i)[q] = 0.f;
-          if (rank == CS - 1) slot(i)[H + SL + q] = 0.f;
-        }
+    auto zero_outside = [&](int n) {
+      float* v = slot(n);
+      for (int q = SL + 2 * H + tid; q < vld; q += NT) v[q] = 0.f;
+      for (int q = tid; LONG && q < H; q += NT) {   // (LONG: nobody stores the halo outside the grid)
+        if (rank == 0) v[q] = 0.f;
+        if (rank == CS - 1) v[H + SL + q] = 0.f;
       }
+    };
+    if ((LONG || !full) && geometry != SL * 4096 + H) {   // (H <= 2048)
+      geometry = SL * 4096 + H;
+      zeroed = 0;
+      for (; LONG && zeroed < 2; ++zeroed) zero_outside(zeroed);   // x
     }
     // the operator constants c = g^2/(2h^2), e = c/4, c_d = 1/dt + 4c from the
     // descriptor's quotients: a division is a dozen FP64 instructions on
@@ -790,6 +792,10 @@ __global__ void __launch_bounds__(NT, MINB) gmres_mixed_kernel(const GmresParams
             if (p.capVb && n < kVbRows)
               p.capVb[((size_t)cidx * kVbRows + n) * p.capVb_ld + base + l] = __float2bfloat16_rn(v);
           }
+        }
+        if ((LONG || !full) && n >= zeroed) {    // (vectors come in order)
+          zero_outside(n);
+          zeroed = n + 1;
         }
         if (CS > 1 && !LONG) {
           const float* wh = whalo + hbuf * 2 * p.hmax;
